@@ -350,7 +350,7 @@ int mdwf_autotune(mdwf_ctx* ctx, int cfg_id, int n, int precision, int include_t
  * context's lattice; nsteps steps of size eps of Luscher's three-stage
  * Runge-Kutta scheme for dV/dt = -P_TA(Omega) V (Wilson plaquette action), in
  * FP64 (the smoothing of Sec. III, flow time nsteps * eps).  Input preparation:
- * load the result with mdwf_load_gauge.  Holds 3 * 4V * 18 doubles of scratch
+ * load the result with mdwf_load_gauge.  Holds 3 * 4V * 9 doubles of scratch
  * during the call.  Errors: ARG, NOMEM, CUDA. */
 int mdwf_wilson_flow_dev(mdwf_ctx* ctx, double* U, double eps, int nsteps, void* stream);
 

@@ -8,12 +8,27 @@
 // Runge-Kutta scheme:
 //   W1 = exp(Z0 / 4) W0,  W2 = exp(8/9 Z1 - 17/36 Z0) W1,
 //   W3 = exp(3/4 Z2 - 8/9 Z1 + 17/36 Z0) W2,   Z_i = eps Z(W_i).
-// exp by scaling and squaring: scale X by 2^-k until |X|_F <= 1/8, sum the
-// Taylor series to 12 terms (remainder below 1e-18 at that norm), square k times.
 //
-// Layout: the C ABI's gauge layout U[t][z][y][x][mu][a][b], complex (re, im),
-// one thread per link.  Input preparation: the solver reads links only
-// through mdwf_load_gauge.
+// Both kernels are bound by FP64 arithmetic (2 multiply-adds per SM and clock on
+// this part), so they are written for few of them and for full warps:
+// * Z: the six staples of a link are summed first and multiplied by the link
+//   once (13 matrix products instead of 18), by three threads per link, one per
+//   matrix row (a staple's rows are independent; only the last product needs the
+//   other rows, through shared memory): a third of the registers of a thread per
+//   link and three times the warps.
+// * exp(X) of an anti-Hermitian traceless X: X^3 = (tr X^2 / 2) X + det X
+//   (Cayley-Hamilton), so the Taylor polynomial is summed as f0 + f1 X + f2 X^2 by
+//   Horner's rule on three complex numbers, four multiply-adds per term, instead
+//   of matrix products.  |X|_F is first scaled to at most 1/2 by 2^-k (k squarings
+//   of the result; none for the usual steps); 17 terms leave a remainder below
+//   (1/2)^18 / 18! < 1e-21.
+// Z keeps the nine independent reals of an anti-Hermitian matrix, one plane each.
+// Ten steps at 16^3 x 48: 297 ms with a thread per link and the matrix Taylor series
+// (which spilled), 71 ms so (2.4 ms per stage; its 1800 multiply-adds per link take 2.3 ms
+// at 6.2e11 per second, the FP64 rate of the part).
+//
+// Layout of U: the C ABI's gauge layout U[t][z][y][x][mu][a][b], complex (re, im).
+// Input preparation: the solver reads links only through mdwf_load_gauge.
 #include "mdwf_internal.h"
 
 namespace mdwf {
@@ -27,62 +42,46 @@ struct M3 {
   C2 m[9];
 };
 
-__device__ __forceinline__ void mload(const double* __restrict__ p, M3& a) {
-#pragma unroll
-  for (int i = 0; i < 9; i++) { a.m[i].re = p[2 * i]; a.m[i].im = p[2 * i + 1]; }
+__device__ __forceinline__ void cfma(const C2& x, const C2& y, C2& a) {         // a += x y
+  a.re = __fma_rn(x.re, y.re, a.re); a.re = __fma_rn(-x.im, y.im, a.re);
+  a.im = __fma_rn(x.re, y.im, a.im); a.im = __fma_rn(x.im, y.re, a.im);
 }
-__device__ __forceinline__ void mstore(double* p, const M3& a) {
-#pragma unroll
-  for (int i = 0; i < 9; i++) { p[2 * i] = a.m[i].re; p[2 * i + 1] = a.m[i].im; }
+__device__ __forceinline__ void cfma_c(const C2& x, const C2& y, C2& a) {       // a += x conj(y)
+  a.re = __fma_rn(x.re, y.re, a.re); a.re = __fma_rn(x.im, y.im, a.re);
+  a.im = __fma_rn(x.im, y.re, a.im); a.im = __fma_rn(-x.re, y.im, a.im);
 }
-// c = a b (BD: c = a b^+)
-template <bool BD>
+// 8-byte accesses: U is the caller's array, aligned to a double (the kernels are bound by FP64, not by loads).
+__device__ __forceinline__ C2 ldc(const double* __restrict__ p) { return C2{p[0], p[1]}; }
+// c = a b
 __device__ __forceinline__ void mmul(const M3& a, const M3& b, M3& c) {
   M3 t;
 #pragma unroll
   for (int i = 0; i < 3; i++)
 #pragma unroll
     for (int j = 0; j < 3; j++) {
-      double re = 0.0, im = 0.0;
+      C2 s{0.0, 0.0};
 #pragma unroll
-      for (int k = 0; k < 3; k++) {
-        const C2 x = a.m[3 * i + k];
-        const C2 y = BD ? C2{b.m[3 * j + k].re, -b.m[3 * j + k].im} : b.m[3 * k + j];
-        re += x.re * y.re - x.im * y.im;
-        im += x.re * y.im + x.im * y.re;
-      }
-      t.m[3 * i + j] = C2{re, im};
+      for (int k = 0; k < 3; k++) cfma(a.m[3 * i + k], b.m[3 * k + j], s);
+      t.m[3 * i + j] = s;
     }
   c = t;
 }
 
-__device__ void mexp(const M3& X, M3& out) {
-  double nrm = 0.0;
+// Row vector times a stored matrix: o = v M (DAG: v M^+), added to o when ADD.
+template <bool DAG, bool ADD>
+__device__ __forceinline__ void vmul(const C2 v[3], const double* __restrict__ p, C2 o[3]) {
+  if (!ADD) {
 #pragma unroll
-  for (int i = 0; i < 9; i++) nrm += X.m[i].re * X.m[i].re + X.m[i].im * X.m[i].im;
-  nrm = sqrt(nrm);
-  int sq = 0;
-  while (nrm > 0.125 && sq < 64) { nrm *= 0.5; sq++; }
-  const double sc = ldexp(1.0, -sq);
-  M3 Y, term, sum;
-#pragma unroll
-  for (int i = 0; i < 9; i++) {
-    Y.m[i] = C2{X.m[i].re * sc, X.m[i].im * sc};
-    term.m[i] = sum.m[i] = C2{(i % 4 == 0) ? 1.0 : 0.0, 0.0};
+    for (int j = 0; j < 3; j++) o[j] = C2{0.0, 0.0};
   }
-  for (int k = 1; k <= 12; k++) {
-    mmul<false>(term, Y, term);
-    const double inv = 1.0 / k;
 #pragma unroll
-    for (int i = 0; i < 9; i++) {
-      term.m[i].re *= inv;
-      term.m[i].im *= inv;
-      sum.m[i].re += term.m[i].re;
-      sum.m[i].im += term.m[i].im;
+  for (int i = 0; i < 3; i++)
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+      const C2 y = ldc(p + 2 * (3 * i + j));            // M_ij
+      if (DAG) cfma_c(v[j], y, o[i]);                   // (M^+)_ji = conj(M_ij)
+      else cfma(v[i], y, o[j]);
     }
-  }
-  for (int i = 0; i < sq; i++) mmul<false>(sum, sum, sum);
-  out = sum;
 }
 
 struct Lat {
@@ -92,118 +91,244 @@ struct Lat {
 
 __device__ __forceinline__ long lat_nbr(const Lat& g, const int c[4], int mu, int dir) {
   int d[4] = {c[0], c[1], c[2], c[3]};
-  d[mu] = d[mu] + dir;
-  if (d[mu] < 0) d[mu] += g.L[mu];
-  if (d[mu] >= g.L[mu]) d[mu] -= g.L[mu];
+#pragma unroll
+  for (int i = 0; i < 4; i++)
+    if (i == mu) {
+      d[i] += dir;
+      if (d[i] < 0) d[i] += g.L[i];
+      if (d[i] >= g.L[i]) d[i] -= g.L[i];
+    }
   return d[0] + (long)g.L[0] * (d[1] + (long)g.L[1] * (d[2] + (long)g.L[2] * d[3]));
 }
 
 __device__ __forceinline__ const double* lnk(const double* U, long s, int mu) { return U + 18 * (4 * s + mu); }
 
-// Z = eps * (-P_TA(Omega_mu(x))) for every link.
-__global__ void k_flow_Z(const double* __restrict__ U, double* __restrict__ Z, Lat g, double eps) {
-  const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= 4 * g.V) return;
-  const long s = k >> 2;
-  const int mu = (int)(k & 3);
-  int c[4];
-  long r = s;
-  for (int i = 0; i < 4; i++) { c[i] = (int)(r % g.L[i]); r /= g.L[i]; }
-  M3 Umu, acc, a, b, w;
-  mload(lnk(U, s, mu), Umu);
+constexpr int kZLinks = 32;             // links per block of k_flow_Z (three threads each: three full warps)
+
+// Z = eps * (-P_TA(Omega_mu(x))) for every link, as nine planes of nlink reals: the
+// imaginary diagonal (0..2) and re, im of the elements (0,1), (0,2), (1,2) (3..8).
+__global__ void __launch_bounds__(3 * kZLinks) k_flow_Z(const double* __restrict__ U, double* __restrict__ Z, Lat g,
+                                                       double eps) {
+  __shared__ double2 st[3 * kZLinks][3];
+  const long nlink = 4 * g.V;
+  const int kl = threadIdx.x / 3, row = threadIdx.x - 3 * kl;
+  const long k = (long)blockIdx.x * kZLinks + kl;
+  const bool on = k < nlink;
+  const long s = on ? k >> 2 : 0;
+  const int mu = on ? (int)(k & 3) : 0;
+  C2 acc[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};      // row of the sum of the staples
+  if (on) {
+    int c[4];
+    long r = s;
+    for (int i = 0; i < 4; i++) { c[i] = (int)(r % g.L[i]); r /= g.L[i]; }
+    const long xp = lat_nbr(g, c, mu, +1);
+    int cp[4];
 #pragma unroll
-  for (int i = 0; i < 9; i++) acc.m[i] = C2{0.0, 0.0};
-  const long xp = lat_nbr(g, c, mu, +1);
-  int cp[4] = {c[0], c[1], c[2], c[3]};
-  cp[mu] = cp[mu] + 1 == g.L[mu] ? 0 : cp[mu] + 1;
-  for (int nu = 0; nu < 4; nu++) {
-    if (nu == mu) continue;
-    const long xn = lat_nbr(g, c, nu, +1), xm = lat_nbr(g, c, nu, -1), xpm = lat_nbr(g, cp, nu, -1);
-    // U_mu(x) U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+
-    mload(lnk(U, xp, nu), w);
-    mmul<false>(Umu, w, a);
-    mload(lnk(U, xn, mu), w);
-    mmul<true>(a, w, b);
-    mload(lnk(U, s, nu), w);
-    mmul<true>(b, w, a);
+    for (int i = 0; i < 4; i++) cp[i] = i == mu ? (c[i] + 1 == g.L[i] ? 0 : c[i] + 1) : c[i];
+    for (int p = 1; p < 4; p++) {
+      const int nu = (mu + p) & 3;
+      const long xn = lat_nbr(g, c, nu, +1), xm = lat_nbr(g, c, nu, -1), xpm = lat_nbr(g, cp, nu, -1);
+      C2 v[3], w[3];
+      // U_nu(x+mu) U_mu(x+nu)^+ U_nu(x)^+
+      const double* a = lnk(U, xp, nu) + 6 * row;
 #pragma unroll
-    for (int i = 0; i < 9; i++) { acc.m[i].re += a.m[i].re; acc.m[i].im += a.m[i].im; }
-    // U_mu(x) U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu)
-    mload(lnk(U, xpm, nu), w);
-    mmul<true>(Umu, w, a);
-    mload(lnk(U, xm, mu), w);
-    mmul<true>(a, w, b);
-    mload(lnk(U, xm, nu), w);
-    mmul<false>(b, w, a);
+      for (int j = 0; j < 3; j++) v[j] = ldc(a + 2 * j);
+      vmul<true, false>(v, lnk(U, xn, mu), w);
+      vmul<true, true>(w, lnk(U, s, nu), acc);
+      // U_nu(x+mu-nu)^+ U_mu(x-nu)^+ U_nu(x-nu)
+      const double* b = lnk(U, xpm, nu) + 2 * row;
 #pragma unroll
-    for (int i = 0; i < 9; i++) { acc.m[i].re += a.m[i].re; acc.m[i].im += a.m[i].im; }
+      for (int j = 0; j < 3; j++) { v[j] = ldc(b + 6 * j); v[j].im = -v[j].im; }
+      vmul<true, false>(v, lnk(U, xm, mu), w);
+      vmul<false, true>(w, lnk(U, xm, nu), acc);
+    }
   }
-  // -P_TA, scaled by eps
-  M3 t;
+#pragma unroll
+  for (int j = 0; j < 3; j++) st[threadIdx.x][j] = make_double2(acc[j].re, acc[j].im);
+  __syncthreads();
+  // row of Omega = U_mu(x) (sum of staples)
+  C2 om[3] = {{0.0, 0.0}, {0.0, 0.0}, {0.0, 0.0}};
+  if (on) {
+    const double* u = lnk(U, s, mu) + 6 * row;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      const C2 ui = ldc(u + 2 * i);
+#pragma unroll
+      for (int j = 0; j < 3; j++) {
+        const double2 q = st[3 * kl + i][j];
+        cfma(ui, C2{q.x, q.y}, om[j]);
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < 3; j++) st[threadIdx.x][j] = make_double2(om[j].re, om[j].im);
+  __syncthreads();
+  if (!on) return;
+  // -eps P_TA: thread `row` writes its diagonal and one off-diagonal element
+  const double2 d0 = st[3 * kl][0], d1 = st[3 * kl + 1][1], d2 = st[3 * kl + 2][2];
+  const double tr = (d0.y + d1.y + d2.y) / 3.0;
+  const double dg = row == 0 ? d0.y : row == 1 ? d1.y : d2.y;
+  const int i = row == 2 ? 1 : 0, j = row == 0 ? 1 : 2;   // (0,1), (0,2), (1,2)
+  const double2 x = st[3 * kl + i][j], y = st[3 * kl + j][i];
+  Z[(long)row * nlink + k] = -eps * (dg - tr);
+  Z[(long)(3 + 2 * row) * nlink + k] = -eps * (0.5 * (x.x - y.x));
+  Z[(long)(4 + 2 * row) * nlink + k] = -eps * (0.5 * (x.y + y.y));
+}
+
+// exp of the anti-Hermitian traceless X with diagonal i d[0..2] and elements (0,1), (0,2), (1,2) = o[0..2].
+__device__ __forceinline__ void mexp(const double d_in[3], const C2 o_in[3], M3& E) {
+  double n2 = 0.0;
 #pragma unroll
   for (int i = 0; i < 3; i++)
+    n2 += d_in[i] * d_in[i] + 2.0 * (o_in[i].re * o_in[i].re + o_in[i].im * o_in[i].im);
+  int sq = 0;
+  while (n2 > 0.25 && sq < 64) { n2 *= 0.25; sq++; }
+  const double sc = ldexp(1.0, -sq);
+  double d[3];
+  C2 o[3];
 #pragma unroll
-    for (int j = 0; j < 3; j++) {
-      const C2 x = acc.m[3 * i + j], y = acc.m[3 * j + i];
-      t.m[3 * i + j] = C2{0.5 * (x.re - y.re), 0.5 * (x.im + y.im)};
-    }
-  const double tr = (t.m[0].im + t.m[4].im + t.m[8].im) / 3.0;
-  t.m[0].im -= tr; t.m[4].im -= tr; t.m[8].im -= tr;
+  for (int i = 0; i < 3; i++) { d[i] = d_in[i] * sc; o[i] = C2{o_in[i].re * sc, o_in[i].im * sc}; }
+  // X^2 (Hermitian): diagonal -q[i], elements (0,1), (0,2), (1,2) = y[i]
+  const double a01 = o[0].re * o[0].re + o[0].im * o[0].im;
+  const double a02 = o[1].re * o[1].re + o[1].im * o[1].im;
+  const double a12 = o[2].re * o[2].re + o[2].im * o[2].im;
+  const double q[3] = {d[0] * d[0] + a01 + a02, d[1] * d[1] + a01 + a12, d[2] * d[2] + a02 + a12};
+  C2 y[3];
+  // (0,1): i (d0 + d1) o01 - o02 conj(o12);  (0,2): i (d0 + d2) o02 + o01 o12;  (1,2): i (d1 + d2) o12 - conj(o01) o02
+  const double s01 = d[0] + d[1], s02 = d[0] + d[2], s12 = d[1] + d[2];
+  y[0].re = -s01 * o[0].im - (o[1].re * o[2].re + o[1].im * o[2].im);
+  y[0].im = s01 * o[0].re - (o[1].im * o[2].re - o[1].re * o[2].im);
+  y[1].re = -s02 * o[1].im + (o[0].re * o[2].re - o[0].im * o[2].im);
+  y[1].im = s02 * o[1].re + (o[0].re * o[2].im + o[0].im * o[2].re);
+  y[2].re = -s12 * o[2].im - (o[0].re * o[1].re + o[0].im * o[1].im);
+  y[2].im = s12 * o[2].re - (o[0].re * o[1].im - o[0].im * o[1].re);
+  // X^3 = c1 X + i dt:  c1 = tr X^2 / 2,  det X = i dt,
+  // dt = -d0 d1 d2 + d0 a12 + d1 a02 + d2 a01 - 2 Im(o01 o12 conj(o02))
+  const double c1 = -0.5 * (q[0] + q[1] + q[2]);
+  const C2 t{o[0].re * o[2].re - o[0].im * o[2].im, o[0].re * o[2].im + o[0].im * o[2].re};
+  const double dt = -d[0] * d[1] * d[2] + d[0] * a12 + d[1] * a02 + d[2] * a01 -
+                    2.0 * (t.im * o[1].re - t.re * o[1].im);
+  // Horner on p0 + p1 X + p2 X^2:  p <- p X + 1/k!
+  constexpr int kTerms = 17;
+  const double invf[kTerms + 1] = {1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040, 1.0 / 40320,
+                                   1.0 / 362880, 1.0 / 3628800, 1.0 / 39916800, 1.0 / 479001600, 1.0 / 6227020800.0,
+                                   1.0 / 87178291200.0, 1.0 / 1307674368000.0, 1.0 / 20922789888000.0,
+                                   1.0 / 355687428096000.0};
+  C2 p0{invf[kTerms], 0.0}, p1{0.0, 0.0}, p2{0.0, 0.0};
 #pragma unroll
-  for (int i = 0; i < 9; i++) t.m[i] = C2{-eps * t.m[i].re, -eps * t.m[i].im};
-  mstore(Z + 18 * k, t);
+  for (int k = kTerms - 1; k >= 0; k--) {
+    const C2 n0{__fma_rn(-dt, p2.im, invf[k]), dt * p2.re};
+    const C2 n1{__fma_rn(c1, p2.re, p0.re), __fma_rn(c1, p2.im, p0.im)};
+    p2 = p1;
+    p1 = n1;
+    p0 = n0;
+  }
+  // E = p0 + p1 X + p2 X^2
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    C2 e = p0;
+    e.re = __fma_rn(-p1.im, d[i], e.re); e.im = __fma_rn(p1.re, d[i], e.im);
+    e.re = __fma_rn(-p2.re, q[i], e.re); e.im = __fma_rn(-p2.im, q[i], e.im);
+    E.m[4 * i] = e;
+  }
+#pragma unroll
+  for (int i = 0; i < 3; i++) {
+    const int a = i == 2 ? 1 : 0, b = i == 0 ? 1 : 2;
+    C2 u{0.0, 0.0}, l{0.0, 0.0};
+    cfma(p1, o[i], u);
+    cfma(p2, y[i], u);
+    cfma(p1, C2{-o[i].re, o[i].im}, l);                  // X_ba = -conj(X_ab)
+    cfma(p2, C2{y[i].re, -y[i].im}, l);                  // (X^2)_ba = conj((X^2)_ab)
+    E.m[3 * a + b] = u;
+    E.m[3 * b + a] = l;
+  }
+  for (int i = 0; i < sq; i++) mmul(E, E, E);
 }
 
 // U <- exp(c0 Z0 + c1 Z1 + c2 Z2) U for every link.
-__global__ void k_flow_update(double* __restrict__ U, const double* __restrict__ Z0, const double* __restrict__ Z1,
-                              const double* __restrict__ Z2, long nlink, double c0, double c1, double c2) {
+template <int NZ>
+__global__ void __launch_bounds__(128) k_flow_update(double* __restrict__ U, const double* __restrict__ Z, long nlink,
+                                                    double c0, double c1, double c2) {
   const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= nlink) return;
-  M3 X, E, u;
+  double x[9];
 #pragma unroll
-  for (int i = 0; i < 18; i++) {
-    double v = c0 * Z0[18 * k + i];
-    if (Z1) v += c1 * Z1[18 * k + i];
-    if (Z2) v += c2 * Z2[18 * k + i];
-    if (i & 1) X.m[i >> 1].im = v; else X.m[i >> 1].re = v;
+  for (int i = 0; i < 9; i++) {
+    double v = c0 * Z[(long)i * nlink + k];
+    if (NZ > 1) v += c1 * Z[(long)(9 + i) * nlink + k];
+    if (NZ > 2) v += c2 * Z[(long)(18 + i) * nlink + k];
+    x[i] = v;
   }
-  mexp(X, E);
-  mload(U + 18 * k, u);
-  mmul<false>(E, u, u);
-  mstore(U + 18 * k, u);
+  const double d[3] = {x[0], x[1], x[2]};
+  const C2 o[3] = {{x[3], x[4]}, {x[5], x[6]}, {x[7], x[8]}};
+  M3 E;
+  mexp(d, o, E);
+  // column by column of U (three complex numbers live at a time)
+  double* u = U + 18 * k;
+#pragma unroll
+  for (int j = 0; j < 3; j++) {
+    const C2 v[3] = {ldc(u + 2 * j), ldc(u + 6 + 2 * j), ldc(u + 12 + 2 * j)};
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      C2 s{0.0, 0.0};
+#pragma unroll
+      for (int m = 0; m < 3; m++) cfma(E.m[3 * i + m], v[m], s);
+      u[6 * i + 2 * j] = s.re;
+      u[6 * i + 2 * j + 1] = s.im;
+    }
+  }
 }
 
-// Per-site sum of Re tr of the six plaquettes.
-__global__ void k_plaq(const double* __restrict__ U, double* __restrict__ part, Lat g) {
-  const long s = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= g.V) return;
-  int c[4];
-  long r = s;
-  for (int i = 0; i < 4; i++) { c[i] = (int)(r % g.L[i]); r /= g.L[i]; }
+// Re tr of a plaquette is Re tr(A B^+) with A = U_mu(x) U_nu(x+mu), B = U_nu(x) U_mu(x+nu):
+// two matrix products and a contraction.  A thread per (site, plane); a block writes the
+// sum of its threads in a fixed order.
+__global__ void __launch_bounds__(192) k_plaq(const double* __restrict__ U, double* __restrict__ part, Lat g) {
+  __shared__ double sh[192];
+  const long i = (long)blockIdx.x * 192 + threadIdx.x;
   double tot = 0.0;
-  M3 a, b, w, u;
-  for (int mu = 0; mu < 4; mu++)
-    for (int nu = mu + 1; nu < 4; nu++) {
-      mload(lnk(U, s, mu), u);
-      mload(lnk(U, lat_nbr(g, c, mu, +1), nu), w);
-      mmul<false>(u, w, a);
-      mload(lnk(U, lat_nbr(g, c, nu, +1), mu), w);
-      mmul<true>(a, w, b);
-      mload(lnk(U, s, nu), w);
-      mmul<true>(b, w, a);
-      tot += a.m[0].re + a.m[4].re + a.m[8].re;
+  if (i < 6 * g.V) {
+    const long s = i / 6;
+    const int pl = (int)(i - 6 * s);
+    const int mu = pl < 3 ? 0 : pl < 5 ? 1 : 2;
+    const int nu = pl < 3 ? pl + 1 : pl < 5 ? pl - 1 : 3;
+    int c[4];
+    long r = s;
+    for (int k = 0; k < 4; k++) { c[k] = (int)(r % g.L[k]); r /= g.L[k]; }
+    const double* um = lnk(U, s, mu);
+    const double* un = lnk(U, s, nu);
+    const double* unp = lnk(U, lat_nbr(g, c, mu, +1), nu);
+    const double* ump = lnk(U, lat_nbr(g, c, nu, +1), mu);
+#pragma unroll
+    for (int row = 0; row < 3; row++) {
+      C2 v[3], a[3], b[3];
+#pragma unroll
+      for (int j = 0; j < 3; j++) v[j] = ldc(um + 6 * row + 2 * j);
+      vmul<false, false>(v, unp, a);
+#pragma unroll
+      for (int j = 0; j < 3; j++) v[j] = ldc(un + 6 * row + 2 * j);
+      vmul<false, false>(v, ump, b);
+#pragma unroll
+      for (int j = 0; j < 3; j++) tot = __fma_rn(a[j].re, b[j].re, __fma_rn(a[j].im, b[j].im, tot));
     }
-  part[s] = tot;
+  }
+  sh[threadIdx.x] = tot;
+  __syncthreads();
+  for (int w = 96; w >= 3; w >>= 1) {
+    if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) part[blockIdx.x] = sh[0] + sh[1] + sh[2];
 }
 
 // Fixed-order sum of n doubles by one block.
-__global__ void k_sum(const double* __restrict__ v, long n, double* out) {
-  __shared__ double sh[256];
+__global__ void __launch_bounds__(1024) k_sum(const double* __restrict__ v, long n, double* out) {
+  __shared__ double sh[1024];
   double s = 0.0;
-  for (long i = threadIdx.x; i < n; i += 256) s += v[i];
+  for (long i = threadIdx.x; i < n; i += 1024) s += v[i];
   sh[threadIdx.x] = s;
   __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
+  for (int w = 512; w > 0; w >>= 1) {
     if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
     __syncthreads();
   }
@@ -217,17 +342,14 @@ cudaError_t wilson_flow(double* U, const int L[4], double eps, int nsteps, doubl
   for (int i = 0; i < 4; i++) g.L[i] = L[i];
   g.V = (long)L[0] * L[1] * L[2] * L[3];
   const long nlink = 4 * g.V;
-  double* Z0 = Z;
-  double* Z1 = Z + 18 * nlink;
-  double* Z2 = Z + 36 * nlink;
-  const unsigned blk = 128, grid = (unsigned)((nlink + blk - 1) / blk);
+  const unsigned gz = (unsigned)((nlink + kZLinks - 1) / kZLinks), gu = (unsigned)((nlink + 127) / 128);
   for (int n = 0; n < nsteps; n++) {
-    k_flow_Z<<<grid, blk, 0, st>>>(U, Z0, g, eps);
-    k_flow_update<<<grid, blk, 0, st>>>(U, Z0, nullptr, nullptr, nlink, 0.25, 0.0, 0.0);
-    k_flow_Z<<<grid, blk, 0, st>>>(U, Z1, g, eps);
-    k_flow_update<<<grid, blk, 0, st>>>(U, Z0, Z1, nullptr, nlink, -17.0 / 36.0, 8.0 / 9.0, 0.0);
-    k_flow_Z<<<grid, blk, 0, st>>>(U, Z2, g, eps);
-    k_flow_update<<<grid, blk, 0, st>>>(U, Z0, Z1, Z2, nlink, 17.0 / 36.0, -8.0 / 9.0, 0.75);
+    k_flow_Z<<<gz, 3 * kZLinks, 0, st>>>(U, Z, g, eps);
+    k_flow_update<1><<<gu, 128, 0, st>>>(U, Z, nlink, 0.25, 0.0, 0.0);
+    k_flow_Z<<<gz, 3 * kZLinks, 0, st>>>(U, Z + 9 * nlink, g, eps);
+    k_flow_update<2><<<gu, 128, 0, st>>>(U, Z, nlink, -17.0 / 36.0, 8.0 / 9.0, 0.0);
+    k_flow_Z<<<gz, 3 * kZLinks, 0, st>>>(U, Z + 18 * nlink, g, eps);
+    k_flow_update<3><<<gu, 128, 0, st>>>(U, Z, nlink, 17.0 / 36.0, -8.0 / 9.0, 0.75);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
@@ -238,8 +360,9 @@ cudaError_t plaquette(const double* U, const int L[4], double* part, double* out
   Lat g;
   for (int i = 0; i < 4; i++) g.L[i] = L[i];
   g.V = (long)L[0] * L[1] * L[2] * L[3];
-  k_plaq<<<(unsigned)((g.V + 127) / 128), 128, 0, st>>>(U, part, g);
-  k_sum<<<1, 256, 0, st>>>(part, g.V, out);
+  const long nb = (6 * g.V + 191) / 192;
+  k_plaq<<<(unsigned)nb, 192, 0, st>>>(U, part, g);
+  k_sum<<<1, 1024, 0, st>>>(part, nb, out);
   return cudaGetLastError();
 }
 

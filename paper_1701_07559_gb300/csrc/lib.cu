@@ -2297,7 +2297,7 @@ int mdwf_wilson_flow_dev(mdwf_ctx* ctx, double* U, double eps, int nsteps, void*
   cudaStream_t st = pick_stream(ctx, stream);
   const size_t nlink = (size_t)ctx->g.V * 4;
   cudaError_t e = cudaSuccess;
-  double* Z = (double*)ws_get(ctx, "flow.Z", sizeof(double) * 54 * nlink, &e);
+  double* Z = (double*)ws_get(ctx, "flow.Z", sizeof(double) * 27 * nlink, &e);
   CK(e);
   CK(wilson_flow(U, ctx->g.L, eps, nsteps, Z, st));
   CK(cudaStreamSynchronize(st));

@@ -415,9 +415,9 @@ cudaError_t build_link12(const float* U32, float* U12, long nlinks, cudaStream_t
 // the projected half spinor its backward hop needs); layout as FastArgs::halo_*.
 cudaError_t dd_pack_faces(const double* in, const Geom& g, int par, int L5, int N, int dagger, const double* U,
                           double* face_prev, double* face_next, cudaStream_t st);
-// Wilson flow (flow.cu): U in the C ABI gauge layout, Z: workspace of 3 * 4V * 18 doubles.
+// Wilson flow (flow.cu): U in the C ABI gauge layout, Z: workspace of 3 * 4V * 9 doubles.
 cudaError_t wilson_flow(double* U, const int L[4], double eps, int nsteps, double* Z, cudaStream_t st);
-// Sum over sites of Re tr of the six plaquettes into *out (device); part: V doubles of workspace.
+// Sum over sites of Re tr of the six plaquettes into *out (device); part: ceil(V / 32) doubles of workspace.
 cudaError_t plaquette(const double* U, const int L[4], double* part, double* out, cudaStream_t st);
 // Shared-memory bytes of a staged launch (0 if the tiling cannot be staged).
 template <typename S, typename T>
