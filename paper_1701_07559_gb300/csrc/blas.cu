@@ -345,17 +345,6 @@ __global__ void k_zero_masked(S* __restrict__ v, float* __restrict__ nrm, Tiling
   store24<S, T>(v, nrm, x.u, z);
 }
 
-// Wall source of a 4D field (API layout): slice 0 gets the P_+ spins (0, 1),
-// slice L5-1 the P_- spins (2, 3); the other slices must already be zero.
-__global__ void k_walls(const double* __restrict__ eta, double* __restrict__ w, long V, int L5) {
-  long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= V * 24) return;
-  const int k = (int)(i % 24);
-  const int spin = k / 6;
-  if (spin < 2) w[i] = eta[i];
-  else w[(long)(L5 - 1) * V * 24 + i] = eta[i];
-}
-
 // Z2 noise source: complex element k of a 4D field ([t][z][y][x][spin][colour],
 // k = 0 .. 12V-1) is (+1, 0) or (-1, 0) by the top bit of the k-th output of
 // SplitMix64 from state `seed` (Steele, Lea and Flood, OOPSLA 2014): the state
@@ -370,96 +359,6 @@ __global__ void k_z2(unsigned long long seed, double* __restrict__ eta, long n) 
   z = z ^ (z >> 31);
   eta[2 * k] = (z >> 63) ? -1.0 : 1.0;
   eta[2 * k + 1] = 0.0;
-}
-
-// One step of gauge-covariant Gaussian source smearing on a 4D field (the sources
-// of the paper's propagators, Sec. VII):
-//   out(x) = in(x) + k sum_{i = x,y,z} [U_i(x) in(x+i) + U_i(x-i)^+ in(x-i) - 2 in(x)],
-// spin-diagonal, no hop in time.  in / out: C ABI layout [t][z][y][x][spin][colour];
-// U: the context's FP64 links [parity][h][mu][18], h = lex / 2.
-__global__ void k_smear_step(const double* __restrict__ U, const double* __restrict__ in, double* __restrict__ out,
-                             Geom g, double k) {
-  const long lex = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (lex >= g.V) return;
-  int c[4];
-  long r = lex;
-  for (int i = 0; i < 4; i++) { c[i] = (int)(r % g.L[i]); r /= g.L[i]; }
-  const double* me = in + lex * 24;
-  double acc[24];
-  for (int i = 0; i < 24; i++) acc[i] = (1.0 - 6.0 * k) * me[i];
-  long stride = 1;
-  for (int mu = 0; mu < 3; mu++) {
-    const int Lm = g.L[mu];
-    const long fw = c[mu] == Lm - 1 ? lex - (long)(Lm - 1) * stride : lex + stride;
-    const long bw = c[mu] == 0 ? lex + (long)(Lm - 1) * stride : lex - stride;
-    const int pf = (c[0] + c[1] + c[2] + c[3]) & 1;
-    const double* uf = U + (((long)pf * g.Vh + (lex >> 1)) * 4 + mu) * 18;            // U_mu(x)
-    const double* ub = U + (((long)(1 - pf) * g.Vh + (bw >> 1)) * 4 + mu) * 18;       // U_mu(x - mu)
-    const double* pf_in = in + fw * 24;
-    const double* pb_in = in + bw * 24;
-    for (int sp = 0; sp < 4; sp++)
-      for (int a = 0; a < 3; a++) {
-        double re = 0.0, im = 0.0;
-        for (int b = 0; b < 3; b++) {
-          const double fr = uf[2 * (3 * a + b)], fi = uf[2 * (3 * a + b) + 1];      // U_ab
-          const double vr = pf_in[6 * sp + 2 * b], vi = pf_in[6 * sp + 2 * b + 1];
-          re += fr * vr - fi * vi;
-          im += fr * vi + fi * vr;
-          const double br = ub[2 * (3 * b + a)], bi = -ub[2 * (3 * b + a) + 1];     // (U^+)_ab = conj(U_ba)
-          const double wr = pb_in[6 * sp + 2 * b], wi = pb_in[6 * sp + 2 * b + 1];
-          re += br * wr - bi * wi;
-          im += br * wi + bi * wr;
-        }
-        acc[6 * sp + 2 * a] += k * re;
-        acc[6 * sp + 2 * a + 1] += k * im;
-      }
-    stride *= Lm;
-  }
-  for (int i = 0; i < 24; i++) out[lex * 24 + i] = acc[i];
-}
-
-// Residual-mass correlators (Eq. mres of arXiv:1701.07559): per 4D site, summed
-// over the n solutions (spin-colour sources), the squared norms of the wall field
-// q = P_- x_0 + P_+ x_{L5-1} and of the midpoint field Q = P_+ x_{L5/2-1} + P_- x_{L5/2};
-// P_+ keeps spins 0, 1 and P_- spins 2, 3 (gamma_5 = diag(1, 1, -1, -1)).  FP64,
-// solutions in the C ABI 5D layout.
-__global__ void k_mres_sites(const double* const* __restrict__ xs, int n, long V, int L5, double* pp, double* j5) {
-  const long x = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (x >= V) return;
-  const int sm = L5 / 2;
-  double a = 0.0, b = 0.0;
-  for (int k = 0; k < n; k++) {
-    const double* f = xs[k];
-    const double* w0 = f + (x) * 24;                          // s = 0
-    const double* wl = f + ((long)(L5 - 1) * V + x) * 24;     // s = L5 - 1
-    const double* m0 = f + ((long)(sm - 1) * V + x) * 24;     // s = L5/2 - 1
-    const double* m1 = f + ((long)sm * V + x) * 24;           // s = L5/2
-    for (int i = 0; i < 12; i++) {                            // spins 0, 1: (re, im) x 3 colours x 2
-      a += wl[i] * wl[i];
-      b += m0[i] * m0[i];
-    }
-    for (int i = 12; i < 24; i++) {                           // spins 2, 3
-      a += w0[i] * w0[i];
-      b += m1[i] * m1[i];
-    }
-  }
-  pp[x] = a;
-  j5[x] = b;
-}
-
-// Per time slice, fixed-order sums of the site values (one block per slice).
-__global__ void k_slice_sum(const double* __restrict__ v, long slice, double* out) {
-  __shared__ double sh[256];
-  const double* p = v + (long)blockIdx.x * slice;
-  double s = 0.0;
-  for (long i = threadIdx.x; i < slice; i += 256) s += p[i];
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if ((int)threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) out[blockIdx.x] = sh[0];
 }
 
 // rho = S(bhat - q) with bhat in FP64 and q in FP32 (the residual of a reliable
@@ -590,28 +489,9 @@ cudaError_t zero_masked(S* v, float* nrm, const Tiling& t, long Vh, int L5, int 
   return cudaGetLastError();
 }
 
-cudaError_t walls(const double* eta, double* w, long V, int L5, cudaStream_t st) {
-  long n = V * 24;
-  k_walls<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(eta, w, V, L5);
-  return cudaGetLastError();
-}
-
 cudaError_t z2_source(unsigned long long seed, double* eta, long V, cudaStream_t st) {
   const long n = V * 12;
   k_z2<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(seed, eta, n);
-  return cudaGetLastError();
-}
-
-cudaError_t smear_step(const double* U, const double* in, double* out, const Geom& g, double k, cudaStream_t st) {
-  k_smear_step<<<(unsigned)((g.V + 127) / 128), 128, 0, st>>>(U, in, out, g, k);
-  return cudaGetLastError();
-}
-
-cudaError_t mres_correlators(const double* const* xs, int n, long V, int Lt, int L5, double* pp, double* j5,
-                             double* c_pp, double* c_j5, cudaStream_t st) {
-  k_mres_sites<<<(unsigned)((V + 255) / 256), 256, 0, st>>>(xs, n, V, L5, pp, j5);
-  k_slice_sum<<<Lt, 256, 0, st>>>(pp, V / Lt, c_pp);
-  k_slice_sum<<<Lt, 256, 0, st>>>(j5, V / Lt, c_j5);
   return cudaGetLastError();
 }
 

@@ -57,11 +57,19 @@ cudaError_t resid_update(const double* bhat, const float* q, S* rho, float* rho_
 template <typename S>
 cudaError_t zero_masked(S* v, float* nrm, const Tiling& t, long Vh, int L5, int N, const int* mask, cudaStream_t st);
 
-cudaError_t walls(const double* eta, double* w, long V, int L5, cudaStream_t st);
 cudaError_t z2_source(unsigned long long seed, double* eta, long V, cudaStream_t st);
-cudaError_t smear_step(const double* U, const double* in, double* out, const Geom& g, double k, cudaStream_t st);
-cudaError_t mres_correlators(const double* const* xs, int n, long V, int Lt, int L5, double* pp, double* j5,
-                             double* c_pp, double* c_j5, cudaStream_t st);
+
+// 4D sources and sinks (sources.cu).
+// src = f w + hc H w, w = P_+ eta on slice 0 and P_- eta on slice L5 - 1.
+cudaError_t wall_source(const double* U, const double* eta, double* src, const Geom& g, int L5, int anti, double f,
+                        double hc, cudaStream_t st);
+// n_iter smearing steps of eta in place; tmp: V * 24 doubles, flags: Lt ints.
+cudaError_t smear(const double* U, double* eta, double* tmp, int* flags, const Geom& g, double k, int n_iter,
+                  cudaStream_t st);
+// c[2][Lt]: the two residual-mass correlators; part: 2 Lt mres_blocks(V / Lt) doubles.
+int mres_blocks(long slice_sites);
+cudaError_t mres_correlators(const double* const* xs, int n, long V, int Lt, int L5, double* part, double* c,
+                             cudaStream_t st);
 
 cudaError_t finalize(const double* partials, long ntiles, int N, double* out, cudaStream_t st);
 

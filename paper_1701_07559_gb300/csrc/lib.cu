@@ -1603,7 +1603,7 @@ int upload5(mdwf_ctx* ctx, const double* h, size_t n, DBuf& d, cudaStream_t st) 
 
 // Generic FP64 operator on device API-layout 5D fields, single RHS.
 //   kind 0: dslash (out_par, dagger)   1: mdwf D / D^+   2: 5D local op (op, dagger)
-//   3: make_source walls -> source     4: Schur (dagger, precision)
+//   4: Schur (dagger, precision)
 template <typename S>
 int schur_apply_impl(mdwf_ctx* ctx, Cfg* cfg, const double* in_dev, double* out_dev, int dagger, cudaStream_t st);
 
@@ -1661,21 +1661,17 @@ int apply_dev(mdwf_ctx* ctx, Cfg* cfg, int kind, int arg1, int arg2, const doubl
     const double* G = M[kinds[arg1][arg2 ? 1 : 0]];
     CK(op.run(false, 0, 0, ie.f(), none, G, none, nullptr, 0.0, oe.f(), nullptr, nullptr));
     CK(op.run(false, 1, 0, io.f(), none, G, none, nullptr, 0.0, oo.f(), nullptr, nullptr));
-  } else if (kind == 3) {
-    // src = (1 - c5 D_W) w = (1 - c5 d) w + c5/2 H w
-    Tables sc;
-    sc.L5 = L5; sc.N = 1;
-    sc.h.assign(sc.block(), 0.0);
-    const double f = 1.0 - cfg->act.c5 * (4.0 - cfg->act.M5);
-    for (int chi = 0; chi < 2; chi++) for (int s = 0; s < L5; s++) sc.h[((size_t)chi * L5 + s) * L5 + s] = f;
-    DevTables<double> G;
-    CK(upload_tables_ws<double>(ctx, "apply.stables", sc, &G, st));
-    CK(op.run(true, 0, 0, io.f(), ie.f(), G[0], none, nullptr, 0.5 * cfg->act.c5, oe.f(), nullptr, nullptr));
-    CK(op.run(true, 1, 0, ie.f(), io.f(), G[0], none, nullptr, 0.5 * cfg->act.c5, oo.f(), nullptr, nullptr));
   }
   CK(unpack_rhs<double>(oe.w.v, nullptr, out_dev, g, L5, 1, 0, 0, st));
   CK(unpack_rhs<double>(oo.w.v, nullptr, out_dev, g, L5, 1, 1, 0, st));
   CK(cudaStreamSynchronize(st));
+  return MDWF_OK;
+}
+
+// src = (1 - c5 D_W) w = (1 - c5 d) w + c5/2 H w for the wall field w of a 4D source (device arrays).
+int make_source_impl(mdwf_ctx* ctx, const Cfg* cfg, const double* eta, double* src, cudaStream_t st) {
+  const Action& a = cfg->act;
+  CK(wall_source(cfg->U64, eta, src, ctx->g, a.L5, cfg->anti, 1.0 - a.c5 * (4.0 - a.M5), 0.5 * a.c5, st));
   return MDWF_OK;
 }
 
@@ -2024,18 +2020,16 @@ int mdwf_make_source(mdwf_ctx* ctx, int cfg_id, const double* eta4d, double* src
   int rc = check_cfg(ctx, cfg_id, &cfg);
   if (rc) return rc;
   if (!eta4d || !src5d) return fail(ctx, MDWF_ERR_ARG, "make_source: null pointer");
-  const long V = ctx->g.V;
-  const int L5 = cfg->act.L5;
-  if (!all_finite(eta4d, (size_t)V * 24)) return fail(ctx, MDWF_ERR_NONFINITE, "source has NaN/Inf");
-  // walls: P_+ eta on s = 0 (spins 0,1), P_- eta on s = L5-1 (spins 2,3)
-  std::vector<double> w((size_t)L5 * V * 24, 0.0);
-  for (long x = 0; x < V; x++)
-    for (int k = 0; k < 24; k++) {
-      int spin = k / 6;
-      if (spin < 2) w[(size_t)x * 24 + k] = eta4d[(size_t)x * 24 + k];
-      else w[((size_t)(L5 - 1) * V + x) * 24 + k] = eta4d[(size_t)x * 24 + k];
-    }
-  return host_apply(ctx, cfg_id, 3, 0, 0, w.data(), src5d, w.size());
+  const size_t n4 = (size_t)ctx->g.V * 24, n5 = n4 * cfg->act.L5;
+  CK(cudaSetDevice(ctx->device));
+  cudaStream_t st = ctx->stream;
+  DBuf din, dout;
+  if ((rc = upload5(ctx, eta4d, n4, din, st))) return rc;
+  CK(dout.alloc(sizeof(double) * n5));
+  if ((rc = make_source_impl(ctx, cfg, din.as<double>(), dout.as<double>(), st))) return rc;
+  CK(cudaMemcpyAsync(src5d, dout.p, sizeof(double) * n5, cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  return MDWF_OK;
 }
 
 int mdwf_solve_batch(mdwf_ctx* ctx, int cfg_id, int n, const double* const* srcs, const double* masses,
@@ -2243,13 +2237,9 @@ int mdwf_make_source_dev(mdwf_ctx* ctx, int cfg_id, const double* eta4d, double*
   if (!eta4d || !src5d) return fail(ctx, MDWF_ERR_ARG, "make_source_dev: null pointer");
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = pick_stream(ctx, stream);
-  const size_t n5 = (size_t)cfg->act.L5 * ctx->g.V * 24;
-  cudaError_t e = cudaSuccess;
-  double* w = (double*)ws_get(ctx, "make_source.walls", sizeof(double) * n5, &e);
-  CK(e);
-  CK(cudaMemsetAsync(w, 0, sizeof(double) * n5, st));
-  CK(walls(eta4d, w, ctx->g.V, cfg->act.L5, st));
-  return apply_dev(ctx, cfg, 3, 0, 0, w, src5d, st);
+  if ((rc = make_source_impl(ctx, cfg, eta4d, src5d, st))) return rc;
+  CK(cudaStreamSynchronize(st));
+  return MDWF_OK;
 }
 
 int mdwf_z2_source_dev(mdwf_ctx* ctx, unsigned long long seed, double* eta4d, void* stream) {
@@ -2336,12 +2326,14 @@ int mdwf_mres_correlators_dev(mdwf_ctx* ctx, int cfg_id, int n, double* const* x
   cudaError_t e = cudaSuccess;
   double** dptr = (double**)ws_get(ctx, "mres.ptrs", sizeof(double*) * n, &e);
   CK(e);
-  double* site = (double*)ws_get(ctx, "mres.site", sizeof(double) * (2 * V + 2 * Lt), &e);
+  const size_t npart = (size_t)2 * Lt * mres_blocks(V / Lt);
+  double* part = (double*)ws_get(ctx, "mres.part", sizeof(double) * (npart + 2 * Lt), &e);
   CK(e);
+  double* c = part + npart;
   CK(cudaMemcpyAsync(dptr, xs, sizeof(double*) * n, cudaMemcpyHostToDevice, st));
-  CK(mres_correlators(dptr, n, V, Lt, cfg->act.L5, site, site + V, site + 2 * V, site + 2 * V + Lt, st));
-  CK(cudaMemcpyAsync(c_pp, site + 2 * V, sizeof(double) * Lt, cudaMemcpyDeviceToHost, st));
-  CK(cudaMemcpyAsync(c_j5q, site + 2 * V + Lt, sizeof(double) * Lt, cudaMemcpyDeviceToHost, st));
+  CK(mres_correlators(dptr, n, V, Lt, cfg->act.L5, part, c, st));
+  CK(cudaMemcpyAsync(c_pp, c, sizeof(double) * Lt, cudaMemcpyDeviceToHost, st));
+  CK(cudaMemcpyAsync(c_j5q, c + Lt, sizeof(double) * Lt, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
   return MDWF_OK;
 }
@@ -2358,14 +2350,10 @@ int mdwf_smear_source_dev(mdwf_ctx* ctx, int cfg_id, double* eta4d, double sigma
   cudaError_t e = cudaSuccess;
   double* tmp = (double*)ws_get(ctx, "smear.tmp", sizeof(double) * 24 * (size_t)ctx->g.V, &e);
   CK(e);
+  int* flags = (int*)ws_get(ctx, "smear.flags", sizeof(int) * ctx->g.L[3], &e);
+  CK(e);
   const double k = sigma * sigma / (4.0 * n_iter);
-  double* a = eta4d;
-  double* b = tmp;
-  for (int i = 0; i < n_iter; i++) {
-    CK(smear_step(it->second.U64, a, b, ctx->g, k, st));
-    std::swap(a, b);
-  }
-  if (a != eta4d) CK(cudaMemcpyAsync(eta4d, a, sizeof(double) * 24 * (size_t)ctx->g.V, cudaMemcpyDeviceToDevice, st));
+  CK(smear(it->second.U64, eta4d, tmp, flags, ctx->g, k, n_iter, st));
   CK(cudaStreamSynchronize(st));
   return MDWF_OK;
 }
