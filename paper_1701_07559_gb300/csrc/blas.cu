@@ -285,9 +285,9 @@ __global__ void k_bop(const S* __restrict__ xv, const float* __restrict__ x_nrm,
   load_part<S, T>(xv, x_nrm, (x.h * L5 + s_dn) * N + x.r, 0, up);
   load_part<S, T>(xv, x_nrm, (x.h * L5 + s_up) * N + x.r, 1, lo);
 #pragma unroll
-  for (int i = 0; i < 12; i++) y[i] = f.b5 * y[i] + f.c5 * w_dn * up[i];
+  for (int i = 0; i < 12; i++) y[i] = bop_term(f.b5, y[i], f.c5 * w_dn, up[i]);
 #pragma unroll
-  for (int i = 0; i < 12; i++) y[12 + i] = f.b5 * y[12 + i] + f.c5 * w_up * lo[i];
+  for (int i = 0; i < 12; i++) y[12 + i] = bop_term(f.b5, y[12 + i], f.c5 * w_up, lo[i]);
   store24<S, T>(uv, u_nrm, x.u, y);
 }
 

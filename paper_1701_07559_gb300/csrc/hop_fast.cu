@@ -189,36 +189,9 @@ __device__ __forceinline__ void hop_term_at(const FastArgs<S, T>& a, int hn, boo
   reconstruct<MU, T>(chi, f, f * sg, acc);
 }
 
-// A time hop across an edge of a decomposed lattice, from the neighbouring
-// sub-domain's face (same operations and order as the local term: the sender
-// projected, and for the backward hop multiplied by U^+, exactly as hop_term_at).
-template <bool FWD, typename S, typename T>
-__device__ __forceinline__ void halo_term(const FastArgs<S, T>& a, const Site& x, long h, int s, int r, T* acc) {
-  const T sg = (a.dagger ? T(1) : T(-1)) * (FWD ? T(1) : T(-1));
-  const long lex3 = x.lex - (long)x.c[3] * x.stride[3];
-  const T* p = (FWD ? a.halo_fwd : a.halo_bwd) + ((lex3 * a.L5 + s) * a.N + r) * 12;
-  T hh[12], chi[12];
-#pragma unroll
-  for (int i = 0; i < 12; i++) hh[i] = p[i];
-  const T f = FWD ? a.halo_sgn_fwd : a.halo_sgn_bwd;
-  if (FWD) {
-    T l[18];
-    load_link<T>(a.U, ((long)a.out_par * a.g.Vh + h) * 4 + 3, l);
-    su3_mul<T, false>(l, hh, chi);
-    su3_mul<T, false>(l, hh + 6, chi + 6);
-    reconstruct<3, T>(chi, f, f * sg, acc);
-  } else {
-    reconstruct<3, T>(hh, f, f * sg, acc);
-  }
-}
-
 template <int MU, bool FWD, typename S, typename T>
 __device__ __forceinline__ void hop_term(const FastArgs<S, T>& a, const Site& x, long h, int s, int r, const S* sp,
                                          float snrm, T* acc) {
-  if (MU == 3 && a.halo_fwd != nullptr && (FWD ? x.c[3] == a.g.L[3] - 1 : x.c[3] == 0)) {
-    halo_term<FWD, S, T>(a, x, h, s, r, acc);
-    return;
-  }
   const bool bflip = MU == 3 && a.antiperiodic && (FWD ? x.c[3] == a.g.L[3] - 1 : x.c[3] == 0);
   hop_term_at<MU, FWD, S, T>(a, nbr_half<MU, FWD>(a.g, x), bflip, h, s, r, sp, snrm, acc);
 }
@@ -573,11 +546,6 @@ template <typename S, typename T, int EPI>
 __global__ void __maxnreg__(72) hop_fast_kernel(FastArgs<S, T> a, Tiling tl) {
   hop_fast_body<S, T, EPI>(a, tl);
 }
-// FP64 arithmetic: no cap (24 doubles of accumulator alone take 48 registers).
-template <typename S, typename T, int EPI>
-__global__ void hop_fast_kernel_f64(FastArgs<S, T> a, Tiling tl) {
-  hop_fast_body<S, T, EPI>(a, tl);
-}
 
 // ---------------------------------------------------------------------------
 // Staged variant.  Every wait is bounded; on a timeout the block records an
@@ -720,7 +688,7 @@ cudaError_t launch_one(const FastArgs<S, T>& a, const Tiling& t, cudaStream_t st
     return cudaGetLastError();
   }
   const size_t smem = direct_tile_bytes<T>(t.threads);
-  auto* kern = std::is_same<T, double>::value ? hop_fast_kernel_f64<S, T, EPI> : hop_fast_kernel<S, T, EPI>;
+  auto* kern = hop_fast_kernel<S, T, EPI>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
@@ -732,7 +700,7 @@ cudaError_t launch_one(const FastArgs<S, T>& a, const Tiling& t, cudaStream_t st
 template <typename S, typename T, int EPI>
 int max_threads_one() {
   cudaFuncAttributes fa, fb;
-  auto* kern = std::is_same<T, double>::value ? hop_fast_kernel_f64<S, T, EPI> : hop_fast_kernel<S, T, EPI>;
+  auto* kern = hop_fast_kernel<S, T, EPI>;
   if (cudaFuncGetAttributes(&fa, kern) != cudaSuccess) return 128;
   if (cudaFuncGetAttributes(&fb, hop_staged_kernel<S, T, EPI>) != cudaSuccess) return 128;
   return fa.maxThreadsPerBlock < fb.maxThreadsPerBlock ? fa.maxThreadsPerBlock : fb.maxThreadsPerBlock;
@@ -1474,7 +1442,6 @@ cudaError_t dd_pack_faces(const double* in, const Geom& g, int par, int L5, int 
   template int fast_max_threads<S, T>();                                                             \
   template size_t staged_smem_bytes<S, T>(const Tiling&, int, int);
 
-MDWF_INST_FAST(double, double)
 MDWF_INST_FAST(float, float)
 MDWF_INST_FAST(__half, float)
 MDWF_INST_FAST(__nv_bfloat16, float)

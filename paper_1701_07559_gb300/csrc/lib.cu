@@ -455,10 +455,14 @@ struct FastOp {
   bool mma_pipelined = false;         // its bulk-copy pipelined form
 
   cudaError_t dispatch(const FastArgs<S, T>& a, int epi) const {
-    if constexpr (std::is_same<S, __half>::value) {
-      if (mma) return launch_fast_mma(a, tl, epi, st, stage, mma_pipelined);
+    if constexpr (std::is_same<S, double>::value) {
+      return launch_hop64(a, epi, st);
+    } else {
+      if constexpr (std::is_same<S, __half>::value) {
+        if (mma) return launch_fast_mma(a, tl, epi, st, stage, mma_pipelined);
+      }
+      return launch_fast<S, T>(a, tl, epi, st, stage);
     }
-    return launch_fast<S, T>(a, tl, epi, st, stage);
   }
 
   cudaError_t run(int epi, int out_par, int dagger, F<S> in, F<S> same, F<S> add, T g_same, T kappa, F<S> out,
@@ -556,11 +560,14 @@ void choose_hop(FastOp<S, T>& op, const Cfg* cfg, int nsb_req, int variant, cons
 template <typename S>
 Tiling fast_tiling(const Geom& g, int L5, int N, int nsb_req, bool* staged, bool allow_staging) {
   using T = typename StoreTraits<S>::T;
+  *staged = false;
+  if constexpr (std::is_same<S, double>::value) {
+    return make_tiling(g.Vh, L5, N, 1, 512);   // the FP64 hop has its own shape (hop64.cu)
+  } else {
   int maxthr = fast_max_threads<S, T>();
   if (maxthr > 1024) maxthr = 1024;
   const int upb = L5 * N;
-  *staged = false;
-  if (allow_staging && !std::is_same<S, double>::value && upb <= maxthr) {
+  if (allow_staging && upb <= maxthr) {
     int nsb = nsb_req > 0 ? nsb_req : (128 / upb > 1 ? 128 / upb : 1);
     if (nsb > 64) nsb = 64;
     for (; nsb >= 1; nsb--) {
@@ -573,11 +580,11 @@ Tiling fast_tiling(const Geom& g, int L5, int N, int nsb_req, bool* staged, bool
   if (smem_thr < maxthr) maxthr = smem_thr;
   int nsb = nsb_req > 0 ? nsb_req : 2;
   if (nsb > 64) nsb = 64;
-  // by default keep every RHS slot of a site in one block (no ragged slot groups,
-  // whose idle lanes cost the FP64 hop 40 % of its time when 2 sites did not fit)
+  // by default keep every RHS slot of a site in one block (no ragged slot groups)
   if (nsb_req <= 0)
     while (nsb > 1 && nsb * L5 * N > maxthr) nsb--;
   return make_tiling(g.Vh, L5, N, nsb, maxthr);
+  }
 }
 
 // Bound of device-side waits in clock cycles.
@@ -1101,15 +1108,10 @@ int solve_batch_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const* srcs, 
       CK(cudaMemcpyAsync(bo.data(), tmp, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
       CK(cudaStreamSynchronize(st));
     }
-    Op<double, double> loc;
-    loc.g = g; loc.L5 = L5; loc.N = N; loc.anti = cfg->anti; loc.U = cfg->U64; loc.st = st;
-    loc.tl = tiling_for<double>(g, L5, N, sv.op64.tl.nsb, true);
-    loc.launches = &sv.launches;
-    Tables tab;
-    tab.build(cfg->act, masses);
-    DevTables<double> M;
-    CK(upload_tables_ws<double>(ctx, sv.wsp + "tables", tab, &M, st));
-    CK(loc.run(false, 1, 0, sv.b_o, none, M[MK_BAinv], none, nullptr, 0.0, sv.t64, nullptr, nullptr));
+    // B A^-1 b_o
+    sv.launches += 1;
+    CK(sv.op64.run(E_AINV_SAME, 1, 0, none, sv.b_o, none, 0.0, 0.0, sv.u64, nullptr, nullptr));
+    CK(bop<double>(sv.u64.v, nullptr, sv.t64.v, nullptr, sv.op64.f, sv.tl_blas, g.Vh, L5, N, nullptr, st));
     CK(sv.op64.run(E_RAW, 0, 0, sv.t64, none, sv.b_e, 0.0, 0.5, sv.bhat, nullptr, nullptr));
     if (sv.sym) {   // symmetric form: the right-hand side A^-1 bhat
       CK(sv.op64.run(E_AINV_SAME, 0, 0, none, sv.bhat, none, 0.0, 0.0, sv.t64, nullptr, nullptr));
@@ -1446,14 +1448,8 @@ struct SessionImpl : SessionBase {
     // bhat_e = b_e + 1/2 H_eo B A^-1 b_o on this slot
     {
       F<double> none;
-      Op<double, double> loc;
-      loc.g = g; loc.L5 = L5; loc.N = N; loc.anti = cfg->anti; loc.U = cfg->U64; loc.st = st;
-      loc.tl = tiling_for<double>(g, L5, N, sv.op64.tl.nsb, true);
-      Tables tab;
-      tab.build(cfg->act, masses);
-      DevTables<double> M;
-      CK(upload_tables_ws<double>(ctx, sv.wsp + "tables", tab, &M, st));
-      CK(loc.run(false, 1, 0, sv.b_o, none, M[MK_BAinv], none, nullptr, 0.0, sv.t64, m, nullptr));
+      CK(sv.op64.run(E_AINV_SAME, 1, 0, none, sv.b_o, none, 0.0, 0.0, sv.u64, m, nullptr));
+      CK(bop<double>(sv.u64.v, nullptr, sv.t64.v, nullptr, sv.op64.f, sv.tl_blas, g.Vh, L5, N, m, st));
       CK(sv.op64.run(E_RAW, 0, 0, sv.t64, none, sv.b_e, 0.0, 0.5, sv.bhat, m, nullptr));
       if (sv.sym) {
         CK(sv.op64.run(E_AINV_SAME, 0, 0, none, sv.bhat, none, 0.0, 0.0, sv.t64, m, nullptr));
@@ -1601,14 +1597,53 @@ int upload5(mdwf_ctx* ctx, const double* h, size_t n, DBuf& d, cudaStream_t st) 
   return MDWF_OK;
 }
 
-// Generic FP64 operator on device API-layout 5D fields, single RHS.
-//   kind 0: dslash (out_par, dagger)   1: mdwf D / D^+   2: 5D local op (op, dagger)
-//   4: Schur (dagger, precision)
-template <typename S>
-int schur_apply_impl(mdwf_ctx* ctx, Cfg* cfg, const double* in_dev, double* out_dev, int dagger, cudaStream_t st);
+// H, H^+ (kind 0) or D, D^+ (kind 1) of one field on the caller's layout, FP64, without packing it: the hop kernel
+// reads and writes the 5D arrays.  With halos: the time hops across the edges of a decomposed lattice.
+int hop_api(mdwf_ctx* ctx, const Cfg* cfg, int kind, int dagger, int out_par, const double* in, double* out,
+            const double* halo_next, const double* halo_prev, double sign_next, double sign_prev, cudaStream_t st) {
+  const Geom& g = ctx->g;
+  const Action& act = cfg->act;
+  const int L5 = act.L5;
+  const size_t n5 = (size_t)24 * g.V * L5;
+  cudaError_t e = cudaSuccess;
+  if (in < out + n5 && out < in + n5) {   // in place (or overlapping): the hop reads other sites than it writes
+    double* copy = (double*)ws_get(ctx, "apply.in", sizeof(double) * n5, &e);
+    CK(e);
+    CK(cudaMemcpyAsync(copy, in, sizeof(double) * n5, cudaMemcpyDeviceToDevice, st));
+    in = copy;
+  }
+  double* mass = (double*)ws_get(ctx, "apply.mass", sizeof(double), &e);
+  CK(e);
+  CK(cudaMemcpyAsync(mass, &act.mf, sizeof(double), cudaMemcpyHostToDevice, st));
+  FastArgs<double, double> a;
+  a.g = g; a.L5 = L5; a.N = 1; a.out_par = out_par; a.dagger = dagger; a.antiperiodic = cfg->anti;
+  a.in = in; a.in_nrm = nullptr; a.same = in; a.same_nrm = nullptr; a.add = nullptr; a.add_nrm = nullptr;
+  a.out = out; a.out_nrm = nullptr; a.U = cfg->U64; a.F16 = nullptr;
+  a.halo_fwd = halo_next; a.halo_bwd = halo_prev; a.halo_sgn_fwd = sign_next; a.halo_sgn_bwd = sign_prev;
+  a.f = make_fifth<double>(act, mass);
+  a.active = nullptr; a.partials = nullptr;
+  if (kind == 0) {
+    a.g_same = 0.0; a.kappa = 1.0;
+    if (out_par >= 0) CK(cudaMemsetAsync(out, 0, sizeof(double) * n5, st));
+    CK(launch_hop64_api(a, E_RAW, st));
+  } else {
+    a.g_same = 1.0; a.kappa = -0.5;
+    if (!dagger) {   // D x = A x - 1/2 H B x
+      double* u = (double*)ws_get(ctx, "apply.u", sizeof(double) * n5, &e);
+      CK(e);
+      CK(bop_api(in, u, g.V, L5, act.b5, act.c5, act.mf, st));
+      a.in = u;
+      CK(launch_hop64_api(a, E_A_SAME, st));
+    } else {         // D^+ x = A^+ x - 1/2 B^+ H^+ x
+      CK(launch_hop64_api(a, E_AD_SAME_BD, st));
+    }
+  }
+  return MDWF_OK;
+}
 
-int apply_dev(mdwf_ctx* ctx, Cfg* cfg, int kind, int arg1, int arg2, const double* in_dev, double* out_dev,
-              cudaStream_t st) {
+// A, B, A^-1 (op 0, 1, 2) or an adjoint on the caller's layout, FP64.
+int apply_5d_dev(mdwf_ctx* ctx, const Cfg* cfg, int which, int dagger, const double* in_dev, double* out_dev,
+                 cudaStream_t st) {
   const Geom& g = ctx->g;
   const int L5 = cfg->act.L5;
   Op<double, double> op;
@@ -1618,52 +1653,33 @@ int apply_dev(mdwf_ctx* ctx, Cfg* cfg, int kind, int arg1, int arg2, const doubl
   tab.build(cfg->act, std::vector<double>(1, cfg->act.mf));
   DevTables<double> M;
   CK(upload_tables_ws<double>(ctx, "apply.tables", tab, &M, st));
-  long units = g.Vh * L5;
-  // fields of the context's workspace: no allocation (and no device-wide
-  // synchronisation of a free) once they exist
-  struct WF {
-    F<double> w;
-    F<double> f() const { return w; }
-  } ie, io, oe, oo, te, to;
-  const char* names[] = {"apply.ie", "apply.io", "apply.oe", "apply.oo", "apply.te", "apply.to"};
-  WF* fs[] = {&ie, &io, &oe, &oo, &te, &to};
-  for (int i = 0; i < 6; i++) CK(ws_field<double>(ctx, names[i], units, &fs[i]->w));
-  CK(pack_rhs<double>(in_dev, ie.w.v, nullptr, g, L5, 1, 0, 0, st));
-  CK(pack_rhs<double>(in_dev, io.w.v, nullptr, g, L5, 1, 1, 0, st));
-  CK(cudaMemsetAsync(oe.w.v, 0, sizeof(double) * 24 * (size_t)units, st));
-  CK(cudaMemsetAsync(oo.w.v, 0, sizeof(double) * 24 * (size_t)units, st));
-  F<double> none;
-  cudaError_t me = cudaSuccess;
-  double* mass = (double*)ws_get(ctx, "apply.mass", sizeof(double), &me);
-  CK(me);
-  CK(cudaMemcpyAsync(mass, &cfg->act.mf, sizeof(double), cudaMemcpyHostToDevice, st));
-  FastOp<double, double> fo;
-  fo.g = g; fo.L5 = L5; fo.N = 1; fo.anti = cfg->anti; fo.U = cfg->U64; fo.st = st;
-  fo.f = make_fifth<double>(cfg->act, mass);
-  choose_hop(fo, cfg, 0, HOP_DIRECT, nullptr);
-  Tiling tb = make_tiling(g.Vh, L5, 1, 2, 512);
-  if (kind == 0) {
-    int par = arg1, dag = arg2;
-    if (par == 0 || par == -1) CK(fo.run(E_RAW, 0, dag, io.f(), none, none, 0.0, 1.0, oe.f(), nullptr, nullptr));
-    if (par == 1 || par == -1) CK(fo.run(E_RAW, 1, dag, ie.f(), none, none, 0.0, 1.0, oo.f(), nullptr, nullptr));
-  } else if (kind == 1) {
-    if (!arg1) {  // D x = A x - 1/2 H B x
-      CK(bop<double>(ie.f().v, nullptr, te.f().v, nullptr, fo.f, tb, g.Vh, L5, 1, nullptr, st));
-      CK(bop<double>(io.f().v, nullptr, to.f().v, nullptr, fo.f, tb, g.Vh, L5, 1, nullptr, st));
-      CK(fo.run(E_A_SAME, 0, 0, to.f(), ie.f(), none, 1.0, -0.5, oe.f(), nullptr, nullptr));
-      CK(fo.run(E_A_SAME, 1, 0, te.f(), io.f(), none, 1.0, -0.5, oo.f(), nullptr, nullptr));
-    } else {      // D^+ x = A^+ x - 1/2 B^+ H^+ x
-      CK(fo.run(E_AD_SAME_BD, 0, 1, io.f(), ie.f(), none, 1.0, -0.5, oe.f(), nullptr, nullptr));
-      CK(fo.run(E_AD_SAME_BD, 1, 1, ie.f(), io.f(), none, 1.0, -0.5, oo.f(), nullptr, nullptr));
-    }
-  } else if (kind == 2) {
-    static const int kinds[3][2] = {{MK_A, MK_Ad}, {MK_B, MK_Bd}, {MK_Ainv, MK_Ainvd}};
-    const double* G = M[kinds[arg1][arg2 ? 1 : 0]];
-    CK(op.run(false, 0, 0, ie.f(), none, G, none, nullptr, 0.0, oe.f(), nullptr, nullptr));
-    CK(op.run(false, 1, 0, io.f(), none, G, none, nullptr, 0.0, oo.f(), nullptr, nullptr));
+  const long units = g.Vh * L5;
+  F<double> in, out, none;
+  CK(ws_field<double>(ctx, "apply.ie", units, &in));
+  CK(ws_field<double>(ctx, "apply.oe", units, &out));
+  static const int kinds[3][2] = {{MK_A, MK_Ad}, {MK_B, MK_Bd}, {MK_Ainv, MK_Ainvd}};
+  const double* G = M[kinds[which][dagger ? 1 : 0]];
+  for (int par = 0; par < 2; par++) {
+    CK(pack_rhs<double>(in_dev, in.v, nullptr, g, L5, 1, par, 0, st));
+    CK(op.run(false, par, 0, in, none, G, none, nullptr, 0.0, out, nullptr, nullptr));
+    CK(unpack_rhs<double>(out.v, nullptr, out_dev, g, L5, 1, par, 0, st));
   }
-  CK(unpack_rhs<double>(oe.w.v, nullptr, out_dev, g, L5, 1, 0, 0, st));
-  CK(unpack_rhs<double>(oo.w.v, nullptr, out_dev, g, L5, 1, 1, 0, st));
+  CK(cudaStreamSynchronize(st));
+  return MDWF_OK;
+}
+
+// Generic FP64 operator on device API-layout 5D fields, single RHS.
+//   kind 0: dslash (out_par, dagger)   1: mdwf D / D^+   2: 5D local op (op, dagger)
+//   4: Schur (dagger, precision)
+template <typename S>
+int schur_apply_impl(mdwf_ctx* ctx, Cfg* cfg, const double* in_dev, double* out_dev, int dagger, cudaStream_t st);
+
+int apply_dev(mdwf_ctx* ctx, Cfg* cfg, int kind, int arg1, int arg2, const double* in_dev, double* out_dev,
+              cudaStream_t st) {
+  if (kind == 2) return apply_5d_dev(ctx, cfg, arg1, arg2, in_dev, out_dev, st);
+  int rc = hop_api(ctx, cfg, kind, kind == 0 ? arg2 : arg1, kind == 0 ? arg1 : -1, in_dev, out_dev, nullptr, nullptr,
+                   1.0, 1.0, st);
+  if (rc) return rc;
   CK(cudaStreamSynchronize(st));
   return MDWF_OK;
 }
@@ -1686,8 +1702,14 @@ int dd_impl(mdwf_ctx* ctx, Cfg* cfg, bool pack, int kind, int dagger, const doub
   const Geom& g = ctx->g;
   const int L5 = cfg->act.L5;
   if (g.L[3] < 2 || (g.L[3] & 1)) return fail(ctx, MDWF_ERR_ARG, "dd: the local time extent must be even");
+  if (!pack) {
+    int rc = hop_api(ctx, cfg, kind, dagger, -1, in_dev, out_dev, halo_next, halo_prev, sign_next, sign_prev, st);
+    if (rc) return rc;
+    CK(cudaStreamSynchronize(st));
+    return MDWF_OK;
+  }
   const long units = g.Vh * L5;
-  F<double> ie, io, te, to, oe, oo;
+  F<double> ie, io, te, to;
   CK(ws_field<double>(ctx, "dd.ie", units, &ie));
   CK(ws_field<double>(ctx, "dd.io", units, &io));
   CK(ws_field<double>(ctx, "dd.te", units, &te));
@@ -1698,43 +1720,17 @@ int dd_impl(mdwf_ctx* ctx, Cfg* cfg, bool pack, int kind, int dagger, const doub
   double* mass = (double*)ws_get(ctx, "dd.mass", sizeof(double), &me);
   CK(me);
   CK(cudaMemcpyAsync(mass, &cfg->act.mf, sizeof(double), cudaMemcpyHostToDevice, st));
-  FastOp<double, double> fo;
-  fo.g = g; fo.L5 = L5; fo.N = 1; fo.anti = cfg->anti; fo.U = cfg->U64; fo.st = st;
-  fo.f = make_fifth<double>(cfg->act, mass);
-  choose_hop(fo, cfg, 0, HOP_DIRECT, nullptr);
+  const Fifth<double> f = make_fifth<double>(cfg->act, mass);
   Tiling tb = make_tiling(g.Vh, L5, 1, 2, 512);
   // the field the hop reads: B in for D, in otherwise
   const bool bfirst = kind == 1 && !dagger;
   if (bfirst) {
-    CK(bop<double>(ie.v, nullptr, te.v, nullptr, fo.f, tb, g.Vh, L5, 1, nullptr, st));
-    CK(bop<double>(io.v, nullptr, to.v, nullptr, fo.f, tb, g.Vh, L5, 1, nullptr, st));
+    CK(bop<double>(ie.v, nullptr, te.v, nullptr, f, tb, g.Vh, L5, 1, nullptr, st));
+    CK(bop<double>(io.v, nullptr, to.v, nullptr, f, tb, g.Vh, L5, 1, nullptr, st));
   }
   const F<double> he = bfirst ? te : ie, ho = bfirst ? to : io;
-  if (pack) {
-    CK(dd_pack_faces(he.v, g, 0, L5, 1, dagger, cfg->U64, face_prev, face_next, st));
-    CK(dd_pack_faces(ho.v, g, 1, L5, 1, dagger, cfg->U64, face_prev, face_next, st));
-    CK(cudaStreamSynchronize(st));
-    return MDWF_OK;
-  }
-  CK(ws_field<double>(ctx, "dd.oe", units, &oe));
-  CK(ws_field<double>(ctx, "dd.oo", units, &oo));
-  fo.halo_fwd = halo_next;
-  fo.halo_bwd = halo_prev;
-  fo.halo_sgn_fwd = sign_next;
-  fo.halo_sgn_bwd = sign_prev;
-  F<double> none;
-  if (kind == 0) {
-    CK(fo.run(E_RAW, 0, dagger, ho, none, none, 0.0, 1.0, oe, nullptr, nullptr));
-    CK(fo.run(E_RAW, 1, dagger, he, none, none, 0.0, 1.0, oo, nullptr, nullptr));
-  } else if (!dagger) {   // D x = A x - 1/2 H B x
-    CK(fo.run(E_A_SAME, 0, 0, to, ie, none, 1.0, -0.5, oe, nullptr, nullptr));
-    CK(fo.run(E_A_SAME, 1, 0, te, io, none, 1.0, -0.5, oo, nullptr, nullptr));
-  } else {                // D^+ x = A^+ x - 1/2 B^+ H^+ x
-    CK(fo.run(E_AD_SAME_BD, 0, 1, io, ie, none, 1.0, -0.5, oe, nullptr, nullptr));
-    CK(fo.run(E_AD_SAME_BD, 1, 1, ie, io, none, 1.0, -0.5, oo, nullptr, nullptr));
-  }
-  CK(unpack_rhs<double>(oe.v, nullptr, out_dev, g, L5, 1, 0, 0, st));
-  CK(unpack_rhs<double>(oo.v, nullptr, out_dev, g, L5, 1, 1, 0, st));
+  CK(dd_pack_faces(he.v, g, 0, L5, 1, dagger, cfg->U64, face_prev, face_next, st));
+  CK(dd_pack_faces(ho.v, g, 1, L5, 1, dagger, cfg->U64, face_prev, face_next, st));
   CK(cudaStreamSynchronize(st));
   return MDWF_OK;
 }

@@ -357,7 +357,7 @@ struct FastArgs {
   const T* U;
   const uint32_t* F16;  // tensor-core hop: fp16 B fragments [parity][h][mu][fwd, bwd][lane], or null
   const float* U12 = nullptr;  // two-row (12-real) FP32 links [parity][h][mu][12] (hop_pair.cu only)
-  // Domain decomposition in time (hop_fast.cu kernels): when halo_fwd is set, the
+  // Domain decomposition in time (hop64.cu): when halo_fwd is set, the
   // t-neighbours across both edges of the local lattice come from the faces of
   // the neighbouring sub-domains instead of the local field: halo_fwd[(lex3 L5 + s) N + r]
   // holds the 12 reals of the projected half spinor of the next sub-domain's
@@ -374,6 +374,15 @@ struct FastArgs {
   double* partials;
 };
 
+// B x of one component, b5 x + cw y with y the component of the neighbour slice and cw = c5 times its
+// wall factor: one rounding order for every kernel that forms it.
+__device__ __forceinline__ double bop_term(double b5, double x, double cw, double y) {
+  return __fma_rn(b5, x, __dmul_rn(cw, y));
+}
+__device__ __forceinline__ float bop_term(float b5, float x, float cw, float y) {
+  return __fmaf_rn(b5, x, __fmul_rn(cw, y));
+}
+
 // Shared-memory staging of the neighbour sites (hop_staged_kernel).
 #define MDWF_TIMEOUT_CODE 1
 struct StageInfo {
@@ -387,6 +396,11 @@ struct StageInfo {
 template <typename S, typename T>
 cudaError_t launch_fast(const FastArgs<S, T>& a, const Tiling& t, int epi, cudaStream_t st,
                         const StageInfo* stage = nullptr);
+// FP64 hop (hop64.cu), on parity fields (a.active masks slots) or on the caller's arrays (one slot; out_par -1:
+// both parities; E_RAW, E_A_SAME, E_AD_SAME_BD); u = B x on the caller's layout, V sites.
+cudaError_t launch_hop64(const FastArgs<double, double>& a, int epi, cudaStream_t st);
+cudaError_t launch_hop64_api(const FastArgs<double, double>& a, int epi, cudaStream_t st);
+cudaError_t bop_api(const double* x, double* u, long V, int L5, double b5, double c5, double m, cudaStream_t st);
 // Two-slices-per-thread hop (hop_pair.cu): block (rt, J = ceil(L5 / 2), nsb).
 struct PairShape {
   int J, nsb, rt, threads;
