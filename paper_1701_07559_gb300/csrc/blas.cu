@@ -234,16 +234,74 @@ __global__ void k_norm2(const S* __restrict__ v, const float* __restrict__ v_nrm
   block_partial(n2, x, tl, L5, Vh, partials);
 }
 
-// out[r] = sum_h partials[r][h] in a fixed order that depends on nsites only: a
-// cluster of kFinCluster blocks per slot, block c summing the c-th contiguous
-// chunk (thread t takes sites t, t+256, ... of it, then a fixed tree), and block
-// 0 adding the blocks' sums in rank order through distributed shared memory.
-// Spreading a slot over several SMs matters on a part with few FP64 adders per SM.
+// The scalar step of a CG iteration that needs slot r's sum v.
+//
+// FIN_RHO: the low-precision residual recursion can stagnate for a system whose
+// residual is already tiny: it neither reaches the stopping norm nor drops by
+// delta, so no update would ever come.  After stag_max iterations without an
+// update one is forced; it is followed by an FP64 re-reference and a restart of
+// the search direction (beta = 0).
+template <int OP>
+__device__ __forceinline__ void cg_step(const Scal& c, int r, double v, double* out) {
+  if (OP == FIN_STORE) out[r] = v;
+  if (OP == FIN_ALPHA) {
+    c.qq[r] = v;
+    if (c.active[r]) c.alpha[r] = v > 0.0 ? c.gamma[r] / v : 0.0;
+  }
+  if (OP == FIN_RHO) {
+    c.tmp[r] = v;
+    if (c.active[r]) {
+      c.rho2[r] = v;
+      if (v > c.rho2_max[r]) c.rho2_max[r] = v;
+      if (v <= c.stop2[r]) { c.active[r] = 0; c.flags[r] |= FLAG_INNER_DONE; }
+      else if (v < c.delta2 * c.rho2_max[r] || v <= c.tau2 * c.bhat2[r]) c.flags[r] |= FLAG_UPDATE;
+      else if (c.since[r] >= c.stag_max) c.flags[r] |= FLAG_UPDATE | FLAG_STAG;
+    }
+  }
+  if (OP == FIN_BETA) {
+    c.rr[r] = v;
+    if (c.active[r]) {
+      const double g = c.gamma[r];
+      c.beta[r] = g > 0.0 ? v / g : 0.0;
+      c.gamma_prev[r] = g;
+      c.gamma[r] = v;
+      c.iters[r] += 1;
+      c.since[r] += 1;
+    }
+  }
+}
+
+// Sum of a block's 256 values by its first warp, in thread 0 (fixed order): an FP64 instruction costs a
+// warp 64 clocks whatever its active lanes, so the tree runs on one warp after one exchange.
+__device__ __forceinline__ double block_sum256(double s, double* sh) {
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1) s += __shfl_down_sync(0xffffffffu, s, w);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  __syncthreads();
+  double t = threadIdx.x < 8 ? sh[threadIdx.x] : 0.0;
+  if (threadIdx.x < 32) {
+#pragma unroll
+    for (int w = 4; w > 0; w >>= 1) t += __shfl_down_sync(0xffffffffu, t, w);
+  }
+  return t;
+}
+
+// sum_h partials[r][h] of slot r in a fixed order that depends on nsites only,
+// then the scalar step.  A cluster of kFinCluster blocks per slot: block c sums the
+// c-th contiguous chunk (thread t takes sites t, t+256, ... of it, then a fixed
+// tree), and block 0 adds the blocks' sums in rank order through distributed
+// shared memory.  Spreading a slot over several SMs matters on a part with few FP64
+// adders per SM; up to kFinSmall sites a single block is faster than the
+// cluster's two barriers (5.6 us for the cluster and 3 us for a scalar kernel after it
+// at 2048 sites; 4096 sites are 16 additions per thread).
 constexpr int kFinCluster = 8;
+constexpr long kFinSmall = 4096;
+template <int OP>
 __global__ void __cluster_dims__(kFinCluster, 1, 1) __launch_bounds__(256)
-    k_finalize(const double* __restrict__ partials, long nsites, double* __restrict__ out) {
+    k_finalize(const double* __restrict__ partials, long nsites, Scal sc, double* __restrict__ out) {
   namespace cg = cooperative_groups;
-  __shared__ double sh[256];
+  __shared__ double sh[8];
+  __shared__ double total;
   cg::cluster_group cluster = cg::this_cluster();
   const int r = blockIdx.y;
   const int c = (int)cluster.block_rank();
@@ -252,20 +310,26 @@ __global__ void __cluster_dims__(kFinCluster, 1, 1) __launch_bounds__(256)
   const long end = beg + len < nsites ? beg + len : nsites;
   const double* p = partials + (long)r * nsites;
   double s = 0.0;
-  for (long k = beg + threadIdx.x; k < end; k += blockDim.x) s += p[k];
-  sh[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-    __syncthreads();
-  }
+  for (long k = beg + threadIdx.x; k < end; k += 256) s += p[k];
+  s = block_sum256(s, sh);
+  if (threadIdx.x == 0) total = s;
   cluster.sync();
   if (c == 0 && threadIdx.x == 0) {
     double tot = 0.0;
-    for (int q = 0; q < kFinCluster; q++) tot += *cluster.map_shared_rank(&sh[0], q);
-    out[r] = tot;
+    for (int q = 0; q < kFinCluster; q++) tot += *cluster.map_shared_rank(&total, q);
+    cg_step<OP>(sc, r, tot, out);
   }
   cluster.sync();   // every block's sum stays readable until block 0 has added it
+}
+template <int OP>
+__global__ void __launch_bounds__(256) k_finalize_small(const double* __restrict__ partials, int nsites, Scal sc,
+                                                        double* __restrict__ out) {
+  __shared__ double sh[8];
+  const double* p = partials + (long)blockIdx.x * nsites;
+  double s = 0.0;
+  for (int k = threadIdx.x; k < nsites; k += 256) s += p[k];
+  s = block_sum256(s, sh);
+  if (threadIdx.x == 0) cg_step<OP>(sc, blockIdx.x, s, out);
 }
 
 // u = B x on one parity: P_+ half b5 x_s + c5 x_{s-1}, P_- half b5 x_s + c5 x_{s+1},
@@ -495,9 +559,40 @@ cudaError_t z2_source(unsigned long long seed, double* eta, long V, cudaStream_t
   return cudaGetLastError();
 }
 
-cudaError_t finalize(const double* partials, long ntiles, int N, double* out, cudaStream_t st) {
-  k_finalize<<<dim3(kFinCluster, (unsigned)N), 256, 0, st>>>(partials, ntiles, out);
+template <int OP>
+static cudaError_t finalize_one(const double* partials, long nsites, int N, const Scal& c, double* out, cudaStream_t st) {
+  if (nsites <= kFinSmall) k_finalize_small<OP><<<N, 256, 0, st>>>(partials, (int)nsites, c, out);
+  else k_finalize<OP><<<dim3(kFinCluster, (unsigned)N), 256, 0, st>>>(partials, nsites, c, out);
   return cudaGetLastError();
+}
+cudaError_t finalize(const double* partials, long ntiles, int N, double* out, cudaStream_t st) {
+  return finalize_one<FIN_STORE>(partials, ntiles, N, Scal(), out, st);
+}
+cudaError_t finalize_cg(const double* partials, long nsites, int N, const Scal& c, FinOp op, cudaStream_t st) {
+  switch (op) {
+    case FIN_ALPHA: return finalize_one<FIN_ALPHA>(partials, nsites, N, c, nullptr, st);
+    case FIN_RHO: return finalize_one<FIN_RHO>(partials, nsites, N, c, nullptr, st);
+    case FIN_BETA: return finalize_one<FIN_BETA>(partials, nsites, N, c, nullptr, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+Tiling blas_tiling(long Vh, int L5, int N, int max_threads) {
+  // the threads wanted: 256, fewer on lattices that would leave SMs without a block
+  const long units = Vh * L5 * N;
+  long want = units / 152;
+  want = want > 256 ? 256 : want < 32 ? 32 : want;
+  // the number of sites per block with the best-filled warps among those near that size
+  int best = 1;
+  double score = -1.0;
+  for (int nsb = 1; nsb <= 64 && nsb * L5 <= max_threads; nsb++) {
+    const Tiling t = make_tiling(Vh, L5, N, nsb, max_threads);
+    if (nsb > 1 && (t.ngroups > 1 || t.threads > 1.5 * want)) break;
+    const double fill = (double)t.threads / ((t.threads + 31) / 32 * 32);
+    const double size = t.threads < want ? (double)t.threads / want : 1.0;
+    if (fill * size > score + 1e-9) { score = fill * size; best = nsb; }
+  }
+  return make_tiling(Vh, L5, N, best, max_threads);
 }
 
 #define MDWF_INST_S(S)                                                                                          \

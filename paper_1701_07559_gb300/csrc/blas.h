@@ -4,6 +4,25 @@
 
 namespace mdwf {
 
+// Tiling of the unit-wise kernels: whole sites per block, 32 to 256 threads in full warps where the
+// sizes allow it.
+Tiling blas_tiling(long Vh, int L5, int N, int max_threads);
+
+// Per-slot scalars of the batched CG.
+struct Scal {
+  double *gamma, *gamma_prev, *alpha, *beta, *rho2, *rho2_max, *stop2, *qq, *rr, *tmp, *bhat2, *upd2;
+  int *active, *flags, *iters;
+  int* since;     // CG iterations since the last reliable update of the slot
+  int stag_max;   // that many without one: the inner recursion stagnates
+  double delta2;  // periodic reliable update when |rho|^2 < delta2 * max |rho|^2 since the last one
+  double tau2;    // FP64 re-reference when |rho|^2 <= tau2 * |bhat|^2 (bhat = current reference residual)
+};
+enum { FLAG_INNER_DONE = 1, FLAG_UPDATE = 2, FLAG_DONE = 4, FLAG_REREF = 8, FLAG_STAG = 16 };
+// The reductions of a CG iteration, each with the scalar step it feeds: |q|^2 and alpha, |rho|^2 and the
+// stopping and update decisions, |r|^2 and beta.
+enum FinOp { FIN_STORE = 0, FIN_ALPHA = 1, FIN_RHO = 2, FIN_BETA = 3 };
+cudaError_t finalize_cg(const double* partials, long nsites, int N, const Scal& c, FinOp op, cudaStream_t st);
+
 // API layout (one RHS, [s][t][z][y][x][spin][colour][re,im], FP64, device) <-> slot r of a parity field.
 template <typename S>
 cudaError_t pack_rhs(const double* api, S* out, float* out_nrm, const Geom& g, int L5, int N, int par, int r,

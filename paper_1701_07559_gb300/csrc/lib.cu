@@ -342,49 +342,9 @@ Tiling tiling_for(const Geom& g, int L5, int N, int nsb, bool two_buffers) {
 }
 
 // ---------------------------------------------------------------------------
-// Scalar kernels of the batched CG (one thread per RHS slot)
+// Scalar kernels of the reliable updates (one thread per RHS slot); those of the
+// CG iteration run at the end of its reductions (finalize_cg, blas.cu)
 // ---------------------------------------------------------------------------
-struct Scal {
-  double *gamma, *gamma_prev, *alpha, *beta, *rho2, *rho2_max, *stop2, *qq, *rr, *tmp, *bhat2, *upd2;
-  int *active, *flags, *iters;
-  int* since;     // CG iterations since the last reliable update of the slot
-  int stag_max;   // that many without one: the inner recursion stagnates (see k_after_rho)
-  double delta2;  // periodic reliable update when |rho|^2 < delta2 * max |rho|^2 since the last one
-  double tau2;    // FP64 re-reference when |rho|^2 <= tau2 * |bhat|^2 (bhat = current reference residual)
-};
-enum { FLAG_INNER_DONE = 1, FLAG_UPDATE = 2, FLAG_DONE = 4, FLAG_REREF = 8, FLAG_STAG = 16 };
-
-__global__ void k_alpha(Scal c, int N) {
-  int r = threadIdx.x;
-  if (r < N && c.active[r]) { double q = c.qq[r]; c.alpha[r] = q > 0.0 ? c.gamma[r] / q : 0.0; }
-}
-// The low-precision residual recursion can stagnate for a system whose
-// residual is already tiny: it neither reaches the stopping norm nor drops by
-// delta, so no update would ever come.  After stag_max iterations without an
-// update one is forced; it is followed by an FP64 re-reference and a restart of
-// the search direction (beta = 0).
-__global__ void k_after_rho(Scal c, int N) {
-  int r = threadIdx.x;
-  if (r < N && c.active[r]) {
-    double v = c.tmp[r];
-    c.rho2[r] = v;
-    if (v > c.rho2_max[r]) c.rho2_max[r] = v;
-    if (v <= c.stop2[r]) { c.active[r] = 0; c.flags[r] |= FLAG_INNER_DONE; }
-    else if (v < c.delta2 * c.rho2_max[r] || v <= c.tau2 * c.bhat2[r]) c.flags[r] |= FLAG_UPDATE;
-    else if (c.since[r] >= c.stag_max) c.flags[r] |= FLAG_UPDATE | FLAG_STAG;
-  }
-}
-__global__ void k_beta(Scal c, int N) {
-  int r = threadIdx.x;
-  if (r < N && c.active[r]) {
-    double rr = c.rr[r], g = c.gamma[r];
-    c.beta[r] = g > 0.0 ? rr / g : 0.0;
-    c.gamma_prev[r] = g;
-    c.gamma[r] = rr;
-    c.iters[r] += 1;
-    c.since[r] += 1;
-  }
-}
 // After a residual recomputed with FP32 arithmetic.  Its error grows like
 // 1e-7 kappa(Mhat) |bhat| (x_hi, accumulated since the last re-reference, is
 // about kappa times bhat), so for light quarks it can sit above any fixed
@@ -710,7 +670,7 @@ struct BatchSolver {
     opS.U = kFP64 ? (const T*)cf->U64 : (const T*)cf->U32;
     opS.f = make_fifth<T>(cf->act, kFP64 ? (const T*)mass64 : (const T*)mass32);
     if (nsb * L5 > 1024) nsb = 1;
-    tl_blas = make_tiling(g.Vh, L5, N, 2, kFP64 ? 512 : 1024);
+    tl_blas = blas_tiling(g.Vh, L5, N, kFP64 ? 512 : 1024);
     errw = (int*)ws_get(c, wsp + "errw", sizeof(int), &e); CK(e);
     CK(cudaMemsetAsync(errw, 0, sizeof(int), st));
     stage.spin_bytes = stage.nrm_bytes = 0;
@@ -870,25 +830,22 @@ struct BatchSolver {
     const Geom& g = ctx->g;
     cudaStream_t st = op64.st;
     cudaError_t e;
-    launches += 8;  // xpay_b, axpy, 3 finalize, 3 scalar kernels (+ 4 hops counted in FastOp::run)
+    launches += 5;  // xpay_b, axpy, 3 reductions with the scalar steps (+ 4 hops counted in FastOp::run)
     e = xpay_b<S>(r.v, r.n, p.v, p.n, u.v, u.n, sc.beta, opS.f, tl_blas, g.Vh, L5, N, sc.active, st);
     if (e != cudaSuccess) return e;
     e = sym ? opS.mhat_sym(p, u, t, q, sc.active, part) : opS.mhat(p, u, t, q, sc.active, part);
     if (e != cudaSuccess) return e;
-    e = finalize(part, g.Vh, N, sc.qq, st);
+    e = finalize_cg(part, g.Vh, N, sc, FIN_ALPHA, st);
     if (e != cudaSuccess) return e;
-    k_alpha<<<1, 1024, 0, st>>>(sc, N);
     e = axpy_x_rho<SX, S>(xlo.v, p.v, p.n, rho.v, rho.n, q.v, q.n, sc.alpha, tl_blas, g.Vh, L5, N, sc.active, part, st);
     if (e != cudaSuccess) return e;
-    e = finalize(part, g.Vh, N, sc.tmp, st);
+    e = finalize_cg(part, g.Vh, N, sc, FIN_RHO, st);
     if (e != cudaSuccess) return e;
-    k_after_rho<<<1, 1024, 0, st>>>(sc, N);
     // (u = B p is dead here: the symmetric form's scratch)
     e = sym ? opS.mhat_sym_dag(rho, u, t, r, sc.active, part) : opS.mhat_dag(rho, t, r, sc.active, part);
     if (e != cudaSuccess) return e;
-    e = finalize(part, g.Vh, N, sc.rr, st);
+    e = finalize_cg(part, g.Vh, N, sc, FIN_BETA, st);
     if (e != cudaSuccess) return e;
-    k_beta<<<1, 1024, 0, st>>>(sc, N);
     return cudaGetLastError();
   }
 
@@ -1721,7 +1678,7 @@ int dd_impl(mdwf_ctx* ctx, Cfg* cfg, bool pack, int kind, int dagger, const doub
   CK(me);
   CK(cudaMemcpyAsync(mass, &cfg->act.mf, sizeof(double), cudaMemcpyHostToDevice, st));
   const Fifth<double> f = make_fifth<double>(cfg->act, mass);
-  Tiling tb = make_tiling(g.Vh, L5, 1, 2, 512);
+  Tiling tb = blas_tiling(g.Vh, L5, 1, 512);
   // the field the hop reads: B in for D, in otherwise
   const bool bfirst = kind == 1 && !dagger;
   if (bfirst) {
@@ -1757,7 +1714,7 @@ int schur_apply_impl(mdwf_ctx* ctx, Cfg* cfg, const double* in_dev, double* out_
   si.extra_tx = 0;
   si.err = errw.as<int>();
   choose_hop(op, cfg, 0, HOP_AUTO, &si);
-  Tiling tb = make_tiling(g.Vh, L5, 1, 2, 512);
+  Tiling tb = blas_tiling(g.Vh, L5, 1, 512);
   long units = g.Vh * L5;
   FieldBuf<S> in, u, t, out;
   for (auto* f : {&in, &u, &t, &out}) CK(f->alloc(units));
@@ -1808,7 +1765,7 @@ int schur_batch_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const* in, do
     if (int r12 = ensure_u12(ctx, cfg)) return r12;
     op.U12 = std::is_same<T, double>::value ? nullptr : cfg->U12;
   }
-  Tiling tb = make_tiling(g.Vh, L5, N, 2, 1024);
+  Tiling tb = blas_tiling(g.Vh, L5, N, 1024);
   F<S> fin, fu, ft, fo;
   CK(ws_field<S>(ctx, "sb.in", units, &fin));
   CK(ws_field<S>(ctx, "sb.u", units, &fu));
@@ -2433,7 +2390,7 @@ int schur_batch_noalloc_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const
   op.U = std::is_same<T, double>::value ? (const T*)cfg->U64 : (const T*)cfg->U32;
   op.f = make_fifth<T>(cfg->act, mass);
   choose_hop(op, cfg, 0, HOP_DIRECT, nullptr);
-  Tiling tb = make_tiling(g.Vh, L5, N, 2, 1024);
+  Tiling tb = blas_tiling(g.Vh, L5, N, 1024);
   for (int i = 0; i < N; i++) CK(pack_rhs<S>(in[i], fin.v, fin.n, g, L5, N, 0, i, st));
   if (!dagger) {
     CK(bop<S>(fin.v, fin.n, fu.v, fu.n, op.f, tb, g.Vh, L5, N, nullptr, st));
