@@ -31,43 +31,6 @@ __device__ __forceinline__ Unit unit_of(const Tiling& tl, long Vh, int L5, int N
   return x;
 }
 
-// The FP32 solution accumulator x_lo of the mixed-precision solver is stored
-// tile-major: block b = blockIdx.y * gridDim.x + blockIdx.x of the BLAS tiling
-// holds its T = tl.threads units as six planes of float4 (plane k: components
-// 4k .. 4k+3 of the [spin][colour][re, im] order), thread t's plane k at float4
-// index (6 b + k) T + t.  One plane of a warp is 512 contiguous bytes, where the
-// unit-major layout would stride each thread's 16 bytes by 96.  Every kernel that
-// touches x_lo uses the same tiling; the field holds xlo_units(tl) units.  An
-// FP64 accumulator (the FP64 solver) keeps the unit-major layout.
-template <typename SX>
-struct XloLayout {
-  static __device__ __forceinline__ void load(const SX* v, const Unit& x, const Tiling&, SX a[24]) {
-    load24<SX, SX>(v, nullptr, x.u, a);
-  }
-  static __device__ __forceinline__ void store(SX* v, const Unit& x, const Tiling&, const SX a[24]) {
-    store24<SX, SX>(v, nullptr, x.u, a);
-  }
-};
-template <>
-struct XloLayout<float> {
-  static __device__ __forceinline__ long base(const Tiling& tl) {
-    return ((long)blockIdx.y * gridDim.x + blockIdx.x) * 6 * tl.threads + threadIdx.x;
-  }
-  static __device__ __forceinline__ void load(const float* v, const Unit&, const Tiling& tl, float a[24]) {
-    const float4* p = reinterpret_cast<const float4*>(v) + base(tl);
-#pragma unroll
-    for (int k = 0; k < 6; k++) {
-      const float4 t = __ldg(p + (long)k * tl.threads);
-      a[4 * k] = t.x; a[4 * k + 1] = t.y; a[4 * k + 2] = t.z; a[4 * k + 3] = t.w;
-    }
-  }
-  static __device__ __forceinline__ void store(float* v, const Unit&, const Tiling& tl, const float a[24]) {
-    float4* p = reinterpret_cast<float4*>(v) + base(tl);
-#pragma unroll
-    for (int k = 0; k < 6; k++) p[(long)k * tl.threads] = make_float4(a[4 * k], a[4 * k + 1], a[4 * k + 2], a[4 * k + 3]);
-  }
-};
-
 // Per-site, per-slot sum of `v` over the L5 slices (fixed order), written to
 // partials[r][h]; the final sum over sites is then independent of the tiling.
 __device__ __forceinline__ void block_partial(double v, const Unit& x, const Tiling& tl, int L5, long Vh,
@@ -82,38 +45,50 @@ __device__ __forceinline__ void block_partial(double v, const Unit& x, const Til
   }
 }
 
-template <typename S>
-__global__ void k_pack(const double* __restrict__ api, S* __restrict__ out, float* __restrict__ out_nrm, Geom g,
-                       int L5, int N, int par, int r) {
-  using T = typename StoreTraits<S>::T;
-  long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= g.Vh * L5) return;
-  long h = idx / L5;
-  int s = (int)(idx - h * L5);
-  int c[4];
-  site_coords(g, par, h, c);
-  long lex = lex_index(g, c);
-  const double* src = api + ((long)s * g.V + lex) * 24;
-  T a[24];
-#pragma unroll
-  for (int i = 0; i < 24; i++) a[i] = (T)src[i];
-  store24<S, T>(out, out_nrm, (h * L5 + s) * N + r, a);
-}
+// The caller's fields (C ABI layout, aligned to a double) of the slots r0 .. r0 + nr - 1 <-> one parity of a field.
+// A thread per unit, slots fastest: the words of consecutive slots are contiguous in the planes.
+constexpr int kPtrs = 64;
+template <typename P>
+struct Ptrs {
+  P p[kPtrs];
+};
 
 template <typename S>
-__global__ void k_unpack(const S* __restrict__ in, const float* __restrict__ in_nrm, double* __restrict__ api, Geom g,
-                         int L5, int N, int par, int r) {
+__global__ void __launch_bounds__(256) k_pack(Ptrs<const double*> api, S* __restrict__ out, float* __restrict__ out_nrm,
+                                              Geom g, int L5, int N, int par, int r0, int nr) {
   using T = typename StoreTraits<S>::T;
-  long idx = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= g.Vh * L5) return;
-  long h = idx / L5;
-  int s = (int)(idx - h * L5);
+  const long idx = (long)blockIdx.x * 256 + threadIdx.x;
+  if (idx >= g.Vh * L5 * nr) return;
+  const long hs = idx / nr, h = hs / L5;
+  const int k = (int)(idx - hs * nr), s = (int)(hs - h * L5);
   int c[4];
   site_coords(g, par, h, c);
-  long lex = lex_index(g, c);
-  double* dst = api + ((long)s * g.V + lex) * 24;
+  const double* src = api.p[k] + ((long)s * g.V + lex_index(g, c)) * 24;
   T a[24];
-  load24<S, T>(in, in_nrm, (h * L5 + s) * N + r, a);
+#pragma unroll
+  for (int i = 0; i < 24; i++) a[i] = (T)__ldg(src + i);
+  store24<S, T>(out, out_nrm, g.Vh * L5 * N, hs * N + r0 + k, a);
+}
+
+// in == null: zeros.
+template <typename S>
+__global__ void __launch_bounds__(256) k_unpack(const S* __restrict__ in, const float* __restrict__ in_nrm,
+                                                Ptrs<double*> api, Geom g, int L5, int N, int par, int r0, int nr) {
+  using T = typename StoreTraits<S>::T;
+  const long idx = (long)blockIdx.x * 256 + threadIdx.x;
+  if (idx >= g.Vh * L5 * nr) return;
+  const long hs = idx / nr, h = hs / L5;
+  const int k = (int)(idx - hs * nr), s = (int)(hs - h * L5);
+  int c[4];
+  site_coords(g, par, h, c);
+  double* dst = api.p[k] + ((long)s * g.V + lex_index(g, c)) * 24;
+  T a[24];
+  if (in != nullptr) {
+    load24<S, T>(in, in_nrm, g.Vh * L5 * N, hs * N + r0 + k, a);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 24; i++) a[i] = 0;
+  }
 #pragma unroll
   for (int i = 0; i < 24; i++) dst[i] = (double)a[i];
 }
@@ -121,16 +96,17 @@ __global__ void k_unpack(const S* __restrict__ in, const float* __restrict__ in_
 template <typename Si, typename So>
 __global__ void k_convert(const Si* __restrict__ in, const float* __restrict__ in_nrm, So* __restrict__ out,
                           float* __restrict__ out_nrm, Tiling tl, long Vh, int L5, int N, const int* __restrict__ mask) {
-  Unit x = unit_of(tl, Vh, L5, N);
+  const Unit x = unit_of(tl, Vh, L5, N);
+  const long pl = Vh * L5 * N;
   if (!x.valid || (mask && !mask[x.r])) return;
   using Ti = typename StoreTraits<Si>::T;
   using To = typename StoreTraits<So>::T;
   Ti a[24];
-  load24<Si, Ti>(in, in_nrm, x.u, a);
+  load24<Si, Ti>(in, in_nrm, pl, x.u, a);
   To b[24];
 #pragma unroll
   for (int i = 0; i < 24; i++) b[i] = (To)a[i];
-  store24<So, To>(out, out_nrm, x.u, b);
+  store24<So, To>(out, out_nrm, pl, x.u, b);
 }
 
 // x += alpha_r p ; rho -= alpha_r q ; |rho|^2 of one unit, explicit roundings.
@@ -155,19 +131,20 @@ __global__ void k_axpy_x_rho(SX* __restrict__ xv, const S* __restrict__ p, const
                              int L5, int N, const int* __restrict__ active, double* __restrict__ partials) {
   using T = typename StoreTraits<S>::T;
   using TX = typename StoreTraits<SX>::T;
-  Unit x = unit_of(tl, Vh, L5, N);
+  const Unit x = unit_of(tl, Vh, L5, N);
+  const long pl = Vh * L5 * N;
   double n2 = 0.0;
   if (x.valid && (!active || active[x.r])) {
     const T a = (T)alpha[x.r];
     T pv[24], qv[24], rv[24];
     TX xv_[24];
-    load24<S, T>(p, p_nrm, x.u, pv);
-    load24<S, T>(q, q_nrm, x.u, qv);
-    load24<S, T>(rho, rho_nrm, x.u, rv);
-    XloLayout<SX>::load(xv, x, tl, xv_);
+    load24<S, T>(p, p_nrm, pl, x.u, pv);
+    load24<S, T>(q, q_nrm, pl, x.u, qv);
+    load24<S, T>(rho, rho_nrm, pl, x.u, rv);
+    load24<SX, SX>(xv, nullptr, pl, x.u, xv_);
     n2 = (double)axpy_unit<TX, T>(a, pv, qv, rv, xv_);
-    XloLayout<SX>::store(xv, x, tl, xv_);
-    store24<S, T>(rho, rho_nrm, x.u, rv);
+    store24<SX, SX>(xv, nullptr, pl, x.u, xv_);
+    store24<S, T>(rho, rho_nrm, pl, x.u, rv);
   }
   block_partial(n2, x, tl, L5, Vh, partials);
 }
@@ -178,15 +155,16 @@ __global__ void k_xpay(const S* __restrict__ r, const float* __restrict__ r_nrm,
                        float* __restrict__ p_nrm, const double* __restrict__ beta, Tiling tl, long Vh, int L5, int N,
                        const int* __restrict__ active) {
   using T = typename StoreTraits<S>::T;
-  Unit x = unit_of(tl, Vh, L5, N);
+  const Unit x = unit_of(tl, Vh, L5, N);
+  const long pl = Vh * L5 * N;
   if (!x.valid || (active && !active[x.r])) return;
   const T b = (T)beta[x.r];
   T rv[24], pv[24];
-  load24<S, T>(r, r_nrm, x.u, rv);
-  load24<S, T>(p, p_nrm, x.u, pv);
+  load24<S, T>(r, r_nrm, pl, x.u, rv);
+  load24<S, T>(p, p_nrm, pl, x.u, pv);
 #pragma unroll
   for (int i = 0; i < 24; i++) pv[i] = rv[i] + b * pv[i];
-  store24<S, T>(p, p_nrm, x.u, pv);
+  store24<S, T>(p, p_nrm, pl, x.u, pv);
 }
 
 // xhi += xlo ; xlo = 0
@@ -194,38 +172,29 @@ template <typename SX>
 __global__ void k_accum_xhi(double* __restrict__ xhi, SX* __restrict__ xlo, Tiling tl, long Vh, int L5, int N,
                             const int* __restrict__ mask) {
   using TX = typename StoreTraits<SX>::T;
-  Unit x = unit_of(tl, Vh, L5, N);
+  const Unit x = unit_of(tl, Vh, L5, N);
+  const long pl = Vh * L5 * N;
   if (!x.valid || (mask && !mask[x.r])) return;
   double h[24];
   TX l[24];
-  load24<double, double>(xhi, nullptr, x.u, h);
-  XloLayout<SX>::load(xlo, x, tl, l);
+  load24<double, double>(xhi, nullptr, pl, x.u, h);
+  load24<SX, SX>(xlo, nullptr, pl, x.u, l);
 #pragma unroll
   for (int i = 0; i < 24; i++) { h[i] += (double)l[i]; l[i] = 0; }
-  store24<double, double>(xhi, nullptr, x.u, h);
-  XloLayout<SX>::store(xlo, x, tl, l);
-}
-
-// x_lo = 0 for the slots in mask (x_lo in the accumulator layout)
-template <typename SX>
-__global__ void k_zero_xlo(SX* __restrict__ xlo, Tiling tl, long Vh, int L5, int N, const int* __restrict__ mask) {
-  Unit x = unit_of(tl, Vh, L5, N);
-  if (!x.valid || !mask[x.r]) return;
-  SX z[24];
-#pragma unroll
-  for (int i = 0; i < 24; i++) z[i] = 0;
-  XloLayout<SX>::store(xlo, x, tl, z);
+  store24<double, double>(xhi, nullptr, pl, x.u, h);
+  store24<SX, SX>(xlo, nullptr, pl, x.u, l);
 }
 
 template <typename S>
 __global__ void k_norm2(const S* __restrict__ v, const float* __restrict__ v_nrm, Tiling tl, long Vh, int L5, int N,
                         const int* __restrict__ mask, double* __restrict__ partials) {
   using T = typename StoreTraits<S>::T;
-  Unit x = unit_of(tl, Vh, L5, N);
+  const Unit x = unit_of(tl, Vh, L5, N);
+  const long pl = Vh * L5 * N;
   double n2 = 0.0;
   if (x.valid && (!mask || mask[x.r])) {
     T a[24];
-    load24<S, T>(v, v_nrm, x.u, a);
+    load24<S, T>(v, v_nrm, pl, x.u, a);
     T n2t = 0;
 #pragma unroll
     for (int i = 0; i < 24; i++) n2t += a[i] * a[i];
@@ -339,20 +308,21 @@ __global__ void k_bop(const S* __restrict__ xv, const float* __restrict__ x_nrm,
                       float* __restrict__ u_nrm, Fifth<typename StoreTraits<S>::T> f, Tiling tl, long Vh, int L5, int N,
                       const int* __restrict__ mask) {
   using T = typename StoreTraits<S>::T;
-  Unit x = unit_of(tl, Vh, L5, N);
+  const Unit x = unit_of(tl, Vh, L5, N);
+  const long pl = Vh * L5 * N;
   if (!x.valid || (mask && !mask[x.r])) return;
   const T m = f.mass[x.r];
   const int s_dn = x.s == 0 ? L5 - 1 : x.s - 1, s_up = x.s == L5 - 1 ? 0 : x.s + 1;
   const T w_dn = x.s == 0 ? -m : T(1), w_up = x.s == L5 - 1 ? -m : T(1);
   T y[24], up[12], lo[12];
-  load24<S, T>(xv, x_nrm, x.u, y);
-  load_part<S, T>(xv, x_nrm, (x.h * L5 + s_dn) * N + x.r, 0, up);
-  load_part<S, T>(xv, x_nrm, (x.h * L5 + s_up) * N + x.r, 1, lo);
+  load24<S, T>(xv, x_nrm, pl, x.u, y);
+  load_part<S, T>(xv, x_nrm, pl, (x.h * L5 + s_dn) * N + x.r, 0, up);
+  load_part<S, T>(xv, x_nrm, pl, (x.h * L5 + s_up) * N + x.r, 1, lo);
 #pragma unroll
   for (int i = 0; i < 12; i++) y[i] = bop_term(f.b5, y[i], f.c5 * w_dn, up[i]);
 #pragma unroll
   for (int i = 0; i < 12; i++) y[12 + i] = bop_term(f.b5, y[12 + i], f.c5 * w_up, lo[i]);
-  store24<S, T>(uv, u_nrm, x.u, y);
+  store24<S, T>(uv, u_nrm, pl, x.u, y);
 }
 
 // p = r + beta_r p, then u = B p (the new p of the neighbouring slices comes from
@@ -365,7 +335,8 @@ __global__ void k_xpay_b(const S* __restrict__ r, const float* __restrict__ r_nr
   using T = typename StoreTraits<S>::T;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sP = reinterpret_cast<T*>(smem_raw);
-  Unit x = unit_of(tl, Vh, L5, N);
+  const Unit x = unit_of(tl, Vh, L5, N);
+  const long pl = Vh * L5 * N;
   const bool act = x.valid && (!active || active[x.r]);
   T pv[24];
 #pragma unroll
@@ -373,11 +344,11 @@ __global__ void k_xpay_b(const S* __restrict__ r, const float* __restrict__ r_nr
   if (act) {
     const T b = (T)beta[x.r];
     T rv[24];
-    load24<S, T>(r, r_nrm, x.u, rv);
-    load24<S, T>(p, p_nrm, x.u, pv);
+    load24<S, T>(r, r_nrm, pl, x.u, rv);
+    load24<S, T>(p, p_nrm, pl, x.u, pv);
 #pragma unroll
     for (int i = 0; i < 24; i++) pv[i] = rv[i] + b * pv[i];
-    store24<S, T>(p, p_nrm, x.u, pv);
+    store24<S, T>(p, p_nrm, pl, x.u, pv);
   }
 #pragma unroll
   for (int i = 0; i < 24; i++) sP[threadIdx.x * 25 + i] = pv[i];
@@ -393,7 +364,7 @@ __global__ void k_xpay_b(const S* __restrict__ r, const float* __restrict__ r_nr
   for (int i = 0; i < 12; i++) y[i] = f.b5 * pv[i] + f.c5 * w_dn * nd[i];
 #pragma unroll
   for (int i = 12; i < 24; i++) y[i] = f.b5 * pv[i] + f.c5 * w_up * nu[i];
-  store24<S, T>(uv, u_nrm, x.u, y);
+  store24<S, T>(uv, u_nrm, pl, x.u, y);
 }
 
 // Zero the units of the slots in mask.
@@ -401,12 +372,13 @@ template <typename S>
 __global__ void k_zero_masked(S* __restrict__ v, float* __restrict__ nrm, Tiling tl, long Vh, int L5, int N,
                               const int* __restrict__ mask) {
   using T = typename StoreTraits<S>::T;
-  Unit x = unit_of(tl, Vh, L5, N);
+  const Unit x = unit_of(tl, Vh, L5, N);
+  const long pl = Vh * L5 * N;
   if (!x.valid || !mask[x.r]) return;
   T z[24];
 #pragma unroll
   for (int i = 0; i < 24; i++) z[i] = 0;
-  store24<S, T>(v, nrm, x.u, z);
+  store24<S, T>(v, nrm, pl, x.u, z);
 }
 
 // Z2 noise source: complex element k of a 4D field ([t][z][y][x][spin][colour],
@@ -432,13 +404,14 @@ __global__ void k_resid_update(const double* __restrict__ bhat, const float* __r
                                float* __restrict__ rho_nrm, Tiling tl, long Vh, int L5, int N,
                                const int* __restrict__ mask, double* __restrict__ partials) {
   using T = typename StoreTraits<S>::T;
-  Unit x = unit_of(tl, Vh, L5, N);
+  const Unit x = unit_of(tl, Vh, L5, N);
+  const long pl = Vh * L5 * N;
   double n2 = 0.0;
   if (x.valid && (!mask || mask[x.r])) {
     double b[24];
     float qv[24];
-    load24<double, double>(bhat, nullptr, x.u, b);
-    load24<float, float>(q, nullptr, x.u, qv);
+    load24<double, double>(bhat, nullptr, pl, x.u, b);
+    load24<float, float>(q, nullptr, pl, x.u, qv);
     T o[24];
 #pragma unroll
     for (int i = 0; i < 24; i++) {
@@ -446,7 +419,7 @@ __global__ void k_resid_update(const double* __restrict__ bhat, const float* __r
       n2 += v * v;
       o[i] = (T)v;
     }
-    store24<S, T>(rho, rho_nrm, x.u, o);
+    store24<S, T>(rho, rho_nrm, pl, x.u, o);
   }
   block_partial(n2, x, tl, L5, Vh, partials);
 }
@@ -457,18 +430,26 @@ __global__ void k_resid_update(const double* __restrict__ bhat, const float* __r
 static inline dim3 tile_grid(const Tiling& t) { return dim3((unsigned)t.ntiles, (unsigned)t.ngroups); }
 
 template <typename S>
-cudaError_t pack_rhs(const double* api, S* out, float* out_nrm, const Geom& g, int L5, int N, int par, int r,
-                     cudaStream_t st) {
-  long n = g.Vh * L5;
-  k_pack<S><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(api, out, out_nrm, g, L5, N, par, r);
+cudaError_t pack_rhs(const double* const* api, S* out, float* out_nrm, const Geom& g, int L5, int N, int par, int r0,
+                     int nr, cudaStream_t st) {
+  for (int b = 0; b < nr; b += kPtrs) {
+    const int m = nr - b < kPtrs ? nr - b : kPtrs;
+    Ptrs<const double*> p;
+    for (int k = 0; k < kPtrs; k++) p.p[k] = k < m ? api[b + k] : nullptr;
+    k_pack<S><<<(unsigned)((g.Vh * L5 * m + 255) / 256), 256, 0, st>>>(p, out, out_nrm, g, L5, N, par, r0 + b, m);
+  }
   return cudaGetLastError();
 }
 
 template <typename S>
-cudaError_t unpack_rhs(const S* in, const float* in_nrm, double* api, const Geom& g, int L5, int N, int par, int r,
-                       cudaStream_t st) {
-  long n = g.Vh * L5;
-  k_unpack<S><<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, in_nrm, api, g, L5, N, par, r);
+cudaError_t unpack_rhs(const S* in, const float* in_nrm, double* const* api, const Geom& g, int L5, int N, int par,
+                       int r0, int nr, cudaStream_t st) {
+  for (int b = 0; b < nr; b += kPtrs) {
+    const int m = nr - b < kPtrs ? nr - b : kPtrs;
+    Ptrs<double*> p;
+    for (int k = 0; k < kPtrs; k++) p.p[k] = k < m ? api[b + k] : nullptr;
+    k_unpack<S><<<(unsigned)((g.Vh * L5 * m + 255) / 256), 256, 0, st>>>(in, in_nrm, p, g, L5, N, par, r0 + b, m);
+  }
   return cudaGetLastError();
 }
 
@@ -500,16 +481,6 @@ cudaError_t accum_xhi(double* xhi, SX* xlo, const Tiling& t, long Vh, int L5, in
                       cudaStream_t st) {
   k_accum_xhi<SX><<<tile_grid(t), t.threads, 0, st>>>(xhi, xlo, t, Vh, L5, N, mask);
   return cudaGetLastError();
-}
-
-template <typename SX>
-cudaError_t zero_xlo(SX* xlo, const Tiling& t, long Vh, int L5, int N, const int* mask, cudaStream_t st) {
-  k_zero_xlo<SX><<<tile_grid(t), t.threads, 0, st>>>(xlo, t, Vh, L5, N, mask);
-  return cudaGetLastError();
-}
-
-long xlo_units(const Tiling& t, long units, bool tile_major) {
-  return tile_major ? t.ntiles * (long)t.ngroups * t.threads : units;
 }
 
 template <typename S>
@@ -596,9 +567,10 @@ Tiling blas_tiling(long Vh, int L5, int N, int max_threads) {
 }
 
 #define MDWF_INST_S(S)                                                                                          \
-  template cudaError_t pack_rhs<S>(const double*, S*, float*, const Geom&, int, int, int, int, cudaStream_t);   \
-  template cudaError_t unpack_rhs<S>(const S*, const float*, double*, const Geom&, int, int, int, int,          \
-                                     cudaStream_t);                                                             \
+  template cudaError_t pack_rhs<S>(const double* const*, S*, float*, const Geom&, int, int, int, int, int,      \
+                                   cudaStream_t);                                                               \
+  template cudaError_t unpack_rhs<S>(const S*, const float*, double* const*, const Geom&, int, int, int, int,   \
+                                     int, cudaStream_t);                                                        \
   template cudaError_t xpay<S>(const S*, const float*, S*, float*, const double*, const Tiling&, long, int, int, \
                                const int*, cudaStream_t);                                                       \
   template cudaError_t norm2_partials<S>(const S*, const float*, const Tiling&, long, int, int, const int*,      \
@@ -647,7 +619,5 @@ MDWF_INST_AXPY(float, __nv_bfloat16)
 
 template cudaError_t accum_xhi<double>(double*, double*, const Tiling&, long, int, int, const int*, cudaStream_t);
 template cudaError_t accum_xhi<float>(double*, float*, const Tiling&, long, int, int, const int*, cudaStream_t);
-template cudaError_t zero_xlo<double>(double*, const Tiling&, long, int, int, const int*, cudaStream_t);
-template cudaError_t zero_xlo<float>(float*, const Tiling&, long, int, int, const int*, cudaStream_t);
 
 }  // namespace mdwf

@@ -23,13 +23,14 @@ enum { FLAG_INNER_DONE = 1, FLAG_UPDATE = 2, FLAG_DONE = 4, FLAG_REREF = 8, FLAG
 enum FinOp { FIN_STORE = 0, FIN_ALPHA = 1, FIN_RHO = 2, FIN_BETA = 3 };
 cudaError_t finalize_cg(const double* partials, long nsites, int N, const Scal& c, FinOp op, cudaStream_t st);
 
-// API layout (one RHS, [s][t][z][y][x][spin][colour][re,im], FP64, device) <-> slot r of a parity field.
+// API layout (one field per RHS, [s][t][z][y][x][spin][colour][re,im], FP64, device) <-> slots r0 .. r0 + nr - 1
+// of a parity field; api: nr device pointers (host array).  unpack_rhs with in == null writes zeros.
 template <typename S>
-cudaError_t pack_rhs(const double* api, S* out, float* out_nrm, const Geom& g, int L5, int N, int par, int r,
-                     cudaStream_t st);
+cudaError_t pack_rhs(const double* const* api, S* out, float* out_nrm, const Geom& g, int L5, int N, int par, int r0,
+                     int nr, cudaStream_t st);
 template <typename S>
-cudaError_t unpack_rhs(const S* in, const float* in_nrm, double* api, const Geom& g, int L5, int N, int par, int r,
-                       cudaStream_t st);
+cudaError_t unpack_rhs(const S* in, const float* in_nrm, double* const* api, const Geom& g, int L5, int N, int par,
+                       int r0, int nr, cudaStream_t st);
 
 template <typename Si, typename So>
 cudaError_t convert(const Si* in, const float* in_nrm, So* out, float* out_nrm, const Tiling& t, long Vh, int L5,
@@ -47,15 +48,6 @@ cudaError_t xpay(const S* r, const float* r_nrm, S* p, float* p_nrm, const doubl
 template <typename SX>
 cudaError_t accum_xhi(double* xhi, SX* xlo, const Tiling& t, long Vh, int L5, int N, const int* mask,
                       cudaStream_t st);
-// x_lo = 0 for the slots in mask.
-template <typename SX>
-cudaError_t zero_xlo(SX* xlo, const Tiling& t, long Vh, int L5, int N, const int* mask, cudaStream_t st);
-// Units a solution accumulator x_lo holds for the tiling t: an FP32 accumulator
-// is stored tile-major (see blas.cu) and spans every thread of the grid; an
-// FP64 one is unit-major, `units` long.  axpy_x_rho, accum_xhi and zero_xlo read
-// and write x_lo in that layout, and must be given the same tiling.
-long xlo_units(const Tiling& t, long units, bool tile_major);
-
 template <typename S>
 cudaError_t norm2_partials(const S* v, const float* v_nrm, const Tiling& t, long Vh, int L5, int N, const int* mask,
                            double* partials, cudaStream_t st);

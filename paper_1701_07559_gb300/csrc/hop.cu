@@ -107,7 +107,7 @@ __device__ __forceinline__ void hop_dir(const HopArgs<S, T>& a, const int c[4], 
     T phase = (MU == 3 && a.antiperiodic && c[3] == a.g.L[3] - 1) ? T(-1) : T(1);
     long hn = lex_index(a.g, n) >> 1;
     T psi[24], hh[12], chi[12], l[18];
-    load24<S, T>(a.in, a.in_nrm, (hn * a.L5 + s) * a.N + r, psi);
+    load24<S, T>(a.in, a.in_nrm, plane_of(a), (hn * a.L5 + s) * a.N + r, psi);
     load_link<T>(a.U, ((long)par * a.g.Vh + h) * 4 + MU, l);
     const T sg = a.dagger ? T(1) : T(-1);
     project<MU, T>(psi, sg, hh);
@@ -124,7 +124,7 @@ __device__ __forceinline__ void hop_dir(const HopArgs<S, T>& a, const int c[4], 
     T phase = (MU == 3 && a.antiperiodic && c[3] == 0) ? T(-1) : T(1);
     long hn = lex_index(a.g, n) >> 1;
     T psi[24], hh[12], chi[12], l[18];
-    load24<S, T>(a.in, a.in_nrm, (hn * a.L5 + s) * a.N + r, psi);
+    load24<S, T>(a.in, a.in_nrm, plane_of(a), (hn * a.L5 + s) * a.N + r, psi);
     load_link<T>(a.U, ((long)(1 - par) * a.g.Vh + hn) * 4 + MU, l);
     const T sg = a.dagger ? T(-1) : T(1);
     project<MU, T>(psi, sg, hh);
@@ -166,7 +166,7 @@ __global__ void hop_kernel(HopArgs<S, T> a, Tiling tl) {
       hop_dir<2, S, T>(a, c, h, s, r, acc);
       hop_dir<3, S, T>(a, c, h, s, r, acc);
     } else {
-      load24<S, T>(a.in, a.in_nrm, u, acc);
+      load24<S, T>(a.in, a.in_nrm, plane_of(a), u, acc);
     }
   }
 #pragma unroll
@@ -176,7 +176,7 @@ __global__ void hop_kernel(HopArgs<S, T> a, Tiling tl) {
     T tmp[24];
 #pragma unroll
     for (int i = 0; i < 24; i++) tmp[i] = 0;
-    if (act) load24<S, T>(a.same, a.same_nrm, u, tmp);
+    if (act) load24<S, T>(a.same, a.same_nrm, plane_of(a), u, tmp);
 #pragma unroll
     for (int i = 0; i < 24; i++) sG[tid * kPad + i] = tmp[i];
   }
@@ -186,7 +186,7 @@ __global__ void hop_kernel(HopArgs<S, T> a, Tiling tl) {
   if (act) {
     T o[24];
     if (a.add != nullptr) {
-      load24<S, T>(a.add, a.add_nrm, u, o);
+      load24<S, T>(a.add, a.add_nrm, plane_of(a), u, o);
     } else {
 #pragma unroll
       for (int i = 0; i < 24; i++) o[i] = 0;
@@ -222,7 +222,7 @@ __global__ void hop_kernel(HopArgs<S, T> a, Tiling tl) {
         for (int i = 12; i < 24; i++) o[i] += gl * src[i];
       }
     }
-    store24<S, T>(a.out, a.out_nrm, u, o);
+    store24<S, T>(a.out, a.out_nrm, plane_of(a), u, o);
     if (a.partials != nullptr) {
 #pragma unroll
       for (int i = 0; i < 24; i++) n2 += (double)o[i] * (double)o[i];
@@ -280,8 +280,5 @@ int hop_max_threads() {
   template size_t hop_smem_bytes<S, T>(const Tiling&, bool);
 
 MDWF_INSTANTIATE_HOP(double, double)
-MDWF_INSTANTIATE_HOP(float, float)
-MDWF_INSTANTIATE_HOP(__half, float)
-MDWF_INSTANTIATE_HOP(__nv_bfloat16, float)
 
 }  // namespace mdwf

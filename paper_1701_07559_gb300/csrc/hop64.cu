@@ -35,19 +35,37 @@ namespace mdwf {
 
 namespace {
 
-// Unit index (in 24-double units) of slice s, slot r at a site, and site enumeration.
+// Element index of component cp of slice s, slot r at a site.
 template <bool API>
 struct Map;
 template <>
-struct Map<false> {      // [h][s][r]
-  static __device__ __forceinline__ long unit(const FastArgs<double, double>& a, long lex, int s, int r) {
-    return ((lex >> 1) * a.L5 + s) * a.N + r;
+struct Map<false> {      // parity field: planes of 16-byte words, unit (h L5 + s) N + r
+  static __device__ __forceinline__ long at(const FastArgs<double, double>& a, long lex, int s, int r, int cp) {
+    return 2 * ((cp >> 1) * plane_of(a) + ((lex >> 1) * a.L5 + s) * a.N + r) + (cp & 1);
+  }
+  // the six reals of a spin
+  static __device__ __forceinline__ void load6(const FastArgs<double, double>& a, const double* __restrict__ f, long lex,
+                                               int s, int r, int spin, double* v) {
+    const long pl = plane_of(a);
+    const double2* p = reinterpret_cast<const double2*>(f) + 3 * spin * pl + ((lex >> 1) * a.L5 + s) * a.N + r;
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      const double2 t = __ldg(p + i * pl);
+      v[2 * i] = t.x;
+      v[2 * i + 1] = t.y;
+    }
   }
 };
 template <>
-struct Map<true> {       // [s][lex], one slot
-  static __device__ __forceinline__ long unit(const FastArgs<double, double>& a, long lex, int s, int) {
-    return (long)s * a.g.V + lex;
+struct Map<true> {       // the caller's layout [s][lex][24], one slot; aligned to a double
+  static __device__ __forceinline__ long at(const FastArgs<double, double>& a, long lex, int s, int, int cp) {
+    return ((long)s * a.g.V + lex) * 24 + cp;
+  }
+  static __device__ __forceinline__ void load6(const FastArgs<double, double>& a, const double* __restrict__ f, long lex,
+                                               int s, int r, int spin, double* v) {
+    const double* p = f + at(a, lex, s, r, 6 * spin);
+#pragma unroll
+    for (int i = 0; i < 6; i++) v[i] = __ldg(p + i);
   }
 };
 
@@ -79,22 +97,6 @@ __device__ __forceinline__ void colour_mul(const double* __restrict__ l, const d
     }
     o[2 * a] = re;
     o[2 * a + 1] = im;
-  }
-}
-
-// Six doubles of a spin (8-byte aligned in the caller's arrays, 16 in the parity fields).
-template <bool API>
-__device__ __forceinline__ void load6(const double* __restrict__ p, double* v) {
-  if (API) {
-#pragma unroll
-    for (int i = 0; i < 6; i++) v[i] = __ldg(p + i);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 3; i++) {
-      const double2 t = __ldg(reinterpret_cast<const double2*>(p) + i);
-      v[2 * i] = t.x;
-      v[2 * i + 1] = t.y;
-    }
   }
 }
 
@@ -215,10 +217,9 @@ __global__ void __launch_bounds__(256) hop64_kernel(FastArgs<double, double> a, 
       const bool flf = mu == 3 && ef && a.antiperiodic, flb = mu == 3 && eb && a.antiperiodic;
       // projected neighbours
       auto project = [&](long n, double sg, double* v) {
-        const double* ps = a.in + Map<API>::unit(a, n, s, r) * 24;
         double e[6];
-        load6<API>(ps + 6 * j, v);
-        load6<API>(ps + 6 * spin_p, e);
+        Map<API>::load6(a, a.in, n, s, r, j, v);
+        Map<API>::load6(a, a.in, n, s, r, spin_p, e);
         const double f = sg * sig, f0 = sw ? -f : f;
 #pragma unroll
         for (int b = 0; b < 3; b++) {
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(256) hop64_kernel(FastArgs<double, double> a, 
       if (kSameFirst || a.kappa != 1.0)
         for (int s = 0; s < L5; s++) {
           const double hv = a.in != nullptr ? col[s * st] : 0.0;
-          col[s * st] = kSameFirst ? __fma_rn(a.kappa, hv, a.same[Map<API>::unit(a, lex, s, r) * 24 + cp]) : a.kappa * hv;
+          col[s * st] = kSameFirst ? __fma_rn(a.kappa, hv, a.same[Map<API>::at(a, lex, s, r, cp)]) : a.kappa * hv;
         }
       const bool upper = cp < 12, down = (EPI == E_AINVD_BD || EPI == E_AINVD_SAME) ? !upper : upper;
       column64<EPI>(down ? col : col + (L5 - 1) * st, down ? st : -st, L5, a.f, a.f.mass[r]);
@@ -335,14 +336,14 @@ __global__ void __launch_bounds__(256) hop64_kernel(FastArgs<double, double> a, 
       const int sn = from_up ? sp : sd;
       double gw = gb;
       if (from_up ? s == L5 - 1 : s == 0) gw = gb * -a.f.mass[r];
-      const double y = a.same[Map<API>::unit(a, lex, s, r) * 24 + cp];
-      const double yn = a.same[Map<API>::unit(a, lex, sn, r) * 24 + cp];
+      const double y = a.same[Map<API>::at(a, lex, s, r, cp)];
+      const double yn = a.same[Map<API>::at(a, lex, sn, r, cp)];
       o = __fma_rn(ga, y, __fma_rn(gw, yn, o));
     }
     if ((EPI == E_SAME_AINV || EPI == E_SAME_BD) && a.g_same != 0.0)
-      o = __fma_rn(a.g_same, a.same[Map<API>::unit(a, lex, s, r) * 24 + cp], o);
-    if (kAdd && a.add != nullptr) o += a.add[Map<API>::unit(a, lex, s, r) * 24 + cp];
-    a.out[Map<API>::unit(a, lex, s, r) * 24 + cp] = o;
+      o = __fma_rn(a.g_same, a.same[Map<API>::at(a, lex, s, r, cp)], o);
+    if (kAdd && a.add != nullptr) o += a.add[Map<API>::at(a, lex, s, r, cp)];
+    a.out[Map<API>::at(a, lex, s, r, cp)] = o;
     // the B^+ forms still read the tile of other units: their norms are formed from the stored output
     if (norm && !kBdag) *t = o;
   }
@@ -358,9 +359,11 @@ __global__ void __launch_bounds__(256) hop64_kernel(FastArgs<double, double> a, 
         const int k = ul / na, r = slots[1 + ul - k * na], site_l = k / L5, s = k - site_l * L5;
         long lex;
         site_of(site_l, &lex);
-        const double* o = a.out + Map<API>::unit(a, lex, s, r) * 24 + 3 * (lane & 7);
 #pragma unroll
-        for (int b = 0; b < 3; b++) n2 = __fma_rn(o[b], o[b], n2);
+        for (int b = 0; b < 3; b++) {
+          const double o = a.out[Map<API>::at(a, lex, s, r, 3 * (lane & 7) + b)];
+          n2 = __fma_rn(o, o, n2);
+        }
       } else {
 #pragma unroll
         for (int b = 0; b < 3; b++) n2 = __fma_rn(t[b], t[b], n2);

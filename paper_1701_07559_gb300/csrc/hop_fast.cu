@@ -99,38 +99,37 @@ __device__ __forceinline__ void project(const T* p, T sg, T* h) {
 // and is applied in the reconstruction.
 template <int MU, typename S, typename T>
 struct Proj {
-  static __device__ __forceinline__ T global(const S* __restrict__ v, const float* __restrict__ nrm, long u, T sg,
-                                             T* h) {
+  static __device__ __forceinline__ T global(const S* __restrict__ v, const float* __restrict__ nrm, long pl, long u,
+                                             T sg, T* h) {
     T psi[24];
-    load24<S, T>(v, nrm, u, psi);
+    load24<S, T>(v, nrm, pl, u, psi);
     project<MU, T>(psi, sg, h);
     return T(1);
   }
-  static __device__ __forceinline__ T shared(const S* sp, float nrm, T sg, T* h) {
+  static __device__ __forceinline__ T shared(const uint4* sp, int pl, float nrm, T sg, T* h) {
     T psi[24];
-    load24_smem<S, T>(sp, psi);
+    load24_smem<S, T>(sp, pl, psi);
     project<MU, T>(psi, sg, h);
     return StoreTraits<S>::kNorm ? (T)nrm : T(1);
   }
 };
 template <int MU>
 struct Proj<MU, __half, float> {
-  static __device__ __forceinline__ float global(const __half* __restrict__ v, const float* __restrict__ nrm, long u,
-                                                 float sg, float* h) {
-    const uint4* p = reinterpret_cast<const uint4*>(v + 24 * u);
+  static __device__ __forceinline__ float global(const __half* __restrict__ v, const float* __restrict__ nrm, long pl,
+                                                 long u, float sg, float* h) {
+    const uint4* p = reinterpret_cast<const uint4*>(v) + u;
     uint4 q[3];
     q[0] = __ldg(p);
-    q[1] = __ldg(p + 1);
-    q[2] = __ldg(p + 2);
+    q[1] = __ldg(p + pl);
+    q[2] = __ldg(p + 2 * pl);
     project_half<MU>(q, sg, h);
     return __ldg(nrm + u);
   }
-  static __device__ __forceinline__ float shared(const __half* sp, float nrm, float sg, float* h) {
-    const uint4* p = reinterpret_cast<const uint4*>(sp);
+  static __device__ __forceinline__ float shared(const uint4* p, int pl, float nrm, float sg, float* h) {
     uint4 q[3];
     q[0] = p[0];
-    q[1] = p[1];
-    q[2] = p[2];
+    q[1] = p[pl];
+    q[2] = p[2 * pl];
     project_half<MU>(q, sg, h);
     return nrm;
   }
@@ -170,12 +169,12 @@ __device__ __forceinline__ void reconstruct(const T* chi, T f, T fs, T* acc) {
 // from global memory (sp == nullptr) or from the shared staging buffer sp.
 template <int MU, bool FWD, typename S, typename T>
 __device__ __forceinline__ void hop_term_at(const FastArgs<S, T>& a, int hn, bool bflip, long h, int s, int r,
-                                            const S* sp, float snrm, T* acc) {
+                                            const uint4* sp, float snrm, T* acc) {
   const T sg = (a.dagger ? T(1) : T(-1)) * (FWD ? T(1) : T(-1));
   T hh[12], chi[12], l[18];
   T f;
-  if (sp == nullptr) f = Proj<MU, S, T>::global(a.in, a.in_nrm, ((long)hn * a.L5 + s) * a.N + r, sg, hh);
-  else f = Proj<MU, S, T>::shared(sp, snrm, sg, hh);
+  if (sp == nullptr) f = Proj<MU, S, T>::global(a.in, a.in_nrm, plane_of(a), ((long)hn * a.L5 + s) * a.N + r, sg, hh);
+  else f = Proj<MU, S, T>::shared(sp, a.L5 * a.N, snrm, sg, hh);
   if (bflip) f = -f;
   if (FWD) {
     load_link<T>(a.U, ((long)a.out_par * a.g.Vh + h) * 4 + MU, l);
@@ -190,7 +189,7 @@ __device__ __forceinline__ void hop_term_at(const FastArgs<S, T>& a, int hn, boo
 }
 
 template <int MU, bool FWD, typename S, typename T>
-__device__ __forceinline__ void hop_term(const FastArgs<S, T>& a, const Site& x, long h, int s, int r, const S* sp,
+__device__ __forceinline__ void hop_term(const FastArgs<S, T>& a, const Site& x, long h, int s, int r, const uint4* sp,
                                          float snrm, T* acc) {
   const bool bflip = MU == 3 && a.antiperiodic && (FWD ? x.c[3] == a.g.L[3] - 1 : x.c[3] == 0);
   hop_term_at<MU, FWD, S, T>(a, nbr_half<MU, FWD>(a.g, x), bflip, h, s, r, sp, snrm, acc);
@@ -204,15 +203,15 @@ template <typename S, typename T>
 __device__ __forceinline__ void apply_A(const FastArgs<S, T>& a, long h, int s, int r, bool dag, T m, T* o) {
   const int L5 = a.L5;
   T y[24], up[12], lo[12];
-  load24<S, T>(a.same, a.same_nrm, (h * L5 + s) * a.N + r, y);
+  load24<S, T>(a.same, a.same_nrm, plane_of(a), (h * L5 + s) * a.N + r, y);
   const int s_dn = s == 0 ? L5 - 1 : s - 1;
   const int s_up = s == L5 - 1 ? 0 : s + 1;
   const T w_dn = s == 0 ? -m : T(1);
   const T w_up = s == L5 - 1 ? -m : T(1);
   const int su = dag ? s_up : s_dn, sl = dag ? s_dn : s_up;
   const T wu = dag ? w_up : w_dn, wl = dag ? w_dn : w_up;
-  load_part<S, T>(a.same, a.same_nrm, (h * L5 + su) * a.N + r, 0, up);
-  load_part<S, T>(a.same, a.same_nrm, (h * L5 + sl) * a.N + r, 1, lo);
+  load_part<S, T>(a.same, a.same_nrm, plane_of(a), (h * L5 + su) * a.N + r, 0, up);
+  load_part<S, T>(a.same, a.same_nrm, plane_of(a), (h * L5 + sl) * a.N + r, 1, lo);
   const T al = a.f.alpha, bu = a.f.beta * wu, bl = a.f.beta * wl;
 #pragma unroll
   for (int i = 0; i < 12; i++) o[i] = al * y[i] + bu * up[i];
@@ -378,7 +377,7 @@ __device__ __forceinline__ void epilogue(const FastArgs<S, T>& a, const Tiling& 
       for (int i = 0; i < 24; i++) v[i] = a.kappa * acc[i];
       if (kSameFirst && t.act) {
         T y[24];
-        load24<S, T>(a.same, a.same_nrm, t.u, y);
+        load24<S, T>(a.same, a.same_nrm, plane_of(a), t.u, y);
 #pragma unroll
         for (int i = 0; i < 24; i++) v[i] += y[i];
       }
@@ -388,7 +387,7 @@ __device__ __forceinline__ void epilogue(const FastArgs<S, T>& a, const Tiling& 
     } else if (kSameFirst) {
       if (t.act) {
         T y[24];
-        load24<S, T>(a.same, a.same_nrm, t.u, y);
+        load24<S, T>(a.same, a.same_nrm, plane_of(a), t.u, y);
 #pragma unroll
         for (int i = 0; i < 24; i++) sA[t.tid * kPadF + i] += y[i];
       }
@@ -465,18 +464,18 @@ __device__ __forceinline__ void epilogue(const FastArgs<S, T>& a, const Tiling& 
     }
     if ((EPI == E_SAME_AINV || EPI == E_SAME_BD) && a.g_same != T(0)) {
       T y[24];
-      load24<S, T>(a.same, a.same_nrm, t.u, y);
+      load24<S, T>(a.same, a.same_nrm, plane_of(a), t.u, y);
 #pragma unroll
       for (int i = 0; i < 24; i++) o[i] += a.g_same * y[i];
     }
     if ((EPI == E_RAW || EPI == E_A_SAME || EPI == E_AD_SAME_BD || EPI == E_SAME_AINV || EPI == E_SAME_BD) &&
         a.add != nullptr) {
       T y[24];
-      load24<S, T>(a.add, a.add_nrm, t.u, y);
+      load24<S, T>(a.add, a.add_nrm, plane_of(a), t.u, y);
 #pragma unroll
       for (int i = 0; i < 24; i++) o[i] += y[i];
     }
-    store24<S, T>(a.out, a.out_nrm, t.u, o);
+    store24<S, T>(a.out, a.out_nrm, plane_of(a), t.u, o);
     if (a.partials != nullptr) {
 #pragma unroll
       for (int i = 0; i < 24; i++) n2 += o[i] * o[i];
@@ -586,13 +585,13 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, unsigned parity
 
 template <int D, typename S, typename T>
 __device__ __forceinline__ bool staged_term(const FastArgs<S, T>& a, const Tiling& tl, const StageInfo& si,
-                                            const Thr& t, const Site& x, uint64_t* bars, const S* buf,
+                                            const Thr& t, const Site& x, uint64_t* bars, const uint4* buf,
                                             const float* nbuf, bool ok, T* acc) {
   if (ok) ok = mbar_wait_bounded(&bars[D], 0, si.budget);
   if (ok && t.act) {
     const int upb = a.L5 * a.N;
     const int lu = t.s * a.N + t.r;
-    const S* sp = buf + ((size_t)(D * tl.nsb + t.site_l) * upb + lu) * 24;
+    const uint4* sp = buf + (size_t)(D * tl.nsb + t.site_l) * upb * kWords<S> + lu;
     float nrm = 1.0f;
     if (StoreTraits<S>::kNorm) {
       if (si.nrm_bytes) nrm = nbuf[(size_t)(D * tl.nsb + t.site_l) * upb + lu];
@@ -607,7 +606,7 @@ template <typename S, typename T, int EPI>
 __global__ void hop_staged_kernel(FastArgs<S, T> a, Tiling tl, StageInfo si) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw);
-  S* buf = reinterpret_cast<S*>(smem_raw + 128);
+  uint4* buf = reinterpret_cast<uint4*>(smem_raw + 128);
   float* nbuf = reinterpret_cast<float*>(smem_raw + 128 + si.spin_bytes);
   T* sA = reinterpret_cast<T*>(smem_raw + 128 + si.spin_bytes + si.nrm_bytes);
   const Thr t = thread_of(a, tl);
@@ -632,7 +631,9 @@ __global__ void hop_staged_kernel(FastArgs<S, T> a, Tiling tl, StageInfo si) {
       const int d = k / nsites, j = k - d * nsites;
       const Site xj = make_site(a.g, a.out_par, h0 + j);
       const long hn = nbr_half_any(a.g, xj, d);
-      bulk_g2s(buf + ((size_t)(d * tl.nsb + j) * upb) * 24, a.in + (size_t)hn * upb * 24, chunk, &bars[d]);
+      for (int w = 0; w < kWords<S>; w++)
+        bulk_g2s(buf + ((size_t)(d * tl.nsb + j) * kWords<S> + w) * upb,
+                 reinterpret_cast<const uint4*>(a.in) + w * plane_of(a) + (size_t)hn * upb, 16u * (unsigned)upb, &bars[d]);
       if (nchunk) bulk_g2s(nbuf + (size_t)(d * tl.nsb + j) * upb, a.in_nrm + (size_t)hn * upb, nchunk, &bars[d]);
     }
   }
@@ -880,7 +881,7 @@ __global__ void hop_mma_kernel(FastArgs<__half, float> a, Tiling tl, const uint3
     for (int d = 0; d < 8; d++) {
       const uint32_t un = (uint32_t)nb[d] * upm + uo;
       if (live) {
-        q[d] = __ldg(in4 + (size_t)un * 3u + c);
+        q[d] = __ldg(in4 + c * plane_of(a) + un);
         sc[d] = __ldg(a.in_nrm + un);
       } else {
         q[d] = make_uint4(0u, 0u, 0u, 0u);
@@ -998,7 +999,8 @@ __global__ void hop_mma_bulk_kernel(FastArgs<__half, float> a, Tiling tl, const 
         const uint32_t un0 = (uint32_t)tb.nb[8 * j + d] * upm + (uint32_t)u0;
         unsigned char* dst = wbuf + (size_t)bi * kMmaBuf;
         if (kind == 0) {
-          bulk_g2s(dst + d * 384, a.in + (size_t)un0 * 24u, 384u, &wb[bi]);
+          for (int w = 0; w < 3; w++)
+            bulk_g2s(dst + d * 384 + w * 128, reinterpret_cast<const uint4*>(a.in) + w * plane_of(a) + un0, 128u, &wb[bi]);
         } else if (kind == 1) {
           bulk_g2s(dst + 8 * 384 + d * 32, a.in_nrm + un0, 32u, &wb[bi]);
         } else {
@@ -1045,7 +1047,7 @@ __global__ void hop_mma_bulk_kernel(FastArgs<__half, float> a, Tiling tl, const 
       uint32_t b[8];
 #pragma unroll
       for (int d = 0; d < 8; d++) {
-        q[d] = live ? qs[d * 24 + g * 3 + c] : make_uint4(0u, 0u, 0u, 0u);
+        q[d] = live ? qs[d * 24 + c * 8 + g] : make_uint4(0u, 0u, 0u, 0u);
         sc[d] = live ? scs[d * 8 + g] : 0.f;
         b[d] = fs[d * 32 + lane];
       }
@@ -1128,10 +1130,10 @@ __device__ __forceinline__ void tpu_term(const FastArgs<__half, float>& a, const
   uint4 q[3] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
   float sc = 0.f;
   if (act) {
-    const uint4* p = reinterpret_cast<const uint4*>(a.in) + un * 3;
+    const uint4* p = reinterpret_cast<const uint4*>(a.in) + un;
     q[0] = __ldg(p);
-    q[1] = __ldg(p + 1);
-    q[2] = __ldg(p + 2);
+    q[1] = __ldg(p + plane_of(a));
+    q[2] = __ldg(p + 2 * plane_of(a));
     sc = __ldg(a.in_nrm + un);
   }
   const bool neg_sg = FWD ? !dag : dag;
@@ -1409,7 +1411,7 @@ __global__ void k_dd_pack(const double* __restrict__ in, Geom g, int par, int L5
   if (!first && !last) return;
   const long lex3 = x.lex - (long)x.c[3] * x.stride[3];
   double psi[24], hh[12];
-  load24<double, double>(in, nullptr, u, psi);
+  load24<double, double>(in, nullptr, g.Vh * L5 * N, u, psi);
   const double dg = dagger ? 1.0 : -1.0;
   if (first) {        // the previous sub-domain's forward term: sg = dg
     project<3, double>(psi, dg, hh);

@@ -70,11 +70,11 @@ __device__ __forceinline__ void project2(const float2* p, float sg, float2* h) {
 // factor of each projected spinor (the fp16 storage scale; 1 otherwise).
 template <int MU, typename S>
 struct PairProj {
-  static __device__ __forceinline__ void run(const S* __restrict__ v, const float* __restrict__ nrm, long uA, long uB,
+  static __device__ __forceinline__ void run(const S* __restrict__ v, const float* __restrict__ nrm, long pl, long uA, long uB,
                                              float sg, float2* h, float2& f) {
     float pa[24], pb[24];
-    load24<S, float>(v, nrm, uA, pa);
-    load24<S, float>(v, nrm, uB, pb);
+    load24<S, float>(v, nrm, pl, uA, pa);
+    load24<S, float>(v, nrm, pl, uB, pb);
     float2 p[24];
 #pragma unroll
     for (int i = 0; i < 24; i++) p[i] = make_float2(pa[i], pb[i]);
@@ -84,13 +84,13 @@ struct PairProj {
 };
 template <int MU>
 struct PairProj<MU, __half> {
-  static __device__ __forceinline__ void run(const __half* __restrict__ v, const float* __restrict__ nrm, long uA,
+  static __device__ __forceinline__ void run(const __half* __restrict__ v, const float* __restrict__ nrm, long pl, long uA,
                                              long uB, float sg, float2* h, float2& f) {
-    const uint4* pa = reinterpret_cast<const uint4*>(v + 24 * uA);
-    const uint4* pb = reinterpret_cast<const uint4*>(v + 24 * uB);
+    const uint4* pa = reinterpret_cast<const uint4*>(v) + uA;
+    const uint4* pb = reinterpret_cast<const uint4*>(v) + uB;
     uint4 qa[3], qb[3];
-    qa[0] = __ldg(pa); qa[1] = __ldg(pa + 1); qa[2] = __ldg(pa + 2);
-    qb[0] = __ldg(pb); qb[1] = __ldg(pb + 1); qb[2] = __ldg(pb + 2);
+    qa[0] = __ldg(pa); qa[1] = __ldg(pa + pl); qa[2] = __ldg(pa + 2 * pl);
+    qb[0] = __ldg(pb); qb[1] = __ldg(pb + pl); qb[2] = __ldg(pb + 2 * pl);
     float ha[12], hb[12];
     project_half<MU>(qa, sg, ha);
     project_half<MU>(qb, sg, hb);
@@ -204,7 +204,7 @@ __device__ __forceinline__ void pair_term(const FastArgs<S, float>& a, const Sit
   const long uA = ((long)hn * a.L5 + t.s0) * a.N + t.r;
   const long uB = t.two ? uA + a.N : uA;
   float2 hh[12], f;
-  PairProj<MU, S>::run(a.in, a.in_nrm, uA, uB, sg, hh, f);
+  PairProj<MU, S>::run(a.in, a.in_nrm, plane_of(a), uA, uB, sg, hh, f);
   if (bflip) f = neg2(f);
   const float2 fs = mul2(f, f2(sg));
   float l[18];
@@ -341,10 +341,10 @@ __device__ __forceinline__ void col_pairs(float* tile, const PThr& t, int L5, co
 }
 
 template <typename S>
-__device__ __forceinline__ void load_pair24(const S* v, const float* nrm, const PThr& t, int N, float2* y) {
+__device__ __forceinline__ void load_pair24(const S* v, const float* nrm, long pl, const PThr& t, int N, float2* y) {
   float ya[24], yb[24];
-  load24<S, float>(v, nrm, t.u0, ya);
-  if (t.two) load24<S, float>(v, nrm, t.u0 + N, yb);
+  load24<S, float>(v, nrm, pl, t.u0, ya);
+  if (t.two) load24<S, float>(v, nrm, pl, t.u0 + N, yb);
 #pragma unroll
   for (int i = 0; i < 24; i++) y[i] = make_float2(ya[i], t.two ? yb[i] : 0.f);
 }
@@ -372,8 +372,8 @@ __device__ __forceinline__ void apply_A_pair(const FastArgs<S, float>& a, const 
       const int sn = from_up ? s_up : s_dn;
       const float bw = __fmul_rn(a.f.beta, from_up ? w_up : w_dn);
       float y[12], yn[12];
-      load_part<S, float>(a.same, a.same_nrm, (t.h * L5 + s) * a.N + t.r, part, y);
-      load_part<S, float>(a.same, a.same_nrm, (t.h * L5 + sn) * a.N + t.r, part, yn);
+      load_part<S, float>(a.same, a.same_nrm, plane_of(a), (t.h * L5 + s) * a.N + t.r, part, y);
+      load_part<S, float>(a.same, a.same_nrm, plane_of(a), (t.h * L5 + sn) * a.N + t.r, part, yn);
 #pragma unroll
       for (int i = 0; i < 12; i++) {
         const float ay = __fmaf_rn(bw, yn[i], __fmul_rn(al, y[i]));
@@ -386,17 +386,17 @@ __device__ __forceinline__ void apply_A_pair(const FastArgs<S, float>& a, const 
 
 // Store both units (the second only if it exists).
 template <typename S>
-__device__ __forceinline__ void store_pair24(S* v, float* nrm, const PThr& t, int N, const float2* o) {
+__device__ __forceinline__ void store_pair24(S* v, float* nrm, long pl, const PThr& t, int N, const float2* o) {
   float oa[24], ob[24];
 #pragma unroll
   for (int i = 0; i < 24; i++) { oa[i] = o[i].x; ob[i] = o[i].y; }
-  store24<S, float>(v, nrm, t.u0, oa);
-  if (t.two) store24<S, float>(v, nrm, t.u0 + N, ob);
+  store24<S, float>(v, nrm, pl, t.u0, oa);
+  if (t.two) store24<S, float>(v, nrm, pl, t.u0 + N, ob);
 }
 // fp16: the same values as store24 (the scale is a power of two, so the scaling
 // is exact whichever way it is multiplied), with packed multiplies.
 template <>
-__device__ __forceinline__ void store_pair24<__half>(__half* v, float* nrm, const PThr& t, int N, const float2* o) {
+__device__ __forceinline__ void store_pair24<__half>(__half* v, float* nrm, long pl, const PThr& t, int N, const float2* o) {
   float ma = 0.f, mb = 0.f;
 #pragma unroll
   for (int i = 0; i < 24; i++) { ma = fmaxf(ma, fabsf(o[i].x)); mb = fmaxf(mb, fabsf(o[i].y)); }
@@ -418,13 +418,13 @@ __device__ __forceinline__ void store_pair24<__half>(__half* v, float* nrm, cons
       hb[k] = __floats2half2_rn(q[6 * k + 2 * c].y, q[6 * k + 2 * c + 1].y);
     }
   }
-  uint4* pa = reinterpret_cast<uint4*>(v + 24 * t.u0);
+  uint4* pa = reinterpret_cast<uint4*>(v) + t.u0;
   nrm[t.u0] = sa;
-  pa[0] = wa[0]; pa[1] = wa[1]; pa[2] = wa[2];
+  pa[0] = wa[0]; pa[pl] = wa[1]; pa[2 * pl] = wa[2];
   if (t.two) {
-    uint4* pb = reinterpret_cast<uint4*>(v + 24 * (t.u0 + N));
+    uint4* pb = pa + N;
     nrm[t.u0 + N] = sb;
-    pb[0] = wb[0]; pb[1] = wb[1]; pb[2] = wb[2];
+    pb[0] = wb[0]; pb[pl] = wb[1]; pb[2 * pl] = wb[2];
   }
 }
 
@@ -443,7 +443,7 @@ __device__ __forceinline__ void pair_epilogue(const FastArgs<S, float>& a, const
     float2 v[24];
     if (kSameFirst && t.act) {
       float2 y[24];
-      load_pair24<S>(a.same, a.same_nrm, t, a.N, y);
+      load_pair24<S>(a.same, a.same_nrm, plane_of(a), t, a.N, y);
 #pragma unroll
       for (int i = 0; i < 24; i++) v[i] = fma2(kap, acc[i], y[i]);
     } else {
@@ -500,7 +500,7 @@ __device__ __forceinline__ void pair_epilogue(const FastArgs<S, float>& a, const
     if ((EPI == E_A_SAME || EPI == E_AD_SAME_BD) && a.g_same != 0.f) apply_A_pair<S>(a, t, EPI == E_AD_SAME_BD, m, o);
     if ((EPI == E_SAME_AINV || EPI == E_SAME_BD) && a.g_same != 0.f) {
       float2 y[24];
-      load_pair24<S>(a.same, a.same_nrm, t, a.N, y);
+      load_pair24<S>(a.same, a.same_nrm, plane_of(a), t, a.N, y);
       const float2 g = f2(a.g_same);
 #pragma unroll
       for (int i = 0; i < 24; i++) o[i] = fma2(g, y[i], o[i]);
@@ -508,11 +508,11 @@ __device__ __forceinline__ void pair_epilogue(const FastArgs<S, float>& a, const
     if ((EPI == E_RAW || EPI == E_A_SAME || EPI == E_AD_SAME_BD || EPI == E_SAME_AINV || EPI == E_SAME_BD) &&
         a.add != nullptr) {
       float2 y[24];
-      load_pair24<S>(a.add, a.add_nrm, t, a.N, y);
+      load_pair24<S>(a.add, a.add_nrm, plane_of(a), t, a.N, y);
 #pragma unroll
       for (int i = 0; i < 24; i++) o[i] = add2(o[i], y[i]);
     }
-    store_pair24<S>(a.out, a.out_nrm, t, a.N, o);
+    store_pair24<S>(a.out, a.out_nrm, plane_of(a), t, a.N, o);
     if (a.partials != nullptr) {
 #pragma unroll
       for (int i = 0; i < 24; i++) n2 = fma2(o[i], o[i], n2);
@@ -597,15 +597,16 @@ __device__ __forceinline__ void pf_issue(const FastArgs<__half, float>& a, const
   const int hn = nbr_half<MU, FWD>(a.g, x);
   const long uA = ((long)hn * a.L5 + t.s0) * a.N + t.r;
   const long uB = t.two ? uA + a.N : uA;
-  const uint4* pa = reinterpret_cast<const uint4*>(a.in + 24 * uA);
-  const uint4* pb = reinterpret_cast<const uint4*>(a.in + 24 * uB);
+  const long pl = plane_of(a);
+  const uint4* pa = reinterpret_cast<const uint4*>(a.in) + uA;
+  const uint4* pb = reinterpret_cast<const uint4*>(a.in) + uB;
   uint4* d = reinterpret_cast<uint4*>(stage);
   cp_async16(d, pa);
-  cp_async16(d + 1, pa + 1);
-  cp_async16(d + 2, pa + 2);
+  cp_async16(d + 1, pa + pl);
+  cp_async16(d + 2, pa + 2 * pl);
   cp_async16(d + 3, pb);
-  cp_async16(d + 4, pb + 1);
-  cp_async16(d + 5, pb + 2);
+  cp_async16(d + 4, pb + pl);
+  cp_async16(d + 5, pb + 2 * pl);
   float* sc = reinterpret_cast<float*>(d + 6);
   cp_async4(sc, a.in_nrm + uA);
   cp_async4(sc + 1, a.in_nrm + uB);

@@ -623,7 +623,6 @@ struct BatchSolver {
   F<float> xf, uf, tf, qf;       // FP32 reliable updates
   F<S> p, u, t, q, rho, r;       // inner vectors
   F<SX> xlo;
-  long xlo_n = 0;                 // units x_lo holds (tile-major FP32: the whole BLAS grid)
   double* part = nullptr;
   double* mass64 = nullptr;
   float* mass32 = nullptr;
@@ -717,9 +716,7 @@ struct BatchSolver {
     F<S>* fS[] = {&p, &u, &t, &q, &rho, &r};
     const char* nS[] = {"p", "u", "t", "q", "rho", "r"};
     for (int i = 0; i < 6; i++) CK(ws_field<S>(c, wsp + "S." + nS[i], units, fS[i]));
-    // x_lo: tile-major over the BLAS tiling when it is FP32 (axpy_x_rho, accum_xhi, zero_xlo)
-    xlo_n = xlo_units(tl_blas, units, !kFP64);
-    CK(ws_field<SX>(c, wsp + "xlo", xlo_n, &xlo));
+    CK(ws_field<SX>(c, wsp + "xlo", units, &xlo));
     part = (double*)ws_get(c, wsp + "partials", sizeof(double) * g.Vh * N, &e); CK(e);
     double* d = (double*)ws_get(c, wsp + "scal_d", sizeof(double) * 12 * N, &e); CK(e);
     int* ip = (int*)ws_get(c, wsp + "scal_i", sizeof(int) * 4 * N, &e); CK(e);
@@ -735,7 +732,7 @@ struct BatchSolver {
     const size_t b64 = sizeof(double) * 24 * (size_t)units;
     CK(cudaMemsetAsync(x_acc.v, 0, b64, st));
     CK(cudaMemsetAsync(x_hi.v, 0, b64, st));
-    CK(cudaMemsetAsync(xlo.v, 0, sizeof(SX) * 24 * (size_t)xlo_n, st));
+    CK(cudaMemsetAsync(xlo.v, 0, sizeof(SX) * 24 * (size_t)units, st));
     CK(cudaMemsetAsync(p.v, 0, sizeof(S) * 24 * (size_t)units, st));
     if (p.n) CK(cudaMemsetAsync(p.n, 0, sizeof(float) * (size_t)units, st));
     if (tune_request >= 0) {
@@ -1051,13 +1048,11 @@ int solve_batch_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const* srcs, 
   // Schur right-hand side bhat_e = b_e + 1/2 H_eo B A^-1 b_o in bhat (FP64); the
   // sources are packed into rho64 (b_e) and x_hi (b_o), which are free then.
   auto schur_source = [&](bool norms) -> int {
-    sv.launches += 2 * N;
+    sv.launches += 2;
     sv.b_e = sv.rho64;
     sv.b_o = sv.x_hi;
-    for (int i = 0; i < N; i++) {
-      CK(pack_rhs<double>(srcs[i], sv.b_e.v, nullptr, g, L5, N, 0, i, st));
-      CK(pack_rhs<double>(srcs[i], sv.b_o.v, nullptr, g, L5, N, 1, i, st));
-    }
+    CK(pack_rhs<double>(srcs, sv.b_e.v, nullptr, g, L5, N, 0, 0, N, st));
+    CK(pack_rhs<double>(srcs, sv.b_o.v, nullptr, g, L5, N, 1, 0, N, st));
     if (norms) {
       CK(sv.norms(sv.b_e, nullptr, tmp));
       CK(cudaMemcpyAsync(bb.data(), tmp, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
@@ -1175,16 +1170,14 @@ int solve_batch_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const* srcs, 
   // reuses y.  Even sites: b_e - A x_e + 1/2 H_eo B x_o (the second FP64 hop).
   std::vector<double> re(N), ro(N);
   auto finish = [&]() -> int {
-    sv.launches += 2 + 2 * N;
+    sv.launches += 4;
     CK(accum_xhi<typename BatchSolver<S>::SX>(sv.x_hi.v, sv.xlo.v, sv.tl_blas, g.Vh, L5, N, nullptr, st));
     CK(accum_xhi<double>(sv.x_acc.v, sv.x_hi.v, sv.tl_blas, g.Vh, L5, N, nullptr, st));
     // sources again, in fields now free (bhat, x_hi)
     sv.b_e = sv.bhat;
     sv.b_o = sv.x_hi;
-    for (int i = 0; i < N; i++) {
-      CK(pack_rhs<double>(srcs[i], sv.b_e.v, nullptr, g, L5, N, 0, i, st));
-      CK(pack_rhs<double>(srcs[i], sv.b_o.v, nullptr, g, L5, N, 1, i, st));
-    }
+    CK(pack_rhs<double>(srcs, sv.b_e.v, nullptr, g, L5, N, 0, 0, N, st));
+    CK(pack_rhs<double>(srcs, sv.b_o.v, nullptr, g, L5, N, 1, 0, N, st));
     sv.launches += 2;
     CK(bop<double>(sv.x_acc.v, nullptr, sv.u64.v, nullptr, sv.op64.f, sv.tl_blas, g.Vh, L5, N, nullptr, st));
     CK(sv.op64.run(E_RAW, 1, 0, sv.u64, none, sv.b_o, 0.0, 0.5, sv.t64, nullptr, nullptr));
@@ -1199,11 +1192,9 @@ int solve_batch_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const* srcs, 
     CK(sv.norms(sv.rho64, nullptr, tmp));
     CK(cudaMemcpyAsync(re.data(), tmp, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(iters.data(), sv.sc.iters, sizeof(int) * N, cudaMemcpyDeviceToHost, st));
-    sv.launches += 2 * N;
-    for (int i = 0; i < N; i++) {
-      CK(unpack_rhs<double>(sv.x_acc.v, nullptr, xs[i], g, L5, N, 0, i, st));
-      CK(unpack_rhs<double>(x_o.v, nullptr, xs[i], g, L5, N, 1, i, st));
-    }
+    sv.launches += 2;
+    CK(unpack_rhs<double>(sv.x_acc.v, nullptr, xs, g, L5, N, 0, 0, N, st));
+    CK(unpack_rhs<double>(x_o.v, nullptr, xs, g, L5, N, 1, 0, N, st));
     CK(cudaStreamSynchronize(st));
     CK(ph.mark(PH_FINAL, st));
     return MDWF_OK;
@@ -1388,10 +1379,10 @@ struct SessionImpl : SessionBase {
     const int* m = sv.umask_d;
     CK(zero_masked<double>(sv.x_acc.v, nullptr, sv.tl_blas, g.Vh, L5, N, m, st));
     CK(zero_masked<double>(sv.x_hi.v, nullptr, sv.tl_blas, g.Vh, L5, N, m, st));
-    CK(zero_xlo<typename BatchSolver<S>::SX>(sv.xlo.v, sv.tl_blas, g.Vh, L5, N, m, st));
+    CK(zero_masked<typename BatchSolver<S>::SX>(sv.xlo.v, nullptr, sv.tl_blas, g.Vh, L5, N, m, st));
     CK(zero_masked<S>(sv.p.v, sv.p.n, sv.tl_blas, g.Vh, L5, N, m, st));
-    CK(pack_rhs<double>(src, sv.b_e.v, nullptr, g, L5, N, 0, r, st));
-    CK(pack_rhs<double>(src, sv.b_o.v, nullptr, g, L5, N, 1, r, st));
+    CK(pack_rhs<double>(&src, sv.b_e.v, nullptr, g, L5, N, 0, r, 1, st));
+    CK(pack_rhs<double>(&src, sv.b_o.v, nullptr, g, L5, N, 1, r, 1, st));
     std::vector<double> be(N), bo(N);
     CK(sv.norms(sv.b_e, m, sv.sc.tmp));
     CK(cudaMemcpyAsync(be.data(), sv.sc.tmp, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
@@ -1504,8 +1495,8 @@ struct SessionImpl : SessionBase {
     CK(cudaMemcpyAsync(ro.data(), sv.sc.tmp, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
     for (int i = 0; i < N; i++) {
       if (!fin[i]) continue;
-      CK(unpack_rhs<double>(sv.x_acc.v, nullptr, outs[i], g, L5, N, 0, i, st));
-      CK(unpack_rhs<double>(sv.x_o.v, nullptr, outs[i], g, L5, N, 1, i, st));
+      CK(unpack_rhs<double>(sv.x_acc.v, nullptr, &outs[i], g, L5, N, 0, i, 1, st));
+      CK(unpack_rhs<double>(sv.x_o.v, nullptr, &outs[i], g, L5, N, 1, i, 1, st));
     }
     CK(cudaStreamSynchronize(st));
     auto now = std::chrono::steady_clock::now();
@@ -1617,9 +1608,9 @@ int apply_5d_dev(mdwf_ctx* ctx, const Cfg* cfg, int which, int dagger, const dou
   static const int kinds[3][2] = {{MK_A, MK_Ad}, {MK_B, MK_Bd}, {MK_Ainv, MK_Ainvd}};
   const double* G = M[kinds[which][dagger ? 1 : 0]];
   for (int par = 0; par < 2; par++) {
-    CK(pack_rhs<double>(in_dev, in.v, nullptr, g, L5, 1, par, 0, st));
+    CK(pack_rhs<double>(&in_dev, in.v, nullptr, g, L5, 1, par, 0, 1, st));
     CK(op.run(false, par, 0, in, none, G, none, nullptr, 0.0, out, nullptr, nullptr));
-    CK(unpack_rhs<double>(out.v, nullptr, out_dev, g, L5, 1, par, 0, st));
+    CK(unpack_rhs<double>(out.v, nullptr, &out_dev, g, L5, 1, par, 0, 1, st));
   }
   CK(cudaStreamSynchronize(st));
   return MDWF_OK;
@@ -1671,8 +1662,8 @@ int dd_impl(mdwf_ctx* ctx, Cfg* cfg, bool pack, int kind, int dagger, const doub
   CK(ws_field<double>(ctx, "dd.io", units, &io));
   CK(ws_field<double>(ctx, "dd.te", units, &te));
   CK(ws_field<double>(ctx, "dd.to", units, &to));
-  CK(pack_rhs<double>(in_dev, ie.v, nullptr, g, L5, 1, 0, 0, st));
-  CK(pack_rhs<double>(in_dev, io.v, nullptr, g, L5, 1, 1, 0, st));
+  CK(pack_rhs<double>(&in_dev, ie.v, nullptr, g, L5, 1, 0, 0, 1, st));
+  CK(pack_rhs<double>(&in_dev, io.v, nullptr, g, L5, 1, 1, 0, 1, st));
   cudaError_t me = cudaSuccess;
   double* mass = (double*)ws_get(ctx, "dd.mass", sizeof(double), &me);
   CK(me);
@@ -1718,18 +1709,15 @@ int schur_apply_impl(mdwf_ctx* ctx, Cfg* cfg, const double* in_dev, double* out_
   long units = g.Vh * L5;
   FieldBuf<S> in, u, t, out;
   for (auto* f : {&in, &u, &t, &out}) CK(f->alloc(units));
-  FieldBuf<double> o64;
-  CK(o64.alloc(2 * units));
-  CK(pack_rhs<S>(in_dev, in.f().v, in.f().n, g, L5, 1, 0, 0, st));
+  CK(pack_rhs<S>(&in_dev, in.f().v, in.f().n, g, L5, 1, 0, 0, 1, st));
   if (!dagger) {
     CK(bop<S>(in.f().v, in.f().n, u.f().v, u.f().n, op.f, tb, g.Vh, L5, 1, nullptr, st));
     CK(op.mhat(in.f(), u.f(), t.f(), out.f(), nullptr, nullptr));
   } else {
     CK(op.mhat_dag(in.f(), t.f(), out.f(), nullptr, nullptr));
   }
-  CK(unpack_rhs<S>(out.f().v, out.f().n, out_dev, g, L5, 1, 0, 0, st));
-  CK(cudaMemsetAsync(o64.v.p, 0, o64.v.bytes, st));
-  CK(unpack_rhs<double>(o64.f().v, nullptr, out_dev, g, L5, 1, 1, 0, st));
+  CK(unpack_rhs<S>(out.f().v, out.f().n, &out_dev, g, L5, 1, 0, 0, 1, st));
+  CK(unpack_rhs<S>(nullptr, nullptr, &out_dev, g, L5, 1, 1, 0, 1, st));
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, errw.p, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -1771,20 +1759,15 @@ int schur_batch_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const* in, do
   CK(ws_field<S>(ctx, "sb.u", units, &fu));
   CK(ws_field<S>(ctx, "sb.t", units, &ft));
   CK(ws_field<S>(ctx, "sb.out", units, &fo));
-  F<double> zero;
-  CK(ws_field<double>(ctx, "sb.zero", g.Vh * L5, &zero));
-  CK(cudaMemsetAsync(zero.v, 0, sizeof(double) * 24 * (size_t)g.Vh * L5, st));
-  for (int i = 0; i < N; i++) CK(pack_rhs<S>(in[i], fin.v, fin.n, g, L5, N, 0, i, st));
+  CK(pack_rhs<S>(in, fin.v, fin.n, g, L5, N, 0, 0, N, st));
   if (!dagger) {
     CK(bop<S>(fin.v, fin.n, fu.v, fu.n, op.f, tb, g.Vh, L5, N, nullptr, st));
     CK(op.mhat(fin, fu, ft, fo, nullptr, nullptr));
   } else {
     CK(op.mhat_dag(fin, ft, fo, nullptr, nullptr));
   }
-  for (int i = 0; i < N; i++) {
-    CK(unpack_rhs<S>(fo.v, fo.n, out[i], g, L5, N, 0, i, st));
-    CK(unpack_rhs<double>(zero.v, nullptr, out[i], g, L5, 1, 1, 0, st));
-  }
+  CK(unpack_rhs<S>(fo.v, fo.n, out, g, L5, N, 0, 0, N, st));
+  CK(unpack_rhs<S>(nullptr, nullptr, out, g, L5, N, 1, 0, N, st));
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, errw, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -2391,21 +2374,15 @@ int schur_batch_noalloc_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const
   op.f = make_fifth<T>(cfg->act, mass);
   choose_hop(op, cfg, 0, HOP_DIRECT, nullptr);
   Tiling tb = blas_tiling(g.Vh, L5, N, 1024);
-  for (int i = 0; i < N; i++) CK(pack_rhs<S>(in[i], fin.v, fin.n, g, L5, N, 0, i, st));
+  CK(pack_rhs<S>(in, fin.v, fin.n, g, L5, N, 0, 0, N, st));
   if (!dagger) {
     CK(bop<S>(fin.v, fin.n, fu.v, fu.n, op.f, tb, g.Vh, L5, N, nullptr, st));
     CK(op.mhat(fin, fu, ft, fo, nullptr, nullptr));
   } else {
     CK(op.mhat_dag(fin, ft, fo, nullptr, nullptr));
   }
-  // the intermediate odd field is no longer needed: zero it and use it as the
-  // source of the odd sites of every output (they must come out zero)
-  CK(cudaMemsetAsync(ft.v, 0, fbytes, st));
-  if (nbytes) CK(cudaMemsetAsync(ft.n, 0, nbytes, st));
-  for (int i = 0; i < N; i++) {
-    CK(unpack_rhs<S>(fo.v, fo.n, out[i], g, L5, N, 0, i, st));
-    CK(unpack_rhs<S>(ft.v, ft.n, out[i], g, L5, N, 1, i, st));
-  }
+  CK(unpack_rhs<S>(fo.v, fo.n, out, g, L5, N, 0, 0, N, st));
+  CK(unpack_rhs<S>(nullptr, nullptr, out, g, L5, N, 1, 0, N, st));
   CK(cudaStreamSynchronize(st));
   return MDWF_OK;
 }

@@ -1,15 +1,15 @@
 // Internal definitions shared by the libmdwf CUDA sources.
 //
 // Device layouts
-//   spinor field, one parity:   [h][s][r][24]   h = half-lattice site, s = fifth
-//                                                 dimension slice, r = RHS slot,
-//                                                 24 = [spin 4][colour 3][re, im]
+//   spinor field, one parity:   [word][h][s][r] h = half-lattice site, s = fifth dimension slice,
+//                                                 r = RHS slot; the words are the 16-byte pieces
+//                                                 of a unit's 24 reals, [spin 4][colour 3][re, im]
 //   16-bit storage adds a scale per (h, s, r):   nrm[h][s][r] (float); the stored
 //                                                 values are v / nrm, nrm = the smallest power
 //                                                 of two >= max |v| of the unit.
 //   fp16 storage orders the 24 reals of a unit colour-major, [colour][spin][re,im],
-//   so that the four spins of one colour are one 16-byte word (the tensor-core hop
-//   loads them per lane); every other type, and every register copy, uses
+//   so that the four spins of one colour are one 16-byte word (the hops project a
+//   word at a time); every other type, and every register copy, uses
 //   [spin][colour][re,im].
 //   gauge field:                [parity][h][mu][18]   (3x3 complex, row major),
 //                                mu = 0..3 for x, y, z, t; U_mu(x) of the site x;
@@ -67,40 +67,46 @@ template <> struct StoreTraits<float> { using T = float; static constexpr bool k
 template <> struct StoreTraits<__half> { using T = float; static constexpr bool kNorm = true; };
 template <> struct StoreTraits<__nv_bfloat16> { using T = float; static constexpr bool kNorm = false; };
 
-// Load the 24 reals of unit u (unit = (h * L5 + s) * N + r).
+// A field is stored as planes of 16-byte words: word w of unit u (u = (h * L5 + s) * N + r, `pl` units in
+// the field) is the 16 bytes at w * pl + u, so that the lanes of a warp, on consecutive units, read
+// 512 contiguous bytes per load.  (With the 48 to 192 bytes of a unit side by side each such load
+// touched three to twelve times as many cache lines.)  12 words for FP64, 6 for FP32, 3 for the 16-bit types.
+template <typename S> constexpr int kWords = (int)sizeof(S) * 24 / 16;
+
+// Load the 24 reals of unit u.
 template <typename S, typename T>
-__device__ __forceinline__ void load24(const S* __restrict__ v, const float* __restrict__ nrm, long u, T a[24]);
+__device__ __forceinline__ void load24(const S* __restrict__ v, const float* __restrict__ nrm, long pl, long u, T a[24]);
 
 template <>
-__device__ __forceinline__ void load24<double, double>(const double* __restrict__ v, const float*, long u, double a[24]) {
-  const double2* p = reinterpret_cast<const double2*>(v + 24 * u);
+__device__ __forceinline__ void load24<double, double>(const double* __restrict__ v, const float*, long pl, long u, double a[24]) {
+  const double2* p = reinterpret_cast<const double2*>(v) + u;
 #pragma unroll
-  for (int i = 0; i < 12; i++) { double2 t = __ldg(p + i); a[2 * i] = t.x; a[2 * i + 1] = t.y; }
+  for (int i = 0; i < 12; i++) { double2 t = __ldg(p + i * pl); a[2 * i] = t.x; a[2 * i + 1] = t.y; }
 }
 template <>
-__device__ __forceinline__ void load24<float, float>(const float* __restrict__ v, const float*, long u, float a[24]) {
-  const float4* p = reinterpret_cast<const float4*>(v + 24 * u);
+__device__ __forceinline__ void load24<float, float>(const float* __restrict__ v, const float*, long pl, long u, float a[24]) {
+  const float4* p = reinterpret_cast<const float4*>(v) + u;
 #pragma unroll
-  for (int i = 0; i < 6; i++) { float4 t = __ldg(p + i); a[4*i] = t.x; a[4*i+1] = t.y; a[4*i+2] = t.z; a[4*i+3] = t.w; }
+  for (int i = 0; i < 6; i++) { float4 t = __ldg(p + i * pl); a[4*i] = t.x; a[4*i+1] = t.y; a[4*i+2] = t.z; a[4*i+3] = t.w; }
 }
 template <>
-__device__ __forceinline__ void load24<__half, float>(const __half* __restrict__ v, const float* __restrict__ nrm, long u, float a[24]) {
-  const uint4* p = reinterpret_cast<const uint4*>(v + 24 * u);
+__device__ __forceinline__ void load24<__half, float>(const __half* __restrict__ v, const float* __restrict__ nrm, long pl, long u, float a[24]) {
+  const uint4* p = reinterpret_cast<const uint4*>(v) + u;
   const float s = __ldg(nrm + u);
 #pragma unroll
   for (int c = 0; c < 3; c++) {           // word c: spins 0..3 of colour c
-    uint4 t = __ldg(p + c);
+    uint4 t = __ldg(p + c * pl);
     const __half2* hh = reinterpret_cast<const __half2*>(&t);
 #pragma unroll
     for (int k = 0; k < 4; k++) { float2 f = __half22float2(hh[k]); a[6*k+2*c] = f.x * s; a[6*k+2*c+1] = f.y * s; }
   }
 }
 template <>
-__device__ __forceinline__ void load24<__nv_bfloat16, float>(const __nv_bfloat16* __restrict__ v, const float*, long u, float a[24]) {
-  const uint4* p = reinterpret_cast<const uint4*>(v + 24 * u);
+__device__ __forceinline__ void load24<__nv_bfloat16, float>(const __nv_bfloat16* __restrict__ v, const float*, long pl, long u, float a[24]) {
+  const uint4* p = reinterpret_cast<const uint4*>(v) + u;
 #pragma unroll
   for (int i = 0; i < 3; i++) {
-    uint4 t = __ldg(p + i);
+    uint4 t = __ldg(p + i * pl);
     const __nv_bfloat162* hh = reinterpret_cast<const __nv_bfloat162*>(&t);
 #pragma unroll
     for (int j = 0; j < 4; j++) { float2 f = __bfloat1622float2(hh[j]); a[8*i+2*j] = f.x; a[8*i+2*j+1] = f.y; }
@@ -131,77 +137,78 @@ __device__ __forceinline__ void half_scale(float m, float* sc, float* inv) {
 
 // Store the 24 reals of unit u.
 template <typename S, typename T>
-__device__ __forceinline__ void store24(S* __restrict__ v, float* __restrict__ nrm, long u, const T a[24]);
+__device__ __forceinline__ void store24(S* __restrict__ v, float* __restrict__ nrm, long pl, long u, const T a[24]);
 
 template <>
-__device__ __forceinline__ void store24<double, double>(double* __restrict__ v, float*, long u, const double a[24]) {
-  double2* p = reinterpret_cast<double2*>(v + 24 * u);
+__device__ __forceinline__ void store24<double, double>(double* __restrict__ v, float*, long pl, long u, const double a[24]) {
+  double2* p = reinterpret_cast<double2*>(v) + u;
 #pragma unroll
-  for (int i = 0; i < 12; i++) p[i] = make_double2(a[2 * i], a[2 * i + 1]);
+  for (int i = 0; i < 12; i++) p[i * pl] = make_double2(a[2 * i], a[2 * i + 1]);
 }
 template <>
-__device__ __forceinline__ void store24<float, float>(float* __restrict__ v, float*, long u, const float a[24]) {
-  float4* p = reinterpret_cast<float4*>(v + 24 * u);
+__device__ __forceinline__ void store24<float, float>(float* __restrict__ v, float*, long pl, long u, const float a[24]) {
+  float4* p = reinterpret_cast<float4*>(v) + u;
 #pragma unroll
-  for (int i = 0; i < 6; i++) p[i] = make_float4(a[4*i], a[4*i+1], a[4*i+2], a[4*i+3]);
+  for (int i = 0; i < 6; i++) p[i * pl] = make_float4(a[4*i], a[4*i+1], a[4*i+2], a[4*i+3]);
 }
 template <>
-__device__ __forceinline__ void store24<__half, float>(__half* __restrict__ v, float* __restrict__ nrm, long u, const float a[24]) {
+__device__ __forceinline__ void store24<__half, float>(__half* __restrict__ v, float* __restrict__ nrm, long pl, long u, const float a[24]) {
   float m = 0.f;
 #pragma unroll
   for (int i = 0; i < 24; i++) m = fmaxf(m, fabsf(a[i]));
   float sc, inv;
   half_scale(m, &sc, &inv);
   nrm[u] = sc;
-  uint4* p = reinterpret_cast<uint4*>(v + 24 * u);
+  uint4* p = reinterpret_cast<uint4*>(v) + u;
 #pragma unroll
   for (int c = 0; c < 3; c++) {
     uint4 t;
     __half2* hh = reinterpret_cast<__half2*>(&t);
 #pragma unroll
     for (int k = 0; k < 4; k++) hh[k] = __floats2half2_rn(a[6*k+2*c] * inv, a[6*k+2*c+1] * inv);
-    p[c] = t;
+    p[c * pl] = t;
   }
 }
 template <>
-__device__ __forceinline__ void store24<__nv_bfloat16, float>(__nv_bfloat16* __restrict__ v, float*, long u, const float a[24]) {
-  uint4* p = reinterpret_cast<uint4*>(v + 24 * u);
+__device__ __forceinline__ void store24<__nv_bfloat16, float>(__nv_bfloat16* __restrict__ v, float*, long pl, long u, const float a[24]) {
+  uint4* p = reinterpret_cast<uint4*>(v) + u;
 #pragma unroll
   for (int i = 0; i < 3; i++) {
     uint4 t;
     __nv_bfloat162* hh = reinterpret_cast<__nv_bfloat162*>(&t);
 #pragma unroll
     for (int j = 0; j < 4; j++) hh[j] = __floats2bfloat162_rn(a[8*i+2*j], a[8*i+2*j+1]);
-    p[i] = t;
+    p[i * pl] = t;
   }
 }
 
 // Half of a stored spinor: part 0 = spins 0,1 (components 0..11), part 1 = spins 2,3.
 template <typename S, typename T>
-__device__ __forceinline__ void load_part(const S* __restrict__ v, const float* __restrict__ nrm, long u, int part,
+__device__ __forceinline__ void load_part(const S* __restrict__ v, const float* __restrict__ nrm, long pl, long u, int part,
                                           T* o);
 template <>
-__device__ __forceinline__ void load_part<double, double>(const double* __restrict__ v, const float*, long u, int part,
+__device__ __forceinline__ void load_part<double, double>(const double* __restrict__ v, const float*, long pl, long u, int part,
                                                           double* o) {
-  const double2* p = reinterpret_cast<const double2*>(v + 24 * u + 12 * part);
+  const double2* p = reinterpret_cast<const double2*>(v) + 6 * part * pl + u;
 #pragma unroll
-  for (int i = 0; i < 6; i++) { double2 t = __ldg(p + i); o[2 * i] = t.x; o[2 * i + 1] = t.y; }
+  for (int i = 0; i < 6; i++) { double2 t = __ldg(p + i * pl); o[2 * i] = t.x; o[2 * i + 1] = t.y; }
 }
 template <>
-__device__ __forceinline__ void load_part<float, float>(const float* __restrict__ v, const float*, long u, int part,
+__device__ __forceinline__ void load_part<float, float>(const float* __restrict__ v, const float*, long pl, long u, int part,
                                                         float* o) {
-  const float4* p = reinterpret_cast<const float4*>(v + 24 * u + 12 * part);
+  const float4* p = reinterpret_cast<const float4*>(v) + 3 * part * pl + u;
 #pragma unroll
-  for (int i = 0; i < 3; i++) { float4 t = __ldg(p + i); o[4*i] = t.x; o[4*i+1] = t.y; o[4*i+2] = t.z; o[4*i+3] = t.w; }
+  for (int i = 0; i < 3; i++) { float4 t = __ldg(p + i * pl); o[4*i] = t.x; o[4*i+1] = t.y; o[4*i+2] = t.z; o[4*i+3] = t.w; }
 }
 template <>
 __device__ __forceinline__ void load_part<__half, float>(const __half* __restrict__ v, const float* __restrict__ nrm,
-                                                         long u, int part, float* o) {
-  // colour-major storage: spins 2 part, 2 part + 1 of colour c are the 8 bytes at 16 c + 8 part
+                                                         long pl, long u, int part, float* o) {
+  // colour-major storage: spins 2 part, 2 part + 1 of colour c are half `part` of word c
+  const uint2* p = reinterpret_cast<const uint2*>(v) + 2 * u + part;
   const float s = __ldg(nrm + u);
 #pragma unroll
   for (int c = 0; c < 3; c++) {
-    uint2 t = __ldg(reinterpret_cast<const uint2*>(v + 24 * u + 8 * c + 4 * part));
+    uint2 t = __ldg(p + 2 * c * pl);
     const __half2* hh = reinterpret_cast<const __half2*>(&t);
     float2 a = __half22float2(hh[0]), b = __half22float2(hh[1]);
     o[2*c] = a.x * s; o[2*c+1] = a.y * s; o[6+2*c] = b.x * s; o[6+2*c+1] = b.y * s;
@@ -209,49 +216,31 @@ __device__ __forceinline__ void load_part<__half, float>(const __half* __restric
 }
 template <>
 __device__ __forceinline__ void load_part<__nv_bfloat16, float>(const __nv_bfloat16* __restrict__ v, const float*,
-                                                                long u, int part, float* o) {
-  const uint2* p = reinterpret_cast<const uint2*>(v + 24 * u + 12 * part);
+                                                                long pl, long u, int part, float* o) {
+  const uint2* p = reinterpret_cast<const uint2*>(v) + 2 * u;
 #pragma unroll
   for (int i = 0; i < 3; i++) {
-    uint2 t = __ldg(p + i);
+    const int k = 3 * part + i;            // half words of the unit: half k & 1 of word k >> 1
+    uint2 t = __ldg(p + 2 * (k >> 1) * pl + (k & 1));
     const __nv_bfloat162* hh = reinterpret_cast<const __nv_bfloat162*>(&t);
     float2 a = __bfloat1622float2(hh[0]), b = __bfloat1622float2(hh[1]);
     o[4*i] = a.x; o[4*i+1] = a.y; o[4*i+2] = b.x; o[4*i+3] = b.y;
   }
 }
 
-// Plain (shared-memory) loads of a stored spinor, without the fp16 scale.
+// Plain (shared-memory) loads of a staged spinor, without the fp16 scale: words `pl` apart.
 template <typename S, typename T>
-__device__ __forceinline__ void load24_smem(const S* p, T a[24]);
+__device__ __forceinline__ void load24_smem(const uint4* q, int pl, T a[24]);
 template <>
-__device__ __forceinline__ void load24_smem<double, double>(const double* p, double a[24]) {
-  const double2* q = reinterpret_cast<const double2*>(p);
+__device__ __forceinline__ void load24_smem<float, float>(const uint4* q, int pl, float a[24]) {
 #pragma unroll
-  for (int i = 0; i < 12; i++) { double2 t = q[i]; a[2 * i] = t.x; a[2 * i + 1] = t.y; }
+  for (int i = 0; i < 6; i++) { const float4 t = reinterpret_cast<const float4*>(q)[i * pl]; a[4*i] = t.x; a[4*i+1] = t.y; a[4*i+2] = t.z; a[4*i+3] = t.w; }
 }
 template <>
-__device__ __forceinline__ void load24_smem<float, float>(const float* p, float a[24]) {
-  const float4* q = reinterpret_cast<const float4*>(p);
-#pragma unroll
-  for (int i = 0; i < 6; i++) { float4 t = q[i]; a[4*i] = t.x; a[4*i+1] = t.y; a[4*i+2] = t.z; a[4*i+3] = t.w; }
-}
-template <>
-__device__ __forceinline__ void load24_smem<__half, float>(const __half* p, float a[24]) {
-  const uint4* q = reinterpret_cast<const uint4*>(p);
-#pragma unroll
-  for (int c = 0; c < 3; c++) {
-    uint4 t = q[c];
-    const __half2* hh = reinterpret_cast<const __half2*>(&t);
-#pragma unroll
-    for (int k = 0; k < 4; k++) { float2 f = __half22float2(hh[k]); a[6*k+2*c] = f.x; a[6*k+2*c+1] = f.y; }
-  }
-}
-template <>
-__device__ __forceinline__ void load24_smem<__nv_bfloat16, float>(const __nv_bfloat16* p, float a[24]) {
-  const uint4* q = reinterpret_cast<const uint4*>(p);
+__device__ __forceinline__ void load24_smem<__nv_bfloat16, float>(const uint4* q, int pl, float a[24]) {
 #pragma unroll
   for (int i = 0; i < 3; i++) {
-    uint4 t = q[i];
+    uint4 t = q[i * pl];
     const __nv_bfloat162* hh = reinterpret_cast<const __nv_bfloat162*>(&t);
 #pragma unroll
     for (int j = 0; j < 4; j++) { float2 f = __bfloat1622float2(hh[j]); a[8*i+2*j] = f.x; a[8*i+2*j+1] = f.y; }
@@ -385,6 +374,10 @@ __device__ __forceinline__ float bop_term(float b5, float x, float cw, float y) 
 
 // Shared-memory staging of the neighbour sites (hop_staged_kernel).
 #define MDWF_TIMEOUT_CODE 1
+// Units of a hop's fields.
+template <typename A>
+__host__ __device__ __forceinline__ long plane_of(const A& a) { return a.g.Vh * a.L5 * a.N; }
+
 struct StageInfo {
   unsigned spin_bytes;  // 8 * nsb * (L5 N) stored spinors
   unsigned nrm_bytes;   // 8 * nsb * (L5 N) fp16 scales (0: loaded directly)
