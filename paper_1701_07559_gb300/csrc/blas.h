@@ -74,8 +74,8 @@ cudaError_t z2_source(unsigned long long seed, double* eta, long V, cudaStream_t
 // src = f w + hc H w, w = P_+ eta on slice 0 and P_- eta on slice L5 - 1.
 cudaError_t wall_source(const double* U, const double* eta, double* src, const Geom& g, int L5, int anti, double f,
                         double hc, cudaStream_t st);
-// n_iter smearing steps of eta in place; tmp: V * 24 doubles, flags: Lt ints.
-cudaError_t smear(const double* U, double* eta, double* tmp, int* flags, const Geom& g, double k, int n_iter,
+// n_iter smearing steps of eta in place; tmp: V * 24 doubles, slices: 2 Lt + 1 ints.
+cudaError_t smear(const double* U, double* eta, double* tmp, int* slices, const Geom& g, double k, int n_iter,
                   cudaStream_t st);
 // c[2][Lt]: the two residual-mass correlators; part: 2 Lt mres_blocks(V / Lt) doubles.
 int mres_blocks(long slice_sites);

@@ -2286,10 +2286,10 @@ int mdwf_smear_source_dev(mdwf_ctx* ctx, int cfg_id, double* eta4d, double sigma
   cudaError_t e = cudaSuccess;
   double* tmp = (double*)ws_get(ctx, "smear.tmp", sizeof(double) * 24 * (size_t)ctx->g.V, &e);
   CK(e);
-  int* flags = (int*)ws_get(ctx, "smear.flags", sizeof(int) * ctx->g.L[3], &e);
+  int* slices = (int*)ws_get(ctx, "smear.slices", sizeof(int) * (2 * ctx->g.L[3] + 1), &e);
   CK(e);
   const double k = sigma * sigma / (4.0 * n_iter);
-  CK(smear(it->second.U64, eta4d, tmp, flags, ctx->g, k, n_iter, st));
+  CK(smear(it->second.U64, eta4d, tmp, slices, ctx->g, k, n_iter, st));
   CK(cudaStreamSynchronize(st));
   return MDWF_OK;
 }
