@@ -52,6 +52,7 @@ struct Cfg {
 
 struct mdwf_ctx {
   int device = 0;
+  int clock_khz = 2000000;   // SM clock, read once: the query takes 0.6 ms
   Geom g;
   std::map<int, Cfg> cfgs;
   std::string err;
@@ -548,11 +549,7 @@ Tiling fast_tiling(const Geom& g, int L5, int N, int nsb_req, bool* staged, bool
 }
 
 // Bound of device-side waits in clock cycles.
-long long wait_budget(int device, double seconds) {
-  int khz = 0;
-  if (cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, device) != cudaSuccess || khz <= 0) khz = 2000000;
-  return (long long)(seconds * 1e3 * (double)khz);
-}
+long long wait_budget(const mdwf_ctx* ctx, double seconds) { return (long long)(seconds * 1e3 * (double)ctx->clock_khz); }
 
 template <typename T>
 Fifth<T> make_fifth(const Action& act, const T* mass_dev) {
@@ -673,7 +670,7 @@ struct BatchSolver {
     errw = (int*)ws_get(c, wsp + "errw", sizeof(int), &e); CK(e);
     CK(cudaMemsetAsync(errw, 0, sizeof(int), st));
     stage.spin_bytes = stage.nrm_bytes = 0;
-    stage.budget = wait_budget(c->device, o.wait_timeout_s > 0 ? o.wait_timeout_s : 2.0);
+    stage.budget = wait_budget(c, o.wait_timeout_s > 0 ? o.wait_timeout_s : 2.0);
     stage.extra_tx = o.timeout_test ? 16u : 0u;
     stage.err = errw;
     // the wait-timeout test needs a kernel with waits: the staged one, or the
@@ -1701,7 +1698,7 @@ int schur_apply_impl(mdwf_ctx* ctx, Cfg* cfg, const double* in_dev, double* out_
   CK(cudaMemsetAsync(errw.p, 0, sizeof(int), st));
   StageInfo si;
   si.spin_bytes = si.nrm_bytes = 0;
-  si.budget = wait_budget(ctx->device, 2.0);
+  si.budget = wait_budget(ctx, 2.0);
   si.extra_tx = 0;
   si.err = errw.as<int>();
   choose_hop(op, cfg, 0, HOP_AUTO, &si);
@@ -1745,7 +1742,7 @@ int schur_batch_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const* in, do
   op.f = make_fifth<T>(cfg->act, mass);
   StageInfo si;
   si.spin_bytes = si.nrm_bytes = 0;
-  si.budget = wait_budget(ctx->device, 2.0);
+  si.budget = wait_budget(ctx, 2.0);
   si.extra_tx = 0;
   si.err = errw;
   choose_hop(op, cfg, (flags >> 8) & 0xff, flags & 0xff, &si);
@@ -1838,6 +1835,8 @@ int mdwf_create(const int dims[4], int device, mdwf_ctx** out) {
   mdwf_ctx* c = new mdwf_ctx();
   c->device = device;
   c->g = make_geom(dims);
+  int khz = 0;
+  if (cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, device) == cudaSuccess && khz > 0) c->clock_khz = khz;
   if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) { delete c; return MDWF_ERR_CUDA; }
   *out = c;
   return MDWF_OK;
