@@ -23,9 +23,12 @@
 // * the epilogues run over (unit, component) or (column, component) items of a
 //   shared-memory tile, with the coefficients folded (3 to 4 instructions per
 //   component).
-// D of one field at 16^3 x 48, L5 = 12: 6.61 -> 4.64 ms (1000 instructions per unit and
+// * three blocks of eight warps per SM (80 registers): 24 warps hide the loads and shuffles
+//   better than the 16 of an unbounded kernel (104 registers), 4.68 against 4.50 ms for D below;
+//   32 (64 registers) measured the same as 24.
+// D of one field at 16^3 x 48, L5 = 12: 6.61 -> 4.50 ms (1000 instructions per unit and
 // packing to parity fields before; 870 now, 3.3 ms of FP64); H^+ at 6 x 4 x 2 x 10, L5 = 5:
-// 138 -> 26 us; an FP64 solve at 4^3 x 8, L5 = 4: 28.0 -> 10.5 ms.
+// 138 -> 25 us; an FP64 solve at 4^3 x 8, L5 = 4: 28.0 -> 8.7 ms.
 // A unit's result depends on nothing but its inputs: every block shape, slot count
 // and mask, the decomposed lattice (halo terms) and both layouts give the same bits.
 #include "mdwf_internal.h"
@@ -156,7 +159,7 @@ __device__ __forceinline__ void column64(double* c, long st, int L, const Fifth<
 constexpr int kRow64 = 25;       // doubles between the rows of the tile (odd: lanes of one component hit all banks)
 
 template <int EPI, bool API>
-__global__ void __launch_bounds__(256) hop64_kernel(FastArgs<double, double> a, Shape64 p) {
+__global__ void __launch_bounds__(256, 3) hop64_kernel(FastArgs<double, double> a, Shape64 p) {
   extern __shared__ __align__(16) double tile[];            // [nsb L5 rt][kRow64], then the slot list
   constexpr bool kCols = (EPI == E_BAINV || EPI == E_AINVD_BD || EPI == E_AINV_SAME || EPI == E_SAME_AINV ||
                           EPI == E_AINVD_SAME);
@@ -403,7 +406,9 @@ cudaError_t launch64_one(const FastArgs<double, double>& a, cudaStream_t st) {
   const Shape64 p = shape64(a.L5, a.N, a.g.Vh);
   const int units = p.nsb * a.L5 * p.rt;
   const int warps = (units + 3) / 4;
-  const int threads = 32 * (warps > 8 ? 8 : warps);
+  // at least three warps: the epilogue's items (24 per unit) fill them where the units don't
+  // (4^3 x 8, L5 = 4: 9.1 ms per FP64 solve with one warp per block, 8.7 with three)
+  const int threads = 32 * (warps > 8 ? 8 : warps < 3 ? 3 : warps);
   const size_t smem = (size_t)units * kRow64 * sizeof(double) + sizeof(int) * (p.rt + 1);
   auto* kern = hop64_kernel<EPI, API>;
   if (smem > 48 * 1024) {
