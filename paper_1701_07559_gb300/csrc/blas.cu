@@ -210,16 +210,28 @@ __global__ void k_norm2(const S* __restrict__ v, const float* __restrict__ v_nrm
 // delta, so no update would ever come.  After stag_max iterations without an
 // update one is forced; it is followed by an FP64 re-reference and a restart of
 // the search direction (beta = 0).
+// The slot's scalars are loaded while the partial sums are (Slot).
+struct Slot {
+  int active;
+  double gamma;
+};
 template <int OP>
-__device__ __forceinline__ void cg_step(const Scal& c, int r, double v, double* out) {
+__device__ __forceinline__ Slot load_slot(const Scal& c, int r) {
+  Slot s{0, 0.0};
+  if (OP != FIN_STORE) s.active = c.active[r];
+  if (OP == FIN_ALPHA || OP == FIN_BETA) s.gamma = c.gamma[r];
+  return s;
+}
+template <int OP>
+__device__ __forceinline__ void cg_step(const Scal& c, const Slot& s, int r, double v, double* out) {
   if (OP == FIN_STORE) out[r] = v;
   if (OP == FIN_ALPHA) {
     c.qq[r] = v;
-    if (c.active[r]) c.alpha[r] = v > 0.0 ? c.gamma[r] / v : 0.0;
+    if (s.active) c.alpha[r] = v > 0.0 ? s.gamma / v : 0.0;
   }
   if (OP == FIN_RHO) {
     c.tmp[r] = v;
-    if (c.active[r]) {
+    if (s.active) {
       c.rho2[r] = v;
       if (v > c.rho2_max[r]) c.rho2_max[r] = v;
       if (v <= c.stop2[r]) { c.active[r] = 0; c.flags[r] |= FLAG_INNER_DONE; }
@@ -229,10 +241,9 @@ __device__ __forceinline__ void cg_step(const Scal& c, int r, double v, double* 
   }
   if (OP == FIN_BETA) {
     c.rr[r] = v;
-    if (c.active[r]) {
-      const double g = c.gamma[r];
-      c.beta[r] = g > 0.0 ? v / g : 0.0;
-      c.gamma_prev[r] = g;
+    if (s.active) {
+      c.beta[r] = s.gamma > 0.0 ? v / s.gamma : 0.0;
+      c.gamma_prev[r] = s.gamma;
       c.gamma[r] = v;
       c.iters[r] += 1;
       c.since[r] += 1;
@@ -258,11 +269,14 @@ __device__ __forceinline__ double block_sum256(double s, double* sh) {
 // sum_h partials[r][h] of slot r in a fixed order that depends on nsites only,
 // then the scalar step.  A cluster of kFinCluster blocks per slot: block c sums the
 // c-th contiguous chunk (thread t takes sites t, t+256, ... of it, then a fixed
-// tree), and block 0 adds the blocks' sums in rank order through distributed
-// shared memory.  Spreading a slot over several SMs matters on a part with few FP64
-// adders per SM; up to kFinSmall sites a single block is faster than the
-// cluster's two barriers (5.6 us for the cluster and 3 us for a scalar kernel after it
-// at 2048 sites; 4096 sites are 16 additions per thread).
+// tree), and block 0 adds the blocks' sums, which they put into its shared memory
+// behind one barrier.  What bounds it is latency: the barrier that shows that block 0
+// has started is taken while the partial sums load, and the slot's scalars load with them
+// (a session on 8^3 x 24: 54.2 ms with a barrier on both sides of block 0's reads and the
+// scalars loaded after it, 53.5 ms now).  Spreading a slot over several SMs
+// matters on a part with few FP64 adders per SM; up to kFinSmall sites a single block is
+// faster than the cluster's barriers (5.6 us for the cluster and 3 us for a scalar kernel
+// after it at 2048 sites; 4096 sites are 16 additions per thread).
 constexpr int kFinCluster = 8;
 constexpr long kFinSmall = 4096;
 template <int OP>
@@ -270,10 +284,12 @@ __global__ void __cluster_dims__(kFinCluster, 1, 1) __launch_bounds__(256)
     k_finalize(const double* __restrict__ partials, long nsites, Scal sc, double* __restrict__ out) {
   namespace cg = cooperative_groups;
   __shared__ double sh[8];
-  __shared__ double total;
+  __shared__ double total[kFinCluster];
   cg::cluster_group cluster = cg::this_cluster();
   const int r = blockIdx.y;
   const int c = (int)cluster.block_rank();
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  const Slot slot = load_slot<OP>(sc, r);
   const long len = (nsites + kFinCluster - 1) / kFinCluster;
   const long beg = (long)c * len;
   const long end = beg + len < nsites ? beg + len : nsites;
@@ -281,24 +297,26 @@ __global__ void __cluster_dims__(kFinCluster, 1, 1) __launch_bounds__(256)
   double s = 0.0;
   for (long k = beg + threadIdx.x; k < end; k += 256) s += p[k];
   s = block_sum256(s, sh);
-  if (threadIdx.x == 0) total = s;
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
+  if (threadIdx.x == 0) *cluster.map_shared_rank(&total[c], 0) = s;
   cluster.sync();
-  if (c == 0 && threadIdx.x == 0) {
-    double tot = 0.0;
-    for (int q = 0; q < kFinCluster; q++) tot += *cluster.map_shared_rank(&total, q);
-    cg_step<OP>(sc, r, tot, out);
+  if (c == 0 && threadIdx.x < kFinCluster) {
+    double tot = total[threadIdx.x];
+#pragma unroll
+    for (int w = kFinCluster / 2; w > 0; w >>= 1) tot += __shfl_down_sync((1u << kFinCluster) - 1, tot, w);
+    if (threadIdx.x == 0) cg_step<OP>(sc, slot, r, tot, out);
   }
-  cluster.sync();   // every block's sum stays readable until block 0 has added it
 }
 template <int OP>
 __global__ void __launch_bounds__(256) k_finalize_small(const double* __restrict__ partials, int nsites, Scal sc,
                                                         double* __restrict__ out) {
   __shared__ double sh[8];
+  const Slot slot = load_slot<OP>(sc, blockIdx.x);
   const double* p = partials + (long)blockIdx.x * nsites;
   double s = 0.0;
   for (int k = threadIdx.x; k < nsites; k += 256) s += p[k];
   s = block_sum256(s, sh);
-  if (threadIdx.x == 0) cg_step<OP>(sc, blockIdx.x, s, out);
+  if (threadIdx.x == 0) cg_step<OP>(sc, slot, blockIdx.x, s, out);
 }
 
 // u = B x on one parity: P_+ half b5 x_s + c5 x_{s-1}, P_- half b5 x_s + c5 x_{s+1},
