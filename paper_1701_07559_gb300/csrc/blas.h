@@ -8,6 +8,14 @@ namespace mdwf {
 // sizes allow it.
 Tiling blas_tiling(long Vh, int L5, int N, int max_threads);
 
+constexpr int kGroup = 4;
+// The search directions of a group.
+template <typename S>
+struct PGroup {
+  const S* v[kGroup];
+  const float* n[kGroup];
+};
+
 // Per-slot scalars of the batched CG.
 struct Scal {
   double *gamma, *gamma_prev, *alpha, *beta, *rho2, *rho2_max, *stop2, *qq, *rr, *tmp, *bhat2, *upd2;
@@ -15,6 +23,10 @@ struct Scal {
   int* since;     // CG iterations since the last reliable update of the slot
   int stag_max;   // that many without one: the inner recursion stagnates
   double delta2;  // periodic reliable update when |rho|^2 < delta2 * max |rho|^2 since the last one
+  // The iterations of a chunk run in groups of up to kGroup.  The i-th of a group (pos = i) keeps its search
+  // direction and, in alpha (the i-th row of kGroup), its step; x takes them together at the group's end.
+  int* taken;     // iterations that the slot has done in the group
+  int pos;
   double tau2;    // FP64 re-reference when |rho|^2 <= tau2 * |bhat|^2 (bhat = current reference residual)
 };
 enum { FLAG_INNER_DONE = 1, FLAG_UPDATE = 2, FLAG_DONE = 4, FLAG_REREF = 8, FLAG_STAG = 16 };
@@ -40,10 +52,12 @@ template <typename SX, typename S>
 cudaError_t axpy_x_rho(SX* x, const S* p, const float* p_nrm, S* rho, float* rho_nrm, const S* q, const float* q_nrm,
                        const double* alpha, const Tiling& t, long Vh, int L5, int N, const int* active,
                        double* partials, cudaStream_t st);
-
 template <typename S>
-cudaError_t xpay(const S* r, const float* r_nrm, S* p, float* p_nrm, const double* beta, const Tiling& t, long Vh,
-                 int L5, int N, const int* active, cudaStream_t st);
+cudaError_t axpy_rho(S* rho, float* rho_nrm, const S* q, const float* q_nrm, const double* alpha, const Tiling& t,
+                     long Vh, int L5, int N, const int* active, double* partials, cudaStream_t st);
+template <typename SX, typename S>
+cudaError_t axpy_group(SX* x, const PGroup<S>& p, int m, const double* alpha, const int* taken, const Tiling& t, long Vh,
+                       int L5, int N, cudaStream_t st);
 
 template <typename SX>
 cudaError_t accum_xhi(double* xhi, SX* xlo, const Tiling& t, long Vh, int L5, int N, const int* mask,
@@ -57,9 +71,9 @@ cudaError_t bop(const S* x, const float* x_nrm, S* u, float* u_nrm, const Fifth<
                 const Tiling& t, long Vh, int L5, int N, const int* mask, cudaStream_t st);
 
 template <typename S>
-cudaError_t xpay_b(const S* r, const float* r_nrm, S* p, float* p_nrm, S* u, float* u_nrm, const double* beta,
-                   const Fifth<typename StoreTraits<S>::T>& f, const Tiling& t, long Vh, int L5, int N,
-                   const int* active, cudaStream_t st);
+cudaError_t xpay_b(const S* r, const float* r_nrm, const S* p0, const float* p0_nrm, S* p, float* p_nrm, S* u,
+                   float* u_nrm, const double* beta, const Fifth<typename StoreTraits<S>::T>& f, const Tiling& t,
+                   long Vh, int L5, int N, const int* active, const int* taken, cudaStream_t st);
 
 template <typename S>
 cudaError_t resid_update(const double* bhat, const float* q, S* rho, float* rho_nrm, const Tiling& t, long Vh, int L5,

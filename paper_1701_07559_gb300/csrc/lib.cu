@@ -619,6 +619,10 @@ struct BatchSolver {
   F<double> b_e, b_o, x_acc, x_hi, x_o, bhat, rho64, u64, t64;
   F<float> xf, uf, tf, qf;       // FP32 reliable updates
   F<S> p, u, t, q, rho, r;       // inner vectors
+  // The search directions of a group but its last, which is p: views of the FP64 temporaries, which
+  // hold nothing during a chunk.
+  F<S> pg[kGroup - 1];
+  int group = 1;                 // iterations of a group (init)
   F<SX> xlo;
   double* part = nullptr;
   double* mass64 = nullptr;
@@ -714,18 +718,32 @@ struct BatchSolver {
     const char* nS[] = {"p", "u", "t", "q", "rho", "r"};
     for (int i = 0; i < 6; i++) CK(ws_field<S>(c, wsp + "S." + nS[i], units, fS[i]));
     CK(ws_field<SX>(c, wsp + "xlo", units, &xlo));
+    // Both give the same bits.  Where the iteration's vectors fit in the L2 an update of x per iteration
+    // costs no DRAM traffic and saves a launch (8^3 x 16, L5 = 8, fp16: 12.6 MB, 8.32 ms per solve against
+    // 8.36 in groups; FP32, 22 MB: 9.02 against 9.14); beyond it groups do (12^3 x 24, fp16, 1, 2, 4 systems:
+    // 64 MB, 24.61 against 24.63; 127 MB, 38.98 against 38.29; 255 MB, 73.5 against 71.2 ms).
+    group = (double)units * 24 * (6 * sizeof(S) + sizeof(SX)) > 120e6 ? kGroup : 1;
+    static_assert(kGroup <= 4, "a field per search direction");
+    F<double>* room[] = {&u64, &t64, &rho64};
+    for (int i = 0; i < kGroup - 1; i++) {
+      // the norms of an fp16 field come after its 48 bytes per unit
+      pg[i].v = reinterpret_cast<S*>(room[i]->v);
+      pg[i].n = p.n ? reinterpret_cast<float*>(pg[i].v + 24 * (size_t)units) : nullptr;
+    }
     part = (double*)ws_get(c, wsp + "partials", sizeof(double) * g.Vh * N, &e); CK(e);
-    double* d = (double*)ws_get(c, wsp + "scal_d", sizeof(double) * 12 * N, &e); CK(e);
-    int* ip = (int*)ws_get(c, wsp + "scal_i", sizeof(int) * 4 * N, &e); CK(e);
+    double* d = (double*)ws_get(c, wsp + "scal_d", sizeof(double) * (11 + kGroup) * N, &e); CK(e);
+    int* ip = (int*)ws_get(c, wsp + "scal_i", sizeof(int) * 5 * N, &e); CK(e);
     umask_d = (int*)ws_get(c, wsp + "umask", sizeof(int) * N, &e); CK(e);
-    sc.gamma = d; sc.gamma_prev = d + N; sc.alpha = d + 2 * N; sc.beta = d + 3 * N; sc.rho2 = d + 4 * N;
+    sc.gamma = d; sc.gamma_prev = d + N; sc.alpha = d + 11 * N; sc.beta = d + 3 * N; sc.rho2 = d + 4 * N;
     sc.rho2_max = d + 5 * N; sc.stop2 = d + 6 * N; sc.qq = d + 7 * N; sc.rr = d + 8 * N; sc.tmp = d + 9 * N;
     sc.bhat2 = d + 10 * N;
-    sc.upd2 = d + 11 * N;
+    sc.upd2 = d + 2 * N;
     sc.active = ip; sc.flags = ip + N; sc.iters = ip + 2 * N; sc.since = ip + 3 * N;
+    sc.taken = ip + 4 * N;
+    sc.pos = 0;
     sc.stag_max = 128;
-    CK(cudaMemsetAsync(d, 0, sizeof(double) * 12 * N, st));
-    CK(cudaMemsetAsync(ip, 0, sizeof(int) * 4 * N, st));
+    CK(cudaMemsetAsync(d, 0, sizeof(double) * (11 + kGroup) * N, st));
+    CK(cudaMemsetAsync(ip, 0, sizeof(int) * 5 * N, st));
     const size_t b64 = sizeof(double) * 24 * (size_t)units;
     CK(cudaMemsetAsync(x_acc.v, 0, b64, st));
     CK(cudaMemsetAsync(x_hi.v, 0, b64, st));
@@ -819,28 +837,58 @@ struct BatchSolver {
     return finalize(part, ctx->g.Vh, N, dst, op64.st);
   }
 
-  // One CG iteration on all active slots.
-  cudaError_t iteration() {
+  // Iteration i of a group of m on all active slots; the last one adds the group's steps to x.
+  cudaError_t iteration(int i, int m) {
     const Geom& g = ctx->g;
     cudaStream_t st = op64.st;
     cudaError_t e;
+    const F<S> p0 = i == 0 ? p : pg[i - 1], p1 = i == m - 1 ? p : pg[i];
+    Scal si = sc;
+    si.pos = i;
+    si.alpha = sc.alpha + (size_t)i * N;
     launches += 5;  // xpay_b, axpy, 3 reductions with the scalar steps (+ 4 hops counted in FastOp::run)
-    e = xpay_b<S>(r.v, r.n, p.v, p.n, u.v, u.n, sc.beta, opS.f, tl_blas, g.Vh, L5, N, sc.active, st);
+    e = xpay_b<S>(r.v, r.n, p0.v, p0.n, p1.v, p1.n, u.v, u.n, sc.beta, opS.f, tl_blas, g.Vh, L5, N, sc.active,
+                  i == 0 ? nullptr : sc.taken, st);
     if (e != cudaSuccess) return e;
-    e = sym ? opS.mhat_sym(p, u, t, q, sc.active, part) : opS.mhat(p, u, t, q, sc.active, part);
+    e = sym ? opS.mhat_sym(p1, u, t, q, sc.active, part) : opS.mhat(p1, u, t, q, sc.active, part);
     if (e != cudaSuccess) return e;
-    e = finalize_cg(part, g.Vh, N, sc, FIN_ALPHA, st);
+    e = finalize_cg(part, g.Vh, N, si, FIN_ALPHA, st);
     if (e != cudaSuccess) return e;
-    e = axpy_x_rho<SX, S>(xlo.v, p.v, p.n, rho.v, rho.n, q.v, q.n, sc.alpha, tl_blas, g.Vh, L5, N, sc.active, part, st);
+    if (m == 1)
+      e = axpy_x_rho<SX, S>(xlo.v, p.v, p.n, rho.v, rho.n, q.v, q.n, si.alpha, tl_blas, g.Vh, L5, N, sc.active, part, st);
+    else
+      e = axpy_rho<S>(rho.v, rho.n, q.v, q.n, si.alpha, tl_blas, g.Vh, L5, N, sc.active, part, st);
     if (e != cudaSuccess) return e;
-    e = finalize_cg(part, g.Vh, N, sc, FIN_RHO, st);
+    e = finalize_cg(part, g.Vh, N, si, FIN_RHO, st);
     if (e != cudaSuccess) return e;
     // (u = B p is dead here: the symmetric form's scratch)
     e = sym ? opS.mhat_sym_dag(rho, u, t, r, sc.active, part) : opS.mhat_dag(rho, t, r, sc.active, part);
     if (e != cudaSuccess) return e;
-    e = finalize_cg(part, g.Vh, N, sc, FIN_BETA, st);
+    e = finalize_cg(part, g.Vh, N, si, FIN_BETA, st);
     if (e != cudaSuccess) return e;
+    if (i == m - 1 && m > 1) {
+      PGroup<S> ps;
+      for (int j = 0; j < kGroup; j++) {
+        const F<S>& f = j < m - 1 ? pg[j] : p;
+        ps.v[j] = f.v;
+        ps.n[j] = f.n;
+      }
+      launches += 1;
+      e = axpy_group<SX, S>(xlo.v, ps, m, sc.alpha, sc.taken, tl_blas, g.Vh, L5, N, st);
+      if (e != cudaSuccess) return e;
+    }
     return cudaGetLastError();
+  }
+
+  cudaError_t iterations(int k) {
+    for (int b = 0; b < k; b += group) {
+      const int m = k - b < group ? k - b : group;
+      for (int i = 0; i < m; i++) {
+        cudaError_t e = iteration(i, m);
+        if (e != cudaSuccess) return e;
+      }
+    }
+    return cudaSuccess;
   }
 
   // r = Mhat^+ rho and |r|^2 for the slots in um.
@@ -924,7 +972,7 @@ struct BatchSolver {
     mdwf_ctx* ctx = this->ctx;
     cudaStream_t st = op64.st;
     if (!use_graph) {
-      for (int i = 0; i < k; i++) CK(iteration());
+      CK(iterations(k));
       return MDWF_OK;
     }
     if (graph == nullptr || graph_iters != k) {
@@ -934,8 +982,7 @@ struct BatchSolver {
       prof.gused = 0;
       prof.capturing = profiling;
       CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeRelaxed));
-      cudaError_t err = cudaSuccess;
-      for (int i = 0; i < k && err == cudaSuccess; i++) err = iteration();
+      cudaError_t err = iterations(k);
       cudaError_t e2 = cudaStreamEndCapture(st, &gr);
       prof.capturing = false;
       graph_launches = launches - c0;
