@@ -244,27 +244,53 @@ __global__ void k_norm2(const S* __restrict__ v, const float* __restrict__ v_nrm
   block_partial(n2, x, tl, L5, Vh, partials);
 }
 
-// The scalar step of a CG iteration that needs slot r's sum v.
+// The scalar steps of a CG iteration.
 //
-// FIN_RHO: the low-precision residual recursion can stagnate for a system whose
+// |rho|^2: the low-precision residual recursion can stagnate for a system whose
 // residual is already tiny: it neither reaches the stopping norm nor drops by
 // delta, so no update would ever come.  After stag_max iterations without an
 // update one is forced; it is followed by an FP64 re-reference and a restart of
 // the search direction (beta = 0).
-// The slot's scalars are loaded while the partial sums are (Slot).
+// The slot's scalars are loaded while the partial sums are.
 struct Slot {
-  int active;
-  double gamma;
+  int active, flags, since;
+  double gamma, rho2_max, stop2, bhat2;
 };
 template <int OP>
 __device__ __forceinline__ Slot load_slot(const Scal& c, int r) {
-  Slot s{0, 0.0};
-  if (OP != FIN_STORE) s.active = c.active[r];
-  if (OP == FIN_ALPHA || OP == FIN_BETA) s.gamma = c.gamma[r];
+  Slot s{};
+  if (OP != FIN_STORE) {
+    s.active = c.active[r];
+    s.gamma = c.gamma[r];
+  }
+  if (OP == FIN_RHO_BETA) {
+    s.flags = c.flags[r];
+    s.since = c.since[r];
+    s.rho2_max = c.rho2_max[r];
+    s.stop2 = c.stop2[r];
+    s.bhat2 = c.bhat2[r];
+  }
   return s;
 }
+// |rho|^2 = v: true while the slot goes on.
+__device__ __forceinline__ bool rho_step(const Scal& c, const Slot& s, int r, double v) {
+  c.tmp[r] = v;
+  if (!s.active) return false;
+  c.rho2[r] = v;
+  double top = s.rho2_max;
+  if (v > top) c.rho2_max[r] = top = v;
+  if (v <= s.stop2) {
+    c.active[r] = 0;
+    c.flags[r] = s.flags | FLAG_INNER_DONE;
+    return false;
+  }
+  if (v < c.delta2 * top || v <= c.tau2 * s.bhat2) c.flags[r] = s.flags | FLAG_UPDATE;
+  else if (s.since >= c.stag_max) c.flags[r] = s.flags | FLAG_UPDATE | FLAG_STAG;
+  return true;
+}
+// The scalar step of a CG iteration that needs slot r's sums v (and w).
 template <int OP>
-__device__ __forceinline__ void cg_step(const Scal& c, const Slot& s, int r, double v, double* out) {
+__device__ __forceinline__ void cg_step(const Scal& c, const Slot& s, int r, double v, double w, double* out) {
   if (OP == FIN_STORE) out[r] = v;
   if (OP == FIN_ALPHA) {
     c.qq[r] = v;
@@ -272,62 +298,94 @@ __device__ __forceinline__ void cg_step(const Scal& c, const Slot& s, int r, dou
     if (s.active) c.taken[r] = c.pos + 1;
     else if (c.pos == 0) c.taken[r] = 0;
   }
-  if (OP == FIN_RHO) {
-    c.tmp[r] = v;
-    if (s.active) {
-      c.rho2[r] = v;
-      if (v > c.rho2_max[r]) c.rho2_max[r] = v;
-      if (v <= c.stop2[r]) { c.active[r] = 0; c.flags[r] |= FLAG_INNER_DONE; }
-      else if (v < c.delta2 * c.rho2_max[r] || v <= c.tau2 * c.bhat2[r]) c.flags[r] |= FLAG_UPDATE;
-      else if (c.since[r] >= c.stag_max) c.flags[r] |= FLAG_UPDATE | FLAG_STAG;
-    }
-  }
-  if (OP == FIN_BETA) {
-    c.rr[r] = v;
-    if (s.active) {
-      c.beta[r] = s.gamma > 0.0 ? v / s.gamma : 0.0;
+  if (OP == FIN_RHO_BETA) {
+    // a slot that stopped on |rho|^2 keeps its search direction
+    const bool go = rho_step(c, s, r, v);
+    c.rr[r] = w;
+    if (go) {
+      c.beta[r] = s.gamma > 0.0 ? w / s.gamma : 0.0;
       c.gamma_prev[r] = s.gamma;
-      c.gamma[r] = v;
+      c.gamma[r] = w;
       c.iters[r] += 1;
-      c.since[r] += 1;
+      c.since[r] = s.since + 1;
     }
   }
 }
 
-// Sum of a block's 256 values by its first warp, in thread 0 (fixed order): an FP64 instruction costs a
-// warp 64 clocks whatever its active lanes, so the tree runs on one warp after one exchange.
-__device__ __forceinline__ double block_sum256(double s, double* sh) {
+// Sums of one or two arrays (OP) over their sites, in an order that depends on their number only.
+// Thread t adds the sites t, t + 256, ... of [beg, end): eight loads at a time, then their additions.
+template <bool TWO>
+__device__ __forceinline__ void site_sums(const double* __restrict__ p, const double* __restrict__ p2, long beg, long end,
+                                          double* s) {
+  constexpr int B = 8;
+  for (long k = beg + threadIdx.x; k < end; k += B * 256) {
+    double v[B], w[B];
 #pragma unroll
-  for (int w = 16; w > 0; w >>= 1) s += __shfl_down_sync(0xffffffffu, s, w);
-  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-  __syncthreads();
-  double t = threadIdx.x < 8 ? sh[threadIdx.x] : 0.0;
-  if (threadIdx.x < 32) {
+    for (int j = 0; j < B; j++) {
+      const bool in = k + j * 256 < end;
+      v[j] = in ? p[k + j * 256] : 0.0;
+      if (TWO) w[j] = in ? p2[k + j * 256] : 0.0;
+    }
 #pragma unroll
-    for (int w = 4; w > 0; w >>= 1) t += __shfl_down_sync(0xffffffffu, t, w);
+    for (int j = 0; j < B; j++) {
+      if (k + j * 256 >= end) break;
+      s[0] += v[j];
+      if (TWO) s[1] += w[j];
+    }
   }
-  return t;
+}
+// Tree over W lanes for each of two values: the lower and the upper W / 2 lanes take one each after the
+// first step; an FP64 instruction costs a warp 64 clocks whatever its active lanes.
+template <bool TWO, int W>
+__device__ __forceinline__ double lane_sum(double v, double w) {
+  if (TWO) {
+    const bool up = (threadIdx.x & (W / 2)) != 0;
+    const double give = up ? v : w;
+    v = (up ? w : v) + __shfl_xor_sync(0xffffffffu, give, W / 2);
+  } else {
+    v += __shfl_down_sync(0xffffffffu, v, W / 2);
+  }
+#pragma unroll
+  for (int k = W / 4; k > 0; k >>= 1) v += __shfl_down_sync(0xffffffffu, v, k);
+  return v;
+}
+// Sums of a block's 256 values by its first warp, after one exchange: of the first value in lane 0, of the
+// second in lane 8.
+template <bool TWO>
+__device__ __forceinline__ double block_sum256(const double* s, double* sh) {
+  const double t = lane_sum<TWO, 32>(s[0], TWO ? s[1] : 0.0);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) sh[warp] = t;
+  if (TWO && lane == 16) sh[8 + warp] = t;
+  __syncthreads();
+  double u = 0.0;
+  if (threadIdx.x < 32) {
+    u = lane < (TWO ? 16 : 8) ? sh[lane] : 0.0;
+#pragma unroll
+    for (int k = 4; k > 0; k >>= 1) u += __shfl_down_sync(0xffffffffu, u, k);
+  }
+  return u;
 }
 
-// sum_h partials[r][h] of slot r in a fixed order that depends on nsites only,
-// then the scalar step.  A cluster of kFinCluster blocks per slot: block c sums the
-// c-th contiguous chunk (thread t takes sites t, t+256, ... of it, then a fixed
-// tree), and block 0 adds the blocks' sums, which they put into its shared memory
-// behind one barrier.  What bounds it is latency: the barrier that shows that block 0
-// has started is taken while the partial sums load, and the slot's scalars load with them
-// (a session on 8^3 x 24: 54.2 ms with a barrier on both sides of block 0's reads and the
-// scalars loaded after it, 53.5 ms now).  Spreading a slot over several SMs
-// matters on a part with few FP64 adders per SM; up to kFinSmall sites a single block is
+// The sums of slot r over its sites, then the scalar step.  A cluster of kFinCluster
+// blocks per slot: block c sums the c-th contiguous chunk, and block 0 adds the blocks'
+// sums, which they put into its shared memory behind one barrier.  What bounds it is
+// latency: the barrier that shows that block 0 has started is taken while the partial
+// sums load, and the slot's scalars load with them (a session on 8^3 x 24: 54.2 ms with a
+// barrier on both sides of block 0's reads and the scalars loaded after it, 53.5 ms; 51.0 ms
+// with |rho|^2 and |r|^2 added up in one launch).  Spreading a slot over several SMs matters on a part with few FP64 adders per SM; up to kFinSmall sites a single block is
 // faster than the cluster's barriers (5.6 us for the cluster and 3 us for a scalar kernel
 // after it at 2048 sites; 4096 sites are 16 additions per thread).
 constexpr int kFinCluster = 8;
 constexpr long kFinSmall = 4096;
 template <int OP>
 __global__ void __cluster_dims__(kFinCluster, 1, 1) __launch_bounds__(256)
-    k_finalize(const double* __restrict__ partials, long nsites, Scal sc, double* __restrict__ out) {
+    k_finalize(const double* __restrict__ partials, const double* __restrict__ partials2, long nsites, Scal sc,
+               double* __restrict__ out) {
   namespace cg = cooperative_groups;
-  __shared__ double sh[8];
-  __shared__ double total[kFinCluster];
+  constexpr bool TWO = OP == FIN_RHO_BETA;
+  __shared__ double sh[16];
+  __shared__ double total[2 * kFinCluster];
   cg::cluster_group cluster = cg::this_cluster();
   const int r = blockIdx.y;
   const int c = (int)cluster.block_rank();
@@ -336,30 +394,36 @@ __global__ void __cluster_dims__(kFinCluster, 1, 1) __launch_bounds__(256)
   const long len = (nsites + kFinCluster - 1) / kFinCluster;
   const long beg = (long)c * len;
   const long end = beg + len < nsites ? beg + len : nsites;
-  const double* p = partials + (long)r * nsites;
-  double s = 0.0;
-  for (long k = beg + threadIdx.x; k < end; k += 256) s += p[k];
-  s = block_sum256(s, sh);
+  double s[2] = {0.0, 0.0};
+  site_sums<TWO>(partials + (long)r * nsites, partials2 + (long)r * nsites, beg, end, s);
+  const double t = block_sum256<TWO>(s, sh);
   asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-  if (threadIdx.x == 0) *cluster.map_shared_rank(&total[c], 0) = s;
+  if (threadIdx.x == 0) *cluster.map_shared_rank(&total[c], 0) = t;
+  if (TWO && threadIdx.x == 8) *cluster.map_shared_rank(&total[kFinCluster + c], 0) = t;
   cluster.sync();
-  if (c == 0 && threadIdx.x < kFinCluster) {
-    double tot = total[threadIdx.x];
+  if (c == 0 && threadIdx.x < 32) {
+    double tot = threadIdx.x < (TWO ? 2 : 1) * kFinCluster ? total[threadIdx.x] : 0.0;
 #pragma unroll
-    for (int w = kFinCluster / 2; w > 0; w >>= 1) tot += __shfl_down_sync((1u << kFinCluster) - 1, tot, w);
-    if (threadIdx.x == 0) cg_step<OP>(sc, slot, r, tot, out);
+    for (int w = kFinCluster / 2; w > 0; w >>= 1) tot += __shfl_down_sync(0xffffffffu, tot, w);
+    const double second = __shfl_sync(0xffffffffu, tot, kFinCluster);
+    if (threadIdx.x == 0) cg_step<OP>(sc, slot, r, tot, second, out);
   }
 }
 template <int OP>
-__global__ void __launch_bounds__(256) k_finalize_small(const double* __restrict__ partials, int nsites, Scal sc,
+__global__ void __launch_bounds__(256) k_finalize_small(const double* __restrict__ partials,
+                                                        const double* __restrict__ partials2, int nsites, Scal sc,
                                                         double* __restrict__ out) {
-  __shared__ double sh[8];
-  const Slot slot = load_slot<OP>(sc, blockIdx.x);
-  const double* p = partials + (long)blockIdx.x * nsites;
-  double s = 0.0;
-  for (int k = threadIdx.x; k < nsites; k += 256) s += p[k];
-  s = block_sum256(s, sh);
-  if (threadIdx.x == 0) cg_step<OP>(sc, slot, blockIdx.x, s, out);
+  constexpr bool TWO = OP == FIN_RHO_BETA;
+  __shared__ double sh[16];
+  const int r = blockIdx.x;
+  const Slot slot = load_slot<OP>(sc, r);
+  double s[2] = {0.0, 0.0};
+  site_sums<TWO>(partials + (long)r * nsites, partials2 + (long)r * nsites, 0, nsites, s);
+  const double t = block_sum256<TWO>(s, sh);
+  if (threadIdx.x < 32) {
+    const double second = __shfl_sync(0xffffffffu, t, 8);
+    if (threadIdx.x == 0) cg_step<OP>(sc, slot, r, t, second, out);
+  }
 }
 
 // u = B x on one parity: P_+ half b5 x_s + c5 x_{s-1}, P_- half b5 x_s + c5 x_{s+1},
@@ -604,21 +668,21 @@ cudaError_t z2_source(unsigned long long seed, double* eta, long V, cudaStream_t
 }
 
 template <int OP>
-static cudaError_t finalize_one(const double* partials, long nsites, int N, const Scal& c, double* out, cudaStream_t st) {
-  if (nsites <= kFinSmall) k_finalize_small<OP><<<N, 256, 0, st>>>(partials, (int)nsites, c, out);
-  else k_finalize<OP><<<dim3(kFinCluster, (unsigned)N), 256, 0, st>>>(partials, nsites, c, out);
+static cudaError_t finalize_one(const double* partials, const double* partials2, long nsites, int N, const Scal& c,
+                                double* out, cudaStream_t st) {
+  if (nsites <= kFinSmall) k_finalize_small<OP><<<N, 256, 0, st>>>(partials, partials2, (int)nsites, c, out);
+  else k_finalize<OP><<<dim3(kFinCluster, (unsigned)N), 256, 0, st>>>(partials, partials2, nsites, c, out);
   return cudaGetLastError();
 }
 cudaError_t finalize(const double* partials, long ntiles, int N, double* out, cudaStream_t st) {
-  return finalize_one<FIN_STORE>(partials, ntiles, N, Scal(), out, st);
+  return finalize_one<FIN_STORE>(partials, partials, ntiles, N, Scal(), out, st);
 }
-cudaError_t finalize_cg(const double* partials, long nsites, int N, const Scal& c, FinOp op, cudaStream_t st) {
-  switch (op) {
-    case FIN_ALPHA: return finalize_one<FIN_ALPHA>(partials, nsites, N, c, nullptr, st);
-    case FIN_RHO: return finalize_one<FIN_RHO>(partials, nsites, N, c, nullptr, st);
-    case FIN_BETA: return finalize_one<FIN_BETA>(partials, nsites, N, c, nullptr, st);
-    default: return cudaErrorInvalidValue;
-  }
+cudaError_t finalize_alpha(const double* qq, long nsites, int N, const Scal& c, cudaStream_t st) {
+  return finalize_one<FIN_ALPHA>(qq, qq, nsites, N, c, nullptr, st);
+}
+cudaError_t finalize_rho_beta(const double* rho2, const double* rr, long nsites, int N, const Scal& c,
+                              cudaStream_t st) {
+  return finalize_one<FIN_RHO_BETA>(rho2, rr, nsites, N, c, nullptr, st);
 }
 
 Tiling blas_tiling(long Vh, int L5, int N, int max_threads) {

@@ -30,10 +30,12 @@ struct Scal {
   double tau2;    // FP64 re-reference when |rho|^2 <= tau2 * |bhat|^2 (bhat = current reference residual)
 };
 enum { FLAG_INNER_DONE = 1, FLAG_UPDATE = 2, FLAG_DONE = 4, FLAG_REREF = 8, FLAG_STAG = 16 };
-// The reductions of a CG iteration, each with the scalar step it feeds: |q|^2 and alpha, |rho|^2 and the
-// stopping and update decisions, |r|^2 and beta.
-enum FinOp { FIN_STORE = 0, FIN_ALPHA = 1, FIN_RHO = 2, FIN_BETA = 3 };
-cudaError_t finalize_cg(const double* partials, long nsites, int N, const Scal& c, FinOp op, cudaStream_t st);
+// The reductions of a CG iteration with the scalar steps that they feed: |q|^2 and alpha; |rho|^2 with the
+// stopping and update decisions, and |r|^2 with beta, in one launch.
+enum FinOp { FIN_STORE = 0, FIN_ALPHA = 1, FIN_RHO_BETA = 2 };
+cudaError_t finalize_alpha(const double* qq, long nsites, int N, const Scal& c, cudaStream_t st);
+cudaError_t finalize_rho_beta(const double* rho2, const double* rr, long nsites, int N, const Scal& c,
+                              cudaStream_t st);
 
 // API layout (one field per RHS, [s][t][z][y][x][spin][colour][re,im], FP64, device) <-> slots r0 .. r0 + nr - 1
 // of a parity field; api: nr device pointers (host array).  unpack_rhs with in == null writes zeros.

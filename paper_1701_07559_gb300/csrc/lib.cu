@@ -344,7 +344,7 @@ Tiling tiling_for(const Geom& g, int L5, int N, int nsb, bool two_buffers) {
 
 // ---------------------------------------------------------------------------
 // Scalar kernels of the reliable updates (one thread per RHS slot); those of the
-// CG iteration run at the end of its reductions (finalize_cg, blas.cu)
+// CG iteration run at the end of its reductions (cg_step, blas.cu)
 // ---------------------------------------------------------------------------
 // After a residual recomputed with FP32 arithmetic.  Its error grows like
 // 1e-7 kappa(Mhat) |bhat| (x_hi, accumulated since the last re-reference, is
@@ -624,7 +624,8 @@ struct BatchSolver {
   F<S> pg[kGroup - 1];
   int group = 1;                 // iterations of a group (init)
   F<SX> xlo;
-  double* part = nullptr;
+  double* part = nullptr;         // partial sums of a reduction
+  double* part2 = nullptr;        // of |rho|^2, which are added up with those of |r|^2
   double* mass64 = nullptr;
   float* mass32 = nullptr;
   Scal sc;
@@ -731,6 +732,7 @@ struct BatchSolver {
       pg[i].n = p.n ? reinterpret_cast<float*>(pg[i].v + 24 * (size_t)units) : nullptr;
     }
     part = (double*)ws_get(c, wsp + "partials", sizeof(double) * g.Vh * N, &e); CK(e);
+    part2 = (double*)ws_get(c, wsp + "partials2", sizeof(double) * g.Vh * N, &e); CK(e);
     double* d = (double*)ws_get(c, wsp + "scal_d", sizeof(double) * (11 + kGroup) * N, &e); CK(e);
     int* ip = (int*)ws_get(c, wsp + "scal_i", sizeof(int) * 5 * N, &e); CK(e);
     umask_d = (int*)ws_get(c, wsp + "umask", sizeof(int) * N, &e); CK(e);
@@ -846,25 +848,23 @@ struct BatchSolver {
     Scal si = sc;
     si.pos = i;
     si.alpha = sc.alpha + (size_t)i * N;
-    launches += 5;  // xpay_b, axpy, 3 reductions with the scalar steps (+ 4 hops counted in FastOp::run)
+    launches += 4;  // xpay_b, axpy, 2 reductions with the scalar steps (+ 4 hops counted in FastOp::run)
     e = xpay_b<S>(r.v, r.n, p0.v, p0.n, p1.v, p1.n, u.v, u.n, sc.beta, opS.f, tl_blas, g.Vh, L5, N, sc.active,
                   i == 0 ? nullptr : sc.taken, st);
     if (e != cudaSuccess) return e;
     e = sym ? opS.mhat_sym(p1, u, t, q, sc.active, part) : opS.mhat(p1, u, t, q, sc.active, part);
     if (e != cudaSuccess) return e;
-    e = finalize_cg(part, g.Vh, N, si, FIN_ALPHA, st);
+    e = finalize_alpha(part, g.Vh, N, si, st);
     if (e != cudaSuccess) return e;
     if (m == 1)
-      e = axpy_x_rho<SX, S>(xlo.v, p.v, p.n, rho.v, rho.n, q.v, q.n, si.alpha, tl_blas, g.Vh, L5, N, sc.active, part, st);
+      e = axpy_x_rho<SX, S>(xlo.v, p.v, p.n, rho.v, rho.n, q.v, q.n, si.alpha, tl_blas, g.Vh, L5, N, sc.active, part2, st);
     else
-      e = axpy_rho<S>(rho.v, rho.n, q.v, q.n, si.alpha, tl_blas, g.Vh, L5, N, sc.active, part, st);
-    if (e != cudaSuccess) return e;
-    e = finalize_cg(part, g.Vh, N, si, FIN_RHO, st);
+      e = axpy_rho<S>(rho.v, rho.n, q.v, q.n, si.alpha, tl_blas, g.Vh, L5, N, sc.active, part2, st);
     if (e != cudaSuccess) return e;
     // (u = B p is dead here: the symmetric form's scratch)
     e = sym ? opS.mhat_sym_dag(rho, u, t, r, sc.active, part) : opS.mhat_dag(rho, t, r, sc.active, part);
     if (e != cudaSuccess) return e;
-    e = finalize_cg(part, g.Vh, N, si, FIN_BETA, st);
+    e = finalize_rho_beta(part2, part, g.Vh, N, si, st);
     if (e != cudaSuccess) return e;
     if (i == m - 1 && m > 1) {
       PGroup<S> ps;
