@@ -496,6 +496,137 @@ __global__ void k_xpay_b(const S* __restrict__ r, const float* __restrict__ r_nr
   store24<S, T>(uv, u_nrm, pl, x.u, y);
 }
 
+// FP64 forms of the two updates.  A warp's FP64 instruction takes 64 clocks, so a thread that walks
+// through the 24 components of its unit spends 3 us on them alone, with most schedulers idle on a small
+// lattice.  Four lanes per unit with three of its 12 words each; a quarter warp reads eight consecutive units of
+// one plane.  The sum of a unit (two steps of shuffles) and of a site do not depend on the other slots.
+// 4^3 x 8, L5 = 4, one system:
+// 8.45 ms per solve with a thread per unit, 7.84 with these; 8^3 x 16, L5 = 8, one to four systems: the same.
+struct Item64 {
+  Unit x;
+  int ul;        // unit of the tile
+  bool in;       // of the tile and of the lattice
+};
+__device__ __forceinline__ Item64 item64(const Tiling& tl, int ul, long Vh, int L5, int N) {
+  Item64 i;
+  i.ul = ul;
+  Unit& x = i.x;
+  x.r_l = ul % tl.rt;
+  x.s = (ul / tl.rt) % L5;
+  x.site_l = ul / (tl.rt * L5);
+  x.h = (long)blockIdx.x * tl.nsb + x.site_l;
+  x.r = blockIdx.y * tl.rt + x.r_l;
+  i.in = ul < tl.threads && x.h < Vh && x.r < N;
+  x.u = (x.h * L5 + x.s) * N + x.r;
+  return i;
+}
+constexpr int kMax64 = 512;      // threads; larger tiles take several passes
+
+// rho -= alpha_r q, |rho|^2; X: x += alpha_r p too.
+template <bool X>
+__global__ void __launch_bounds__(kMax64)
+    k_axpy64(double2* __restrict__ xv, const double2* __restrict__ p, double2* __restrict__ rho,
+             const double2* __restrict__ q, const double* __restrict__ alpha, Tiling tl, long Vh, int L5, int N,
+             const int* __restrict__ active, double* __restrict__ partials) {
+  extern __shared__ double sunit[];
+  const long pl = Vh * L5 * N;
+  const int lane = threadIdx.x & 31, w0 = lane >> 3;
+  for (int base = (threadIdx.x >> 5) * 8; base < tl.threads; base += blockDim.x / 4) {
+    const Item64 it = item64(tl, base + (lane & 7), Vh, L5, N);
+    double n2 = 0.0;
+    if (it.in && active[it.x.r]) {
+      const double a = alpha[it.x.r];
+      double2 qv[3], rv[3], pv[3], xs[3];
+#pragma unroll
+      for (int j = 0; j < 3; j++) {
+        const long o = (w0 + 4 * j) * pl + it.x.u;
+        qv[j] = __ldg(q + o);
+        rv[j] = rho[o];
+        if (X) {
+          pv[j] = __ldg(p + o);
+          xs[j] = xv[o];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 3; j++) {
+        const long o = (w0 + 4 * j) * pl + it.x.u;
+        rv[j].x = __fma_rn(-a, qv[j].x, rv[j].x);
+        rv[j].y = __fma_rn(-a, qv[j].y, rv[j].y);
+        n2 = __fma_rn(rv[j].x, rv[j].x, n2);
+        n2 = __fma_rn(rv[j].y, rv[j].y, n2);
+        rho[o] = rv[j];
+        if (X) {
+          xs[j].x = __fma_rn(a, pv[j].x, xs[j].x);
+          xs[j].y = __fma_rn(a, pv[j].y, xs[j].y);
+          xv[o] = xs[j];
+        }
+      }
+    }
+    n2 += __shfl_xor_sync(0xffffffffu, n2, 8);
+    n2 += __shfl_xor_sync(0xffffffffu, n2, 16);
+    if (w0 == 0 && it.ul < tl.threads) sunit[it.ul] = n2;
+  }
+  __syncthreads();
+  for (int k = threadIdx.x; k < tl.nsb * tl.rt; k += blockDim.x) {
+    const int site_l = k / tl.rt, r_l = k - site_l * tl.rt;
+    const long h = (long)blockIdx.x * tl.nsb + site_l;
+    const int r = blockIdx.y * tl.rt + r_l;
+    if (h >= Vh || r >= N) continue;
+    double sum = 0.0;
+    for (int s = 0; s < L5; s++) sum += sunit[(site_l * L5 + s) * tl.rt + r_l];
+    partials[(long)r * Vh + h] = sum;
+  }
+}
+
+// k_xpay_b in FP64.
+__global__ void __launch_bounds__(kMax64)
+    k_xpay64(const double2* __restrict__ r, const double2* p0, double2* p, double2* __restrict__ uv,
+             const double* __restrict__ beta, Fifth<double> f, Tiling tl, long Vh, int L5, int N,
+             const int* __restrict__ active, const int* __restrict__ taken) {
+  extern __shared__ __align__(16) double2 sP2[];      // [word][unit of the tile]
+  const long pl = Vh * L5 * N;
+  const int lane = threadIdx.x & 31, w0 = lane >> 3, nu = tl.threads;
+  for (int base = (threadIdx.x >> 5) * 8; base < nu; base += blockDim.x / 4) {
+    const Item64 it = item64(tl, base + (lane & 7), Vh, L5, N);
+    if (!it.in) continue;
+    const bool act = active[it.x.r];
+    if (!act && !(taken != nullptr && taken[it.x.r] > 0)) continue;
+    const double b = beta[it.x.r];
+    double2 pv[3], rv[3];
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+      const long o = (w0 + 4 * j) * pl + it.x.u;
+      pv[j] = p0[o];
+      if (act) rv[j] = __ldg(r + o);
+    }
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+      if (act) {
+        pv[j].x = __fma_rn(b, pv[j].x, rv[j].x);
+        pv[j].y = __fma_rn(b, pv[j].y, rv[j].y);
+      }
+      p[(w0 + 4 * j) * pl + it.x.u] = pv[j];
+      sP2[(w0 + 4 * j) * nu + it.ul] = pv[j];
+    }
+  }
+  __syncthreads();
+  for (int base = (threadIdx.x >> 5) * 8; base < nu; base += blockDim.x / 4) {
+    const Item64 it = item64(tl, base + (lane & 7), Vh, L5, N);
+    if (!it.in || !active[it.x.r]) continue;
+    const int s = it.x.s;
+    const double m = f.mass[it.x.r];
+    const int dn = it.ul + ((s == 0 ? L5 : 0) - 1) * tl.rt, up = it.ul + (1 - (s == L5 - 1 ? L5 : 0)) * tl.rt;
+    const double c_dn = f.c5 * (s == 0 ? -m : 1.0), c_up = f.c5 * (s == L5 - 1 ? -m : 1.0);
+#pragma unroll
+    for (int j = 0; j < 3; j++) {
+      const int w = w0 + 4 * j;
+      const double c = w < 6 ? c_dn : c_up;
+      const double2 a = sP2[w * nu + it.ul], b = sP2[w * nu + (w < 6 ? dn : up)];
+      uv[w * pl + it.x.u] = make_double2(__fma_rn(f.b5, a.x, c * b.x), __fma_rn(f.b5, a.y, c * b.y));
+    }
+  }
+}
+
 // Zero the units of the slots in mask.
 template <typename S>
 __global__ void k_zero_masked(S* __restrict__ v, float* __restrict__ nrm, Tiling tl, long Vh, int L5, int N,
@@ -589,20 +720,50 @@ cudaError_t convert(const Si* in, const float* in_nrm, So* out, float* out_nrm, 
   return cudaGetLastError();
 }
 
+// Tile and block of the FP64 forms.
+static Tiling tiling64(long Vh, int L5, int N, int* threads) {
+  const Tiling t = blas_tiling(Vh, L5, N, kMax64, 4);
+  const int n = (t.threads + 7) / 8 * 32;
+  *threads = n < kMax64 ? n : kMax64;
+  return t;
+}
+static cudaError_t room64(const void* kern, size_t smem) {
+  return smem <= 48 * 1024 ? cudaSuccess
+                           : cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+template <bool X>
+static cudaError_t axpy64(double* x, const double* p, double* rho, const double* q, const double* alpha, long Vh, int L5,
+                          int N, const int* active, double* partials, cudaStream_t st) {
+  int threads;
+  const Tiling t = tiling64(Vh, L5, N, &threads);
+  k_axpy64<X><<<tile_grid(t), threads, sizeof(double) * t.threads, st>>>(
+      reinterpret_cast<double2*>(x), reinterpret_cast<const double2*>(p), reinterpret_cast<double2*>(rho),
+      reinterpret_cast<const double2*>(q), alpha, t, Vh, L5, N, active, partials);
+  return cudaGetLastError();
+}
+
 template <typename SX, typename S>
 cudaError_t axpy_x_rho(SX* x, const S* p, const float* p_nrm, S* rho, float* rho_nrm, const S* q, const float* q_nrm,
                        const double* alpha, const Tiling& t, long Vh, int L5, int N, const int* active,
                        double* partials, cudaStream_t st) {
-  k_axpy_x_rho<SX, S><<<tile_grid(t), t.threads, 0, st>>>(x, p, p_nrm, rho, rho_nrm, q, q_nrm, alpha, t, Vh, L5, N,
-                                                           active, partials);
-  return cudaGetLastError();
+  if constexpr (std::is_same<S, double>::value) {
+    return axpy64<true>(x, p, rho, q, alpha, Vh, L5, N, active, partials, st);
+  } else {
+    k_axpy_x_rho<SX, S><<<tile_grid(t), t.threads, 0, st>>>(x, p, p_nrm, rho, rho_nrm, q, q_nrm, alpha, t, Vh, L5, N,
+                                                             active, partials);
+    return cudaGetLastError();
+  }
 }
 
 template <typename S>
 cudaError_t axpy_rho(S* rho, float* rho_nrm, const S* q, const float* q_nrm, const double* alpha, const Tiling& t,
                      long Vh, int L5, int N, const int* active, double* partials, cudaStream_t st) {
-  k_axpy_rho<S><<<tile_grid(t), t.threads, 0, st>>>(rho, rho_nrm, q, q_nrm, alpha, t, Vh, L5, N, active, partials);
-  return cudaGetLastError();
+  if constexpr (std::is_same<S, double>::value) {
+    return axpy64<false>(nullptr, nullptr, rho, q, alpha, Vh, L5, N, active, partials, st);
+  } else {
+    k_axpy_rho<S><<<tile_grid(t), t.threads, 0, st>>>(rho, rho_nrm, q, q_nrm, alpha, t, Vh, L5, N, active, partials);
+    return cudaGetLastError();
+  }
 }
 
 template <typename SX, typename S>
@@ -637,15 +798,27 @@ template <typename S>
 cudaError_t xpay_b(const S* r, const float* r_nrm, const S* p0, const float* p0_nrm, S* p, float* p_nrm, S* u,
                    float* u_nrm, const double* beta, const Fifth<typename StoreTraits<S>::T>& f, const Tiling& t,
                    long Vh, int L5, int N, const int* active, const int* taken, cudaStream_t st) {
-  using T = typename StoreTraits<S>::T;
-  size_t smem = (size_t)t.threads * 25 * sizeof(T);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_xpay_b<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if constexpr (std::is_same<S, double>::value) {
+    int threads;
+    const Tiling t4 = tiling64(Vh, L5, N, &threads);
+    const size_t smem = sizeof(double2) * 12 * (size_t)t4.threads;
+    cudaError_t e = room64((const void*)k_xpay64, smem);
     if (e != cudaSuccess) return e;
+    k_xpay64<<<tile_grid(t4), threads, smem, st>>>(
+        reinterpret_cast<const double2*>(r), reinterpret_cast<const double2*>(p0), reinterpret_cast<double2*>(p),
+        reinterpret_cast<double2*>(u), beta, f, t4, Vh, L5, N, active, taken);
+    return cudaGetLastError();
+  } else {
+    using T = typename StoreTraits<S>::T;
+    size_t smem = (size_t)t.threads * 25 * sizeof(T);
+    if (smem > 48 * 1024) {
+      cudaError_t e = cudaFuncSetAttribute(k_xpay_b<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (e != cudaSuccess) return e;
+    }
+    k_xpay_b<S><<<tile_grid(t), t.threads, smem, st>>>(r, r_nrm, p0, p0_nrm, p, p_nrm, u, u_nrm, beta, f, t, Vh, L5, N, active,
+                                                      taken);
+    return cudaGetLastError();
   }
-  k_xpay_b<S><<<tile_grid(t), t.threads, smem, st>>>(r, r_nrm, p0, p0_nrm, p, p_nrm, u, u_nrm, beta, f, t, Vh, L5, N, active,
-                                                    taken);
-  return cudaGetLastError();
 }
 
 template <typename S>
@@ -685,22 +858,24 @@ cudaError_t finalize_rho_beta(const double* rho2, const double* rr, long nsites,
   return finalize_one<FIN_RHO_BETA>(rho2, rr, nsites, N, c, nullptr, st);
 }
 
-Tiling blas_tiling(long Vh, int L5, int N, int max_threads) {
+Tiling blas_tiling(long Vh, int L5, int N, int max_units, int lanes) {
   // the threads wanted: 256, fewer on lattices that would leave SMs without a block
   const long units = Vh * L5 * N;
+  const long hi = 256 / lanes, lo = 32 / lanes;
   long want = units / 152;
-  want = want > 256 ? 256 : want < 32 ? 32 : want;
+  want = want > hi ? hi : want < lo ? lo : want;
   // the number of sites per block with the best-filled warps among those near that size
   int best = 1;
   double score = -1.0;
-  for (int nsb = 1; nsb <= 64 && nsb * L5 <= max_threads; nsb++) {
-    const Tiling t = make_tiling(Vh, L5, N, nsb, max_threads);
+  for (int nsb = 1; nsb <= 64 && nsb * L5 <= max_units; nsb++) {
+    const Tiling t = make_tiling(Vh, L5, N, nsb, max_units);
     if (nsb > 1 && (t.ngroups > 1 || t.threads > 1.5 * want)) break;
-    const double fill = (double)t.threads / ((t.threads + 31) / 32 * 32);
+    const int n = t.threads * lanes;
+    const double fill = (double)n / ((n + 31) / 32 * 32);
     const double size = t.threads < want ? (double)t.threads / want : 1.0;
     if (fill * size > score + 1e-9) { score = fill * size; best = nsb; }
   }
-  return make_tiling(Vh, L5, N, best, max_threads);
+  return make_tiling(Vh, L5, N, best, max_units);
 }
 
 #define MDWF_INST_S(S)                                                                                          \

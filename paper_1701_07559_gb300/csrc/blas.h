@@ -6,7 +6,8 @@ namespace mdwf {
 
 // Tiling of the unit-wise kernels: whole sites per block, 32 to 256 threads in full warps where the
 // sizes allow it.
-Tiling blas_tiling(long Vh, int L5, int N, int max_threads);
+// lanes: threads per unit.
+Tiling blas_tiling(long Vh, int L5, int N, int max_units, int lanes = 1);
 
 constexpr int kGroup = 4;
 // The search directions of a group.
