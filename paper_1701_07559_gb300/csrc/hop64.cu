@@ -435,6 +435,22 @@ __global__ void __launch_bounds__(256) k_bop_api(const double* __restrict__ x, d
   u[(long)s * n + i] = bop_term(b5, x[(long)s * n + i], cw, x[(long)sn * n + i]);
 }
 
+// A column (one component of one site, all slices) per thread, read once into shared memory.
+constexpr int kLocal5 = 128;
+__global__ void __launch_bounds__(kLocal5) k_local5_api(const double* __restrict__ in, double* __restrict__ out,
+                                                        const double* __restrict__ G, long n, int L5) {
+  extern __shared__ double col[];      // [slice][thread]
+  const long i = (long)blockIdx.x * kLocal5 + threadIdx.x;
+  if (i >= n) return;
+  for (int s = 0; s < L5; s++) col[s * kLocal5 + threadIdx.x] = in[(long)s * n + i];
+  const double* M = G + (i % 24 < 12 ? 0 : L5 * L5);
+  for (int s = 0; s < L5; s++) {
+    double o = 0.0;
+    for (int k = 0; k < L5; k++) o = __fma_rn(__ldg(M + s * L5 + k), col[k * kLocal5 + threadIdx.x], o);
+    out[(long)s * n + i] = o;
+  }
+}
+
 }  // namespace
 
 cudaError_t launch_hop64(const FastArgs<double, double>& a, int epi, cudaStream_t st) {
@@ -466,6 +482,13 @@ cudaError_t launch_hop64_api(const FastArgs<double, double>& a, int epi, cudaStr
 cudaError_t bop_api(const double* x, double* u, long V, int L5, double b5, double c5, double m, cudaStream_t st) {
   const long n = 24 * V;
   k_bop_api<<<dim3((unsigned)((n + 255) / 256), (unsigned)L5), 256, 0, st>>>(x, u, n, L5, b5, c5, m);
+  return cudaGetLastError();
+}
+
+cudaError_t local5_api(const double* in, double* out, const double* G, long V, int L5, cudaStream_t st) {
+  const long n = 24 * V;
+  const size_t smem = sizeof(double) * kLocal5 * L5;
+  k_local5_api<<<(unsigned)((n + kLocal5 - 1) / kLocal5), kLocal5, smem, st>>>(in, out, G, n, L5);
   return cudaGetLastError();
 }
 

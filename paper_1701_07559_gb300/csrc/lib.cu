@@ -126,7 +126,7 @@ bool all_finite(const double* v, size_t n) {
 //   (A^-1)_{s s'} = (-kappa)^k sigma / (alpha (1 + m (-kappa)^L5)),
 // k = number of shift steps from s' to s (mod L5), sigma = -m if the path
 // crosses the wall and 1 otherwise.
-enum MatKind { MK_A, MK_Ad, MK_B, MK_Bd, MK_Ainv, MK_Ainvd, MK_BAinv, MK_AinvdBd, MK_negA, MK_COUNT };
+enum MatKind { MK_A, MK_Ad, MK_B, MK_Bd, MK_Ainv, MK_Ainvd, MK_COUNT };
 
 using Mat = std::vector<double>;
 
@@ -136,15 +136,6 @@ Mat mat_T(const Mat& a, int n) {
   Mat t = mat_zero(n);
   for (int i = 0; i < n; i++) for (int j = 0; j < n; j++) t[(size_t)j * n + i] = a[(size_t)i * n + j];
   return t;
-}
-Mat mat_mul(const Mat& a, const Mat& b, int n) {
-  Mat c = mat_zero(n);
-  for (int i = 0; i < n; i++)
-    for (int k = 0; k < n; k++) {
-      double aik = a[(size_t)i * n + k];
-      for (int j = 0; j < n; j++) c[(size_t)i * n + j] += aik * b[(size_t)k * n + j];
-    }
-  return c;
 }
 Mat mat_lin(double x, const Mat& a, double y, const Mat& b) {
   Mat c(a.size());
@@ -194,35 +185,11 @@ struct Tables {
         Mat A = mat_lin(alpha, I, beta, P);
         Mat B = mat_lin(act.b5, I, act.c5, P);
         Mat Ai = mat_ainv(L5, alpha, beta, masses[r], chi);
-        Mat all[MK_COUNT] = {A, mat_T(A, L5), B, mat_T(B, L5), Ai, mat_T(Ai, L5),
-                             mat_mul(B, Ai, L5), mat_mul(mat_T(Ai, L5), mat_T(B, L5), L5), mat_lin(-1.0, A, 0.0, A)};
+        Mat all[MK_COUNT] = {A, mat_T(A, L5), B, mat_T(B, L5), Ai, mat_T(Ai, L5)};
         for (int k = 0; k < MK_COUNT; k++)
           std::memcpy(&h[k * block() + ((size_t)r * 2 + chi) * L5 * L5], all[k].data(), sizeof(double) * L5 * L5);
       }
   }
-};
-
-// Device copies of the tables in T precision.
-template <typename T>
-struct DevTables {
-  DBuf buf;
-  T* ext = nullptr;     // a buffer of the context's workspace instead of buf (no allocation per call)
-  size_t blk = 0;
-  cudaError_t upload(const Tables& t, cudaStream_t st, T* into = nullptr) {
-    blk = t.block();
-    std::vector<T> v(t.h.size());
-    for (size_t i = 0; i < v.size(); i++) v[i] = (T)t.h[i];
-    ext = into;
-    if (!ext) {
-      cudaError_t e = buf.alloc(sizeof(T) * v.size());
-      if (e != cudaSuccess) return e;
-    }
-    cudaError_t e = cudaMemcpyAsync(base(), v.data(), sizeof(T) * v.size(), cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return e;
-    return cudaStreamSynchronize(st);
-  }
-  T* base() const { return ext ? ext : buf.as<T>(); }
-  const T* operator[](int k) const { return base() + (size_t)k * blk; }
 };
 
 // ---------------------------------------------------------------------------
@@ -284,63 +251,6 @@ struct Prof {
   cudaError_t collect() { cudaError_t e = sum(pool, used); used = 0; return e; }   // after a sync
   cudaError_t collect_graph() { return sum(gpool, gused); }                        // after a graph launch + sync
 };
-
-template <typename S, typename T>
-struct Op {
-  Geom g;
-  int L5 = 0, N = 0, anti = 1;
-  const T* U = nullptr;
-  Tiling tl;
-  cudaStream_t st = nullptr;
-  Prof* prof = nullptr;          // time hop launches when set
-  long long* launches = nullptr; // count launches when set
-
-  // out = add + G same + kappa C H(in)   (hop) ; out = add + G in (local)
-  cudaError_t run(bool hop, int out_par, int dagger, F<S> in, F<S> same, const T* G, F<S> add, const T* C, T kappa,
-                  F<S> out, const int* active, double* partials) const {
-    HopArgs<S, T> a;
-    a.g = g; a.L5 = L5; a.N = N; a.out_par = out_par; a.dagger = dagger; a.antiperiodic = anti;
-    a.in = in.v; a.in_nrm = in.n; a.same = same.v; a.same_nrm = same.n; a.add = add.v; a.add_nrm = add.n;
-    a.out = out.v; a.out_nrm = out.n; a.U = U; a.Gm = G; a.Cm = C; a.kappa = kappa; a.active = active;
-    a.partials = partials;
-    if (launches) *launches += 1;
-    if (prof && hop) {
-      cudaError_t e = prof->record(st);
-      if (e != cudaSuccess) return e;
-      e = launch_hop<S, T>(a, tl, hop, st);
-      if (e != cudaSuccess) return e;
-      return prof->record(st);
-    }
-    return launch_hop<S, T>(a, tl, hop, st);
-  }
-  // q = Mhat p (dagger 0) or Mhat^+ p (dagger 1) on even sites; u, t scratch (even, odd).
-  cudaError_t schur(int dagger, F<S> p, F<S> u, F<S> t, F<S> q, const DevTables<T>& M, const int* active,
-                    double* partials) const {
-    F<S> none;
-    cudaError_t e;
-    if (!dagger) {
-      e = run(false, 0, 0, p, none, M[MK_B], none, nullptr, T(0), u, active, nullptr);
-      if (e != cudaSuccess) return e;
-      e = run(true, 1, 0, u, none, nullptr, none, M[MK_BAinv], T(1), t, active, nullptr);
-      if (e != cudaSuccess) return e;
-      return run(true, 0, 0, t, p, M[MK_A], none, nullptr, T(-0.25), q, active, partials);
-    }
-    e = run(true, 1, 1, p, none, nullptr, none, M[MK_AinvdBd], T(1), t, active, nullptr);
-    if (e != cudaSuccess) return e;
-    return run(true, 0, 1, t, p, M[MK_Ad], none, M[MK_Bd], T(-0.25), q, active, partials);
-  }
-};
-
-template <typename S>
-Tiling tiling_for(const Geom& g, int L5, int N, int nsb, bool two_buffers) {
-  using T = typename StoreTraits<S>::T;
-  int maxthr = hop_max_threads<S, T>();
-  int smem_thr = (int)(200 * 1024 / ((two_buffers ? 2 : 1) * 25 * sizeof(T)));
-  if (smem_thr < maxthr) maxthr = smem_thr;
-  if (maxthr > 1024) maxthr = 1024;
-  if (nsb * L5 > maxthr) nsb = maxthr / L5 > 0 ? maxthr / L5 : 1;
-  return make_tiling(g.Vh, L5, N, nsb, maxthr);
-}
 
 // ---------------------------------------------------------------------------
 // Scalar kernels of the reliable updates (one thread per RHS slot); those of the
@@ -575,16 +485,6 @@ void* ws_get(mdwf_ctx* ctx, const std::string& name, size_t bytes, cudaError_t* 
     e.second = bytes;
   }
   return e.first;
-}
-
-// Tables uploaded into a named workspace buffer of the context (no allocation once it exists).
-template <typename T>
-cudaError_t upload_tables_ws(mdwf_ctx* ctx, const std::string& name, const Tables& t, DevTables<T>* M,
-                             cudaStream_t st) {
-  cudaError_t e = cudaSuccess;
-  T* p = (T*)ws_get(ctx, name, sizeof(T) * t.h.size(), &e);
-  if (e != cudaSuccess) return e;
-  return M->upload(t, st, p);
 }
 
 template <typename S>
@@ -1636,26 +1536,14 @@ int hop_api(mdwf_ctx* ctx, const Cfg* cfg, int kind, int dagger, int out_par, co
 // A, B, A^-1 (op 0, 1, 2) or an adjoint on the caller's layout, FP64.
 int apply_5d_dev(mdwf_ctx* ctx, const Cfg* cfg, int which, int dagger, const double* in_dev, double* out_dev,
                  cudaStream_t st) {
-  const Geom& g = ctx->g;
-  const int L5 = cfg->act.L5;
-  Op<double, double> op;
-  op.g = g; op.L5 = L5; op.N = 1; op.anti = cfg->anti; op.U = cfg->U64; op.st = st;
-  op.tl = tiling_for<double>(g, L5, 1, 2, true);
   Tables tab;
   tab.build(cfg->act, std::vector<double>(1, cfg->act.mf));
-  DevTables<double> M;
-  CK(upload_tables_ws<double>(ctx, "apply.tables", tab, &M, st));
-  const long units = g.Vh * L5;
-  F<double> in, out, none;
-  CK(ws_field<double>(ctx, "apply.ie", units, &in));
-  CK(ws_field<double>(ctx, "apply.oe", units, &out));
+  cudaError_t e = cudaSuccess;
+  double* M = (double*)ws_get(ctx, "apply.tables", sizeof(double) * tab.h.size(), &e);
+  CK(e);
+  CK(cudaMemcpyAsync(M, tab.h.data(), sizeof(double) * tab.h.size(), cudaMemcpyHostToDevice, st));
   static const int kinds[3][2] = {{MK_A, MK_Ad}, {MK_B, MK_Bd}, {MK_Ainv, MK_Ainvd}};
-  const double* G = M[kinds[which][dagger ? 1 : 0]];
-  for (int par = 0; par < 2; par++) {
-    CK(pack_rhs<double>(&in_dev, in.v, nullptr, g, L5, 1, par, 0, 1, st));
-    CK(op.run(false, par, 0, in, none, G, none, nullptr, 0.0, out, nullptr, nullptr));
-    CK(unpack_rhs<double>(out.v, nullptr, &out_dev, g, L5, 1, par, 0, 1, st));
-  }
+  CK(local5_api(in_dev, out_dev, M + kinds[which][dagger ? 1 : 0] * tab.block(), ctx->g.V, cfg->act.L5, st));
   CK(cudaStreamSynchronize(st));
   return MDWF_OK;
 }

@@ -297,29 +297,6 @@ inline Tiling make_tiling(long Vh, int L5, int N, int nsb, int max_threads = 102
   return t;
 }
 
-// Operands of one Wilson-hop + fifth-dimension launch (see hop.cu):
-//   out = add + G . same + kappa * C . H(in)      (HOP = true)
-//   out = add + G . in                            (HOP = false)
-// G, C: per-slot [2][L5][L5] matrices (null C = identity, null G = no term).
-template <typename S, typename T>
-struct HopArgs {
-  Geom g;
-  int L5, N;
-  int out_par;          // parity of the output sites
-  int dagger;           // 1: H^+ (projectors exchanged)
-  int antiperiodic;     // time boundary phase -1
-  const S* in; const float* in_nrm;        // opposite parity (HOP) or same parity (local)
-  const S* same; const float* same_nrm;    // output parity, optional
-  const S* add; const float* add_nrm;      // output parity, optional
-  S* out; float* out_nrm;
-  const T* U;           // gauge [2][Vh][4][18]
-  const T* Gm;          // [N][2][L5][L5] or null
-  const T* Cm;          // [N][2][L5][L5] or null (identity)
-  T kappa;
-  const int* active;    // [N] or null (all active)
-  double* partials;     // [ntiles][N] |out|^2 per tile, or null
-};
-
 // Structured fifth-dimension epilogues of the fast hop kernel (hop_fast.cu).
 enum Epi { E_RAW = 0, E_BAINV = 1, E_AINVD_BD = 2, E_A_SAME = 3, E_AD_SAME_BD = 4, E_AINV_SAME = 5,
            // symmetric Schur form: add + g same + A^-1 (kappa H in); add + g same + kappa B^+ H in;
@@ -394,6 +371,8 @@ cudaError_t launch_fast(const FastArgs<S, T>& a, const Tiling& t, int epi, cudaS
 cudaError_t launch_hop64(const FastArgs<double, double>& a, int epi, cudaStream_t st);
 cudaError_t launch_hop64_api(const FastArgs<double, double>& a, int epi, cudaStream_t st);
 cudaError_t bop_api(const double* x, double* u, long V, int L5, double b5, double c5, double m, cudaStream_t st);
+// out_s = sum_s' G[chirality][s][s'] in_s' on the caller's layout (one right-hand side); L5 <= 32.
+cudaError_t local5_api(const double* in, double* out, const double* G, long V, int L5, cudaStream_t st);
 // Two-slices-per-thread hop (hop_pair.cu): block (rt, J = ceil(L5 / 2), nsb).
 struct PairShape {
   int J, nsb, rt, threads;
@@ -431,13 +410,5 @@ template <typename S, typename T>
 size_t staged_smem_bytes(const Tiling& t, int L5, int N);
 template <typename S, typename T>
 int fast_max_threads();
-
-// Kernel launchers (hop.cu).
-template <typename S, typename T>
-cudaError_t launch_hop(const HopArgs<S, T>& a, const Tiling& t, bool hop, cudaStream_t st);
-template <typename S, typename T>
-int hop_max_threads();
-template <typename S, typename T>
-size_t hop_smem_bytes(const Tiling& t, bool two);
 
 }  // namespace mdwf
