@@ -1567,6 +1567,14 @@ int apply_dev(mdwf_ctx* ctx, Cfg* cfg, int kind, int arg1, int arg2, const doubl
 // src = (1 - c5 D_W) w = (1 - c5 d) w + c5/2 H w for the wall field w of a 4D source (device arrays).
 int make_source_impl(mdwf_ctx* ctx, const Cfg* cfg, const double* eta, double* src, cudaStream_t st) {
   const Action& a = cfg->act;
+  const size_t n4 = (size_t)24 * ctx->g.V;
+  if (eta < src + n4 * a.L5 && src < eta + n4) {   // overlapping: the source reads other sites than it writes
+    cudaError_t e = cudaSuccess;
+    double* copy = (double*)ws_get(ctx, "make_source.eta", sizeof(double) * n4, &e);
+    CK(e);
+    CK(cudaMemcpyAsync(copy, eta, sizeof(double) * n4, cudaMemcpyDeviceToDevice, st));
+    eta = copy;
+  }
   CK(wall_source(cfg->U64, eta, src, ctx->g, a.L5, cfg->anti, 1.0 - a.c5 * (4.0 - a.M5), 0.5 * a.c5, st));
   return MDWF_OK;
 }
@@ -2030,7 +2038,7 @@ long long mdwf_session_bytes(mdwf_ctx* ctx, int cfg_id, int slots, int precision
   const double x = precision == MDWF_PREC_DOUBLE ? 192 : 96;
   // nine FP64 fields (seven solver fields and the slots' own sources; the FP32
   // update fields share two of them), six inner fields, x_lo, partial sums
-  return (long long)(units * (9 * 192 + 6 * s + x) + (double)ctx->g.Vh * slots * 8 + 4096.0 * slots);
+  return (long long)(units * (9 * 192 + 6 * s + x) + (double)ctx->g.Vh * slots * 16 + 4096.0 * slots);
 }
 
 int mdwf_session_create(mdwf_ctx* ctx, int cfg_id, int slots, const mdwf_solver_opts* opts, double tol, void* stream,
