@@ -52,7 +52,7 @@ struct Cfg {
 
 struct mdwf_ctx {
   int device = 0;
-  int clock_khz = 2000000;   // SM clock, read once: the query takes 0.6 ms
+  int clock_khz = 0;         // SM clock, read at the first solve: the query takes 0.6 ms
   Geom g;
   std::map<int, Cfg> cfgs;
   std::string err;
@@ -459,7 +459,14 @@ Tiling fast_tiling(const Geom& g, int L5, int N, int nsb_req, bool* staged, bool
 }
 
 // Bound of device-side waits in clock cycles.
-long long wait_budget(const mdwf_ctx* ctx, double seconds) { return (long long)(seconds * 1e3 * (double)ctx->clock_khz); }
+long long wait_budget(mdwf_ctx* ctx, double seconds) {
+  if (ctx->clock_khz == 0) {
+    int khz = 0;
+    const bool known = cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, ctx->device) == cudaSuccess && khz > 0;
+    ctx->clock_khz = known ? khz : 2000000;
+  }
+  return (long long)(seconds * 1e3 * (double)ctx->clock_khz);
+}
 
 template <typename T>
 Fifth<T> make_fifth(const Action& act, const T* mass_dev) {
@@ -1778,8 +1785,6 @@ int mdwf_create(const int dims[4], int device, mdwf_ctx** out) {
   mdwf_ctx* c = new mdwf_ctx();
   c->device = device;
   c->g = make_geom(dims);
-  int khz = 0;
-  if (cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, device) == cudaSuccess && khz > 0) c->clock_khz = khz;
   if (cudaStreamCreateWithFlags(&c->stream, cudaStreamNonBlocking) != cudaSuccess) { delete c; return MDWF_ERR_CUDA; }
   *out = c;
   return MDWF_OK;
