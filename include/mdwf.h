@@ -231,11 +231,9 @@ int mdwf_apply_schur_batch_dev(mdwf_ctx* ctx, int cfg_id, int n, const double* c
  * when its work on `stream` has finished, so it cannot be captured in a CUDA
  * graph.  It looks up the array's device address on every call (no cached
  * address survives a device reset).  Every call uses the same array, which
- * keeps the previous call's
- * contents (the kernels overwrite what they read, and the one field that must
- * start at zero is cleared by the call itself); calls that overlap on the GPU --
- * from several streams or host threads at once -- race on the array and must be
- * serialised by the caller.  The paper has no counterpart to this entry point.
+ * keeps the previous call's contents (the kernels overwrite what they read);
+ * calls that overlap on the GPU -- from several streams or host threads at
+ * once -- race on the array and must be serialised by the caller.  The paper has no counterpart to this entry point.
  * Errors: ARG (including a problem too large for the array), STATE, CUDA. */
 #define MDWF_NOALLOC_SCRATCH_BYTES (64u * 1024u * 1024u)
 int mdwf_apply_schur_batch_dev_noalloc(mdwf_ctx* ctx, int cfg_id, int n, const double* const* in,

@@ -1,5 +1,7 @@
 // Wilson hop on all L5 slices x RHS slots with the structured fifth-dimension
-// epilogues of the even-odd Moebius operator (the solver's hot path).
+// epilogues of the even-odd Moebius operator, in FP32 arithmetic: one unit per
+// thread, staged and tensor-core forms.  The solver's default form is in
+// hop_pair.cu, the FP64 hop in hop64.cu.
 //
 // With A = alpha + beta P and B = b5 + c5 P (Sec. II of arXiv:1701.07559 and
 // the Brower-Neff-Orginos 5D form), P moves the P_+ half (spins 0,1) one slice

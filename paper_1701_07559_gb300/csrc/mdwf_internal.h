@@ -14,7 +14,7 @@
 //   gauge field:                [parity][h][mu][18]   (3x3 complex, row major),
 //                                mu = 0..3 for x, y, z, t; U_mu(x) of the site x;
 //                                the FP32 copy pads each link to 20 floats.
-//   fifth-dimension matrices:   [r][chirality][L5][L5] real; chirality 0 acts on
+//   fifth-dimension matrices:   [chirality][L5][L5] real; chirality 0 acts on
 //                                spins 0,1 (P_+), chirality 1 on spins 2,3 (P_-).
 // Half-lattice index: lex = x + Lx (y + Ly (z + Lz t)), h = lex >> 1 (Lx even).
 #pragma once
