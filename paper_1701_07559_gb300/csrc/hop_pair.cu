@@ -730,6 +730,16 @@ PairShape pair_shape(int L5, int N, int nsb) {
   int rt = kPairMaxThreads / (nsb * p.J);
   if (rt < 1) rt = 1;
   p.rt = N < rt ? N : rt;
+  // Full warps: where all systems of the block's sites leave a warp partly empty or make a block of more than
+  // 256 threads, of which the registers allow one per SM, a divisor of N that fills two to eight warps takes
+  // part of them (24 systems at L5 = 12, 12^3 x 24: 71.1 us per million units with 144 threads, 67.0 with
+  // 96; 12 systems at L5 = 6, 8^3 x 24: 90.3 with 144, 87.4 with 96).  Every shape gives the same bits.
+  if (p.rt * p.J * p.nsb % 32 != 0 || p.rt * p.J * p.nsb > 256)
+    for (int d = p.rt - 1; d >= 1; d--)
+      if (N % d == 0 && d * p.J * p.nsb % 32 == 0 && d * p.J * p.nsb >= 64 && d * p.J * p.nsb <= 256) {
+        p.rt = d;
+        break;
+      }
   p.threads = p.rt * p.J * p.nsb;
   p.smem = pair_tile_bytes(p.threads, p.nsb, L5, p.rt);
   p.smem_pf = p.smem + pair_pf_bytes(p.threads, p.nsb);

@@ -226,3 +226,23 @@ def test_fp64_solves_of_ragged_tiles(dims, L5, n):
             assert O.true_residual(L.U, b[k], xs[k], *ACT[:3], masses[k]) <= 1e-9
             one, _ = M.mdwf_solve_batch(L.ctx, 0, [b[k]], 1e-9, masses=[masses[k]], opts=opts)
             assert np.array_equal(one[0], xs[k])
+
+
+@pytest.mark.parametrize('n,L5,nsb', [(24, 12, 2), (24, 12, 1), (12, 6, 4), (12, 12, 4), (6, 5, 8)])
+def test_half_hop_with_part_of_the_systems_per_block(n, L5, nsb):
+    """Blocks that take a divisor of the systems to fill their warps: the bits of each system alone."""
+    with Lat((4, 2, 2, 6), L5) as L:
+        masses = [0.02 + 0.01 * (k % 7) for k in range(n)]
+        xs = [torch.from_numpy(O.restrict(synth.gaussian_spinor(L.shape, 80 + k), O.parity_mask(L.dims))).cuda()
+              for k in range(n)]
+        for form in (M.HOP_DIRECT, M.HOP_PAIR_PF):
+            for dagger in (0, 1):
+                outs = [torch.empty_like(x) for x in xs]
+                M.mdwf_apply_schur_batch_dev(L.ctx, 0, xs, outs, masses=masses, dagger=dagger, precision='half',
+                                             hop_variant=form | (nsb << 8))
+                for k in {0, n // 3, n // 2 - 1, n - 1}:
+                    one = torch.empty_like(xs[k])
+                    M.mdwf_apply_schur_batch_dev(L.ctx, 0, [xs[k]], [one], masses=[masses[k]], dagger=dagger,
+                                                 precision='half', hop_variant=form | (1 << 8))
+                    torch.cuda.synchronize()
+                    assert torch.equal(one, outs[k])
