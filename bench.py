@@ -519,7 +519,7 @@ def run_ours(args):
     tuned = M.mdwf_autotune(ctx, 0, len(chunks[0]), prec, include_tensor_core=args.hop_variant == 4) \
         if args.hop_variant in (0, 4) and args.nsb == 0 else None
     variant = tuned['hop_variant'] if tuned else (args.hop_variant or 1)
-    kernel_name = {1: 'hop_pair_kernel' if prec != 'double' else 'hop_fast_kernel_f64',
+    kernel_name = {1: 'hop_pair_kernel' if prec != 'double' else 'hop64_kernel',
                    2: 'hop_staged_kernel', 3: 'hop_mma_kernel', 6: 'hop_fast_kernel'}.get(variant, 'hop_pair_kernel')
     hop_form = 'prefetching' if (variant == 7 and prec == 'half' and args.link_recon == 18) else 'plain'
 
