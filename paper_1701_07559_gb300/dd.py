@@ -231,7 +231,10 @@ def solve(op, bs, tol=1e-10, max_iter=100000, passes=5):
 
 class GPUSubdomain:
     """A sub-domain on the GPU: a context of the local dims with the slab's links
-    and the action; its faces and halos are torch CUDA tensors (FP64)."""
+    and the action; its faces and halos are torch CUDA tensors (FP64).  The library
+    runs on the context's own stream, which waits for no other: what torch has
+    queued for the call's arrays (slabs, halo copies, CG vectors) is waited for
+    first, and the library's calls return when their work is done."""
 
     def __init__(self, M, split, k, U_global, action, device=0, cfg_id=0):
         import torch
@@ -246,12 +249,14 @@ class GPUSubdomain:
         import torch
         fp = torch.empty(self.fshape, dtype=torch.complex128, device=self.device)
         fn = torch.empty_like(fp)
+        torch.cuda.current_stream(self.device).synchronize()
         self.M.mdwf_dd_pack_faces_dev(self.ctx, self.cfg_id, kind, dagger, x, fp, fn)
         return fp, fn
 
     def apply(self, kind, dagger, x, halo_next, halo_prev, sign_next, sign_prev):
         import torch
         out = torch.empty_like(x)
+        torch.cuda.current_stream(self.device).synchronize()
         self.M.mdwf_dd_apply_dev(self.ctx, self.cfg_id, kind, dagger, x, out, halo_next, halo_prev,
                                  sign_next, sign_prev)
         return out
