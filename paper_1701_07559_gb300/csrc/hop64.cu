@@ -12,10 +12,12 @@
 //   lattice are (a thread per unit left half of the lanes idle at N = 1, L5 = 8, and
 //   a 4^3 x 8 lattice on a few schedulers); on small lattices the work spreads eight
 //   times wider.
-// * x_b = U^+ h_b first, then S = x_b + U h_f as one chain of multiply-adds onto it,
-//   and D = 2 x_b - S = x_b - U h_f: the upper spins sum S over the directions, the
-//   lower ones D with the gamma matrices' factors: 99 instructions per lane, 792 per
-//   unit, where the accumulation of both products took 864.
+// * x_b = U^+ h_b and x_f = U h_f, each rounded by itself, then S = x_b + x_f and D = x_b - x_f: the
+//   upper spins sum S over the directions, the lower ones D with the gamma matrices' factors: 105
+//   instructions per lane, 840 per unit, where the accumulation of every product into all four spins took
+//   864.  Chaining U h_f onto x_b and taking D = 2 x_b - S saves 6 of the 105, but rounds at the size of
+//   the sum: 1.05 times the error of that accumulation in H (1.57e-16 against 1.49e-16, rms of the result,
+//   extended precision as the reference), this order 0.93 times (1.38e-16).
 // * the sums over the directions are a reduce-scatter by shuffles; factors 1, -1, i, -i
 //   are exchanges and sign bits.
 // * slots whose mask is off are left out of the enumeration, so a re-reference of a
@@ -82,18 +84,18 @@ __device__ __forceinline__ double flip(double v, unsigned bit31) {      // v or 
 }
 __device__ __forceinline__ double sx(double v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
 
-// o = (or o += when ADD) M v with M_ab = l[a][b] (DAG: conj(l[b][a])), the operations of a
-// colour multiply in their usual order: one multiply and five multiply-adds per real output.
-template <bool DAG, bool ADD>
+// o = M v with M_ab = l[a][b] (DAG: conj(l[b][a])), the operations of a colour multiply in their
+// usual order: one multiply and five multiply-adds per real output.
+template <bool DAG>
 __device__ __forceinline__ void colour_mul(const double* __restrict__ l, const double* v, double* o) {
 #pragma unroll
   for (int a = 0; a < 3; a++) {
-    double re = ADD ? o[2 * a] : 0.0, im = ADD ? o[2 * a + 1] : 0.0;
+    double re, im;
 #pragma unroll
     for (int b = 0; b < 3; b++) {
       const double2 u = __ldg(reinterpret_cast<const double2*>(l) + (DAG ? 3 * b + a : 3 * a + b));
       const double ui = DAG ? -u.y : u.y;
-      if (b == 0 && !ADD) { re = u.x * v[0]; im = u.x * v[1]; }
+      if (b == 0) { re = u.x * v[0]; im = u.x * v[1]; }
       else { re = __fma_rn(u.x, v[2 * b], re); im = __fma_rn(u.x, v[2 * b + 1], im); }
       re = __fma_rn(-ui, v[2 * b + 1], re);
       im = __fma_rn(ui, v[2 * b], im);
@@ -231,21 +233,19 @@ __global__ void __launch_bounds__(256, 3) hop64_kernel(FastArgs<double, double> 
         }
       };
       const long lex3 = lex - (long)c[3] * a.g.L[0] * a.g.L[1] * a.g.L[2];
-      double v[6], S[6], D[6];
+      double v[6], xb[6], xf[6], S[6], D[6];
       if (hb) {
         const double* hp = a.halo_bwd + ((lex3 * L5 + s) * a.N + r) * 12 + 6 * j;
 #pragma unroll
-        for (int b = 0; b < 6; b++) S[b] = hp[b] * a.halo_sgn_bwd;
+        for (int b = 0; b < 6; b++) xb[b] = hp[b] * a.halo_sgn_bwd;
       } else {
         project(nb, -sgf, v);
         if (flb) {
 #pragma unroll
           for (int b = 0; b < 6; b++) v[b] = flip(v[b], 0x80000000u);
         }
-        colour_mul<true, false>(a.U + (((long)(1 - par) * a.g.Vh + (nb >> 1)) * 4 + mu) * 18, v, S);
+        colour_mul<true>(a.U + (((long)(1 - par) * a.g.Vh + (nb >> 1)) * 4 + mu) * 18, v, xb);
       }
-#pragma unroll
-      for (int b = 0; b < 6; b++) D[b] = S[b];                           // x_b
       if (hf) {
         const double* hp = a.halo_fwd + ((lex3 * L5 + s) * a.N + r) * 12 + 6 * j;
 #pragma unroll
@@ -257,9 +257,9 @@ __global__ void __launch_bounds__(256, 3) hop64_kernel(FastArgs<double, double> 
           for (int b = 0; b < 6; b++) v[b] = flip(v[b], 0x80000000u);
         }
       }
-      colour_mul<false, true>(a.U + (((long)par * a.g.Vh + h) * 4 + mu) * 18, v, S);
+      colour_mul<false>(a.U + (((long)par * a.g.Vh + h) * 4 + mu) * 18, v, xf);
 #pragma unroll
-      for (int b = 0; b < 6; b++) D[b] = __fma_rn(2.0, D[b], -S[b]);     // x_b - x_f
+      for (int b = 0; b < 6; b++) { S[b] = xb[b] + xf[b]; D[b] = xb[b] - xf[b]; }
       // factor on the lower spin, then x, y lanes hand theirs to the lane of its spin
       double E[6];
 #pragma unroll
