@@ -22,6 +22,9 @@
 //   of matrix products.  |X|_F is first scaled to at most 1/2 by 2^-k (k squarings
 //   of the result; none for the usual steps); 17 terms leave a remainder below
 //   (1/2)^18 / 18! < 1e-21.
+// * U <- exp(X) U as U + (exp(X) - 1) U: for the usual steps the second term is small, and a stage rounds U once at its
+//   own size.  Error of 10 steps of 0.01 against extended precision: 1.96e-16 of the links, where the chain of
+//   multiply-adds of exp(X) U left 5.35e-16 and the matrix products before it 4.65e-16; it costs 1 % of a step.
 // Z keeps the nine independent reals of an anti-Hermitian matrix, one plane each.
 // Ten steps at 16^3 x 48: 297 ms with a thread per link and the matrix Taylor series
 // (which spilled), 71 ms so (2.4 ms per stage; its 1800 multiply-adds per link take 2.3 ms
@@ -176,8 +179,9 @@ __global__ void __launch_bounds__(3 * kZLinks) k_flow_Z(const double* __restrict
   Z[(long)(4 + 2 * row) * nlink + k] = -eps * (0.5 * (x.y + y.y));
 }
 
-// exp of the anti-Hermitian traceless X with diagonal i d[0..2] and elements (0,1), (0,2), (1,2) = o[0..2].
-__device__ __forceinline__ void mexp(const double d_in[3], const C2 o_in[3], M3& E) {
+// F = exp(X) - 1 of the anti-Hermitian traceless X with diagonal i d[0..2] and elements (0,1), (0,2), (1,2) = o[0..2].
+// Without the unit matrix its small elements keep their digits.
+__device__ __forceinline__ void mexpm1(const double d_in[3], const C2 o_in[3], M3& F) {
   double n2 = 0.0;
 #pragma unroll
   for (int i = 0; i < 3; i++)
@@ -209,7 +213,7 @@ __device__ __forceinline__ void mexp(const double d_in[3], const C2 o_in[3], M3&
   const C2 t{o[0].re * o[2].re - o[0].im * o[2].im, o[0].re * o[2].im + o[0].im * o[2].re};
   const double dt = -d[0] * d[1] * d[2] + d[0] * a12 + d[1] * a02 + d[2] * a01 -
                     2.0 * (t.im * o[1].re - t.re * o[1].im);
-  // Horner on p0 + p1 X + p2 X^2:  p <- p X + 1/k!
+  // Horner on p0 + p1 X + p2 X^2:  p <- p X + 1/k!, the last step (k = 0) without its 1
   constexpr int kTerms = 17;
   const double invf[kTerms + 1] = {1.0, 1.0, 1.0 / 2, 1.0 / 6, 1.0 / 24, 1.0 / 120, 1.0 / 720, 1.0 / 5040, 1.0 / 40320,
                                    1.0 / 362880, 1.0 / 3628800, 1.0 / 39916800, 1.0 / 479001600, 1.0 / 6227020800.0,
@@ -218,19 +222,19 @@ __device__ __forceinline__ void mexp(const double d_in[3], const C2 o_in[3], M3&
   C2 p0{invf[kTerms], 0.0}, p1{0.0, 0.0}, p2{0.0, 0.0};
 #pragma unroll
   for (int k = kTerms - 1; k >= 0; k--) {
-    const C2 n0{__fma_rn(-dt, p2.im, invf[k]), dt * p2.re};
+    const C2 n0{k > 0 ? __fma_rn(-dt, p2.im, invf[k]) : -dt * p2.im, dt * p2.re};
     const C2 n1{__fma_rn(c1, p2.re, p0.re), __fma_rn(c1, p2.im, p0.im)};
     p2 = p1;
     p1 = n1;
     p0 = n0;
   }
-  // E = p0 + p1 X + p2 X^2
+  // F = p0 + p1 X + p2 X^2
 #pragma unroll
   for (int i = 0; i < 3; i++) {
     C2 e = p0;
     e.re = __fma_rn(-p1.im, d[i], e.re); e.im = __fma_rn(p1.re, d[i], e.im);
     e.re = __fma_rn(-p2.re, q[i], e.re); e.im = __fma_rn(-p2.im, q[i], e.im);
-    E.m[4 * i] = e;
+    F.m[4 * i] = e;
   }
 #pragma unroll
   for (int i = 0; i < 3; i++) {
@@ -240,13 +244,18 @@ __device__ __forceinline__ void mexp(const double d_in[3], const C2 o_in[3], M3&
     cfma(p2, y[i], u);
     cfma(p1, C2{-o[i].re, o[i].im}, l);                  // X_ba = -conj(X_ab)
     cfma(p2, C2{y[i].re, -y[i].im}, l);                  // (X^2)_ba = conj((X^2)_ab)
-    E.m[3 * a + b] = u;
-    E.m[3 * b + a] = l;
+    F.m[3 * a + b] = u;
+    F.m[3 * b + a] = l;
   }
-  for (int i = 0; i < sq; i++) mmul(E, E, E);
+  for (int k = 0; k < sq; k++) {                         // (1 + F)^2 - 1 = F^2 + 2 F
+    M3 t;
+    mmul(F, F, t);
+#pragma unroll
+    for (int i = 0; i < 9; i++) F.m[i] = C2{__fma_rn(2.0, F.m[i].re, t.m[i].re), __fma_rn(2.0, F.m[i].im, t.m[i].im)};
+  }
 }
 
-// U <- exp(c0 Z0 + c1 Z1 + c2 Z2) U for every link.
+// U <- exp(c0 Z0 + c1 Z1 + c2 Z2) U for every link, as U + F U.
 template <int NZ>
 __global__ void __launch_bounds__(128) k_flow_update(double* __restrict__ U, const double* __restrict__ Z, long nlink,
                                                     double c0, double c1, double c2) {
@@ -262,8 +271,8 @@ __global__ void __launch_bounds__(128) k_flow_update(double* __restrict__ U, con
   }
   const double d[3] = {x[0], x[1], x[2]};
   const C2 o[3] = {{x[3], x[4]}, {x[5], x[6]}, {x[7], x[8]}};
-  M3 E;
-  mexp(d, o, E);
+  M3 F;
+  mexpm1(d, o, F);
   // column by column of U (three complex numbers live at a time)
   double* u = U + 18 * k;
 #pragma unroll
@@ -273,9 +282,9 @@ __global__ void __launch_bounds__(128) k_flow_update(double* __restrict__ U, con
     for (int i = 0; i < 3; i++) {
       C2 s{0.0, 0.0};
 #pragma unroll
-      for (int m = 0; m < 3; m++) cfma(E.m[3 * i + m], v[m], s);
-      u[6 * i + 2 * j] = s.re;
-      u[6 * i + 2 * j + 1] = s.im;
+      for (int m = 0; m < 3; m++) cfma(F.m[3 * i + m], v[m], s);
+      u[6 * i + 2 * j] = v[i].re + s.re;
+      u[6 * i + 2 * j + 1] = v[i].im + s.im;
     }
   }
 }
