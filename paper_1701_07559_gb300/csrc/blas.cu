@@ -761,6 +761,29 @@ cudaError_t unpack_rhs(const S* in, const float* in_nrm, double* const* api, con
   return cudaGetLastError();
 }
 
+// A launch takes the slots that follow while their arrays share nothing: its threads write in no order.
+template <typename S>
+cudaError_t unpack_all(const S* even, const float* even_nrm, const S* odd, const float* odd_nrm, double* const* api,
+                       const Geom& g, int L5, int N, long long* launches, cudaStream_t st) {
+  const uintptr_t bytes = sizeof(double) * 24 * (uintptr_t)g.V * L5;
+  for (int b = 0, m; b < N; b += m) {
+    for (m = 1; m < kPtrs && b + m < N; m++) {
+      const uintptr_t x = (uintptr_t)api[b + m];
+      bool shares = false;
+      for (int k = b; k < b + m; k++) {
+        const uintptr_t y = (uintptr_t)api[k];
+        shares = shares || (x < y + bytes && y < x + bytes);
+      }
+      if (shares) break;
+    }
+    cudaError_t e = unpack_rhs<S>(even, even_nrm, api + b, g, L5, N, 0, b, m, st);
+    if (e == cudaSuccess) e = unpack_rhs<S>(odd, odd_nrm, api + b, g, L5, N, 1, b, m, st);
+    if (e != cudaSuccess) return e;
+    if (launches) *launches += 2;
+  }
+  return cudaSuccess;
+}
+
 template <typename Si, typename So>
 cudaError_t convert(const Si* in, const float* in_nrm, So* out, float* out_nrm, const Tiling& t, long Vh, int L5,
                     int N, const int* mask, cudaStream_t st) {
@@ -931,6 +954,8 @@ Tiling blas_tiling(long Vh, int L5, int N, int max_units, int lanes) {
                                    cudaStream_t);                                                               \
   template cudaError_t unpack_rhs<S>(const S*, const float*, double* const*, const Geom&, int, int, int, int,   \
                                      int, cudaStream_t);                                                        \
+  template cudaError_t unpack_all<S>(const S*, const float*, const S*, const float*, double* const*, const Geom&, \
+                                     int, int, long long*, cudaStream_t);                                       \
   template cudaError_t norm2_partials<S>(const S*, const float*, const Tiling&, long, int, int, const int*,      \
                                          double*, cudaStream_t);
 

@@ -47,6 +47,13 @@ template <typename S>
 cudaError_t unpack_rhs(const S* in, const float* in_nrm, double* const* api, const Geom& g, int L5, int N, int par,
                        int r0, int nr, cudaStream_t st);
 
+// Both parities of slots 0 .. N - 1 into the caller's arrays (odd == null: zeros on the odd sites).  Arrays that
+// coincide or overlap are written one after the other, as if slot by slot: what they share holds the last
+// slot's values.  Adds the kernels launched to *launches, if given.
+template <typename S>
+cudaError_t unpack_all(const S* even, const float* even_nrm, const S* odd, const float* odd_nrm, double* const* api,
+                       const Geom& g, int L5, int N, long long* launches, cudaStream_t st);
+
 template <typename Si, typename So>
 cudaError_t convert(const Si* in, const float* in_nrm, So* out, float* out_nrm, const Tiling& t, long Vh, int L5,
                     int N, const int* mask, cudaStream_t st);

@@ -1143,9 +1143,7 @@ int solve_batch_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const* srcs, 
     CK(sv.norms(sv.rho64, nullptr, tmp));
     CK(cudaMemcpyAsync(re.data(), tmp, sizeof(double) * N, cudaMemcpyDeviceToHost, st));
     CK(cudaMemcpyAsync(iters.data(), sv.sc.iters, sizeof(int) * N, cudaMemcpyDeviceToHost, st));
-    sv.launches += 2;
-    CK(unpack_rhs<double>(sv.x_acc.v, nullptr, xs, g, L5, N, 0, 0, N, st));
-    CK(unpack_rhs<double>(x_o.v, nullptr, xs, g, L5, N, 1, 0, N, st));
+    CK(unpack_all<double>(sv.x_acc.v, nullptr, x_o.v, nullptr, xs, g, L5, N, &sv.launches, st));
     CK(cudaStreamSynchronize(st));
     CK(ph.mark(PH_FINAL, st));
     return MDWF_OK;
@@ -1713,8 +1711,7 @@ int schur_batch_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const* in, do
   } else {
     CK(op.mhat_dag(fin, ft, fo, nullptr, nullptr));
   }
-  CK(unpack_rhs<S>(fo.v, fo.n, out, g, L5, N, 0, 0, N, st));
-  CK(unpack_rhs<S>(nullptr, nullptr, out, g, L5, N, 1, 0, N, st));
+  CK(unpack_all<S>(fo.v, fo.n, nullptr, nullptr, out, g, L5, N, nullptr, st));
   int herr = 0;
   CK(cudaMemcpyAsync(&herr, errw, sizeof(int), cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
@@ -2328,8 +2325,7 @@ int schur_batch_noalloc_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const
   } else {
     CK(op.mhat_dag(fin, ft, fo, nullptr, nullptr));
   }
-  CK(unpack_rhs<S>(fo.v, fo.n, out, g, L5, N, 0, 0, N, st));
-  CK(unpack_rhs<S>(nullptr, nullptr, out, g, L5, N, 1, 0, N, st));
+  CK(unpack_all<S>(fo.v, fo.n, nullptr, nullptr, out, g, L5, N, nullptr, st));
   CK(cudaStreamSynchronize(st));
   return MDWF_OK;
 }
