@@ -101,8 +101,8 @@ cudaError_t wall_source(const double* U, const double* eta, double* src, const G
 // n_iter smearing steps of eta in place; tmp: V * 24 doubles, slices: 2 Lt + 1 ints.
 cudaError_t smear(const double* U, double* eta, double* tmp, int* slices, const Geom& g, double k, int n_iter,
                   cudaStream_t st);
-// c[2][Lt]: the two residual-mass correlators; part: 2 Lt mres_blocks(V / Lt) doubles.
-int mres_blocks(long slice_sites);
+// c[2][Lt]: the two residual-mass correlators; part: 2 Lt mres_blocks(V / Lt, Lt) doubles.
+int mres_blocks(long slice_sites, int Lt);
 cudaError_t mres_correlators(const double* const* xs, int n, long V, int Lt, int L5, double* part, double* c,
                              cudaStream_t st);
 

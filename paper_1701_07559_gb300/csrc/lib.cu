@@ -2206,7 +2206,7 @@ int mdwf_mres_correlators_dev(mdwf_ctx* ctx, int cfg_id, int n, double* const* x
   cudaError_t e = cudaSuccess;
   double** dptr = (double**)ws_get(ctx, "mres.ptrs", sizeof(double*) * n, &e);
   CK(e);
-  const size_t npart = (size_t)2 * Lt * mres_blocks(V / Lt);
+  const size_t npart = (size_t)2 * Lt * mres_blocks(V / Lt, Lt);
   double* part = (double*)ws_get(ctx, "mres.part", sizeof(double) * (npart + 2 * Lt), &e);
   CK(e);
   double* c = part + npart;
