@@ -737,6 +737,8 @@ __global__ void k_resid_update(const double* __restrict__ bhat, const float* __r
 // ---------------------------------------------------------------------------
 static inline dim3 tile_grid(const Tiling& t) { return dim3((unsigned)t.ntiles, (unsigned)t.ngroups); }
 
+int pack_launches(int nr) { return (nr + kPtrs - 1) / kPtrs; }
+
 template <typename S>
 cudaError_t pack_rhs(const double* const* api, S* out, float* out_nrm, const Geom& g, int L5, int N, int par, int r0,
                      int nr, cudaStream_t st) {

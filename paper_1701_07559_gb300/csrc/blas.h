@@ -47,6 +47,8 @@ template <typename S>
 cudaError_t unpack_rhs(const S* in, const float* in_nrm, double* const* api, const Geom& g, int L5, int N, int par,
                        int r0, int nr, cudaStream_t st);
 
+// Kernels that pack_rhs launches for nr fields.
+int pack_launches(int nr);
 // Both parities of slots 0 .. N - 1 into the caller's arrays (odd == null: zeros on the odd sites).  Arrays that
 // coincide or overlap are written one after the other, as if slot by slot: what they share holds the last
 // slot's values.  Adds the kernels launched to *launches, if given.

@@ -999,7 +999,7 @@ int solve_batch_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const* srcs, 
   // Schur right-hand side bhat_e = b_e + 1/2 H_eo B A^-1 b_o in bhat (FP64); the
   // sources are packed into rho64 (b_e) and x_hi (b_o), which are free then.
   auto schur_source = [&](bool norms) -> int {
-    sv.launches += 2;
+    sv.launches += 2 * pack_launches(N);
     sv.b_e = sv.rho64;
     sv.b_o = sv.x_hi;
     CK(pack_rhs<double>(srcs, sv.b_e.v, nullptr, g, L5, N, 0, 0, N, st));
@@ -1121,7 +1121,7 @@ int solve_batch_impl(mdwf_ctx* ctx, Cfg* cfg, int n, const double* const* srcs, 
   // reuses y.  Even sites: b_e - A x_e + 1/2 H_eo B x_o (the second FP64 hop).
   std::vector<double> re(N), ro(N);
   auto finish = [&]() -> int {
-    sv.launches += 4;
+    sv.launches += 2 + 2 * pack_launches(N);
     CK(accum_xhi<typename BatchSolver<S>::SX>(sv.x_hi.v, sv.xlo.v, sv.tl_blas, g.Vh, L5, N, nullptr, st));
     CK(accum_xhi<double>(sv.x_acc.v, sv.x_hi.v, sv.tl_blas, g.Vh, L5, N, nullptr, st));
     // sources again, in fields now free (bhat, x_hi)
