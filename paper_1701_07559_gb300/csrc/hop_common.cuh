@@ -1,8 +1,14 @@
-// Device helpers shared by the Wilson-hop kernels (hop_fast.cu, hop_pair.cu):
+// Device helpers shared by the Wilson-hop kernels (hop_fast.cu, hop_pair.cu, hop64.cu):
 // the 4D site of a thread with its neighbour indices, and the spin projection
 // of a colour-major fp16 spinor.
 #pragma once
 #include "mdwf_internal.h"
+
+// Lengths of the fifth dimension at which every hop runs the recursions along s on a column in registers: the tuned
+// actions' up to 16 (6, 8, 12, 16) and the even ones between 4 and 12.  Other lengths run the same operations in the
+// shared-memory tile, with the same bits; 20 and 24 in registers gain nothing (FP64 Schur operator of four fields at
+// 8^3 x 16: 1349 against 1351 us, 1588 against 1601) and make the FP64 kernels spill ten times as much.
+#define MDWF_COLUMN_LENGTHS(X) X(4) X(6) X(8) X(10) X(12) X(16)
 
 namespace mdwf {
 namespace hopc {

@@ -401,12 +401,9 @@ __device__ __forceinline__ void epilogue(const FastArgs<S, T>& a, const Tiling& 
         const int st = tl.rt * kPadF;
         T* base = sA + (size_t)(t.site_l * L5 * tl.rt + t.r_l) * kPadF;
         switch (L5) {
-          case 4: cols_regs<4, EPI, T>(base, st, t.s, a.f, m); break;
-          case 6: cols_regs<6, EPI, T>(base, st, t.s, a.f, m); break;
-          case 8: cols_regs<8, EPI, T>(base, st, t.s, a.f, m); break;
-          case 10: cols_regs<10, EPI, T>(base, st, t.s, a.f, m); break;
-          case 12: cols_regs<12, EPI, T>(base, st, t.s, a.f, m); break;
-          case 16: cols_regs<16, EPI, T>(base, st, t.s, a.f, m); break;
+#define MDWF_CASE(L) case L: cols_regs<L, EPI, T>(base, st, t.s, a.f, m); break;
+          MDWF_COLUMN_LENGTHS(MDWF_CASE)
+#undef MDWF_CASE
           default:
         for (int comp = t.s; comp < 24; comp += L5) {
           const bool upper = comp < 12;

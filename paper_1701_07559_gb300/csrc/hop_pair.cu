@@ -329,12 +329,9 @@ __device__ __forceinline__ void col_pairs(float* tile, const PThr& t, int L5, co
   for (int q = t.j; q < 6; q += J) {
     const int p = UPPER ? q : 6 + q;
     switch (L5) {
-      case 4: col_pair<EPI, 4, UPPER>(tile, t.site_l, t.r_l, p, c); break;
-      case 6: col_pair<EPI, 6, UPPER>(tile, t.site_l, t.r_l, p, c); break;
-      case 8: col_pair<EPI, 8, UPPER>(tile, t.site_l, t.r_l, p, c); break;
-      case 10: col_pair<EPI, 10, UPPER>(tile, t.site_l, t.r_l, p, c); break;
-      case 12: col_pair<EPI, 12, UPPER>(tile, t.site_l, t.r_l, p, c); break;
-      case 16: col_pair<EPI, 16, UPPER>(tile, t.site_l, t.r_l, p, c); break;
+#define MDWF_CASE(L) case L: col_pair<EPI, L, UPPER>(tile, t.site_l, t.r_l, p, c); break;
+      MDWF_COLUMN_LENGTHS(MDWF_CASE)
+#undef MDWF_CASE
       default: col_pair_any<EPI, UPPER>(tile, t.site_l, t.r_l, p, L5, c);
     }
   }
