@@ -66,7 +66,8 @@ typedef struct {
   double delta;    /* reliable update when |r| < delta * max |r| since the last one (default 0.1) */
   int chunk;       /* CG iterations per device launch sequence between host checks (default 16) */
   int use_graph;   /* capture each chunk in a CUDA graph (default 1) */
-  int nsb;         /* half-lattice sites per thread block (0 = chosen by the library) */
+  int nsb;         /* half-lattice sites per thread block of the inner hop (0 = chosen by the library; a
+                      block takes fewer where that many do not fit); the result does not depend on it */
   int profile;     /* 1: time every inner-precision hop launch with CUDA events (stats.hop_*) */
   double wait_timeout_s; /* bound of every device-side wait (default 2 s); a wait that runs out ends
                             the call with MDWF_ERR_TIMEOUT and leaves the context usable */
@@ -75,7 +76,8 @@ typedef struct {
   int hop_variant;       /* 0: automatic: the autotuner times the CUDA-core direct hop with 1..8
                             sites per block (and, for fp16 storage, form 7 with 1..4) once per (L5, N,
                             precision) and context and keeps the fastest; all of them give identical
-                            results.
+                            results.  FP64 storage has one form, whichever is asked for, and takes its
+                            sites per block by a rule instead of by timing.
                             1: CUDA-core hop with direct neighbour loads (FP32 arithmetic: two fifth-
                             dimension slices per thread in packed FP32); 2: CUDA-core hop with
                             neighbours staged in shared memory by bulk copies; 3: tensor-core colour
@@ -336,7 +338,8 @@ int mdwf_mres_correlators_dev(mdwf_ctx* ctx, int cfg_id, int n, double* const* x
  * solver uses for n right-hand sides of this configuration at `precision`
  * (include_tensor_core: also try the tensor-core hop), with its time for one
  * Mhat + Mhat^+ application.  Runs the timing once per (L5, n, precision,
- * candidate set) and context, then answers from the cache.  The timing runs use
+ * candidate set) and context, then answers from the cache (FP64: one candidate, the form and the sites per
+ * block that every FP64 hop of this shape takes).  The timing runs use
  * (and leave allocated) the context's solver workspace for n RHS, the fields a
  * solve of n RHS would use.  Outputs may be NULL.
  * Errors: ARG, STATE, NOMEM, CUDA, TIMEOUT. */

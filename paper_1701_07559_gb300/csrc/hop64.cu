@@ -388,38 +388,20 @@ __global__ void __launch_bounds__(256, 3) hop64_kernel(FastArgs<double, double> 
   }
 }
 
-// Sites and slots per block: about 32 units (one pass of eight warps), whole sites; large sites are split
-// into slot groups so that the tile stays within 100 KB (two blocks per SM).
-Shape64 shape64(int L5, int N, long Vh) {
-  Shape64 p;
-  const size_t unit = kRow64 * sizeof(double);
-  int groups = 1;
-  while (groups < N && (size_t)((N + groups - 1) / groups) * L5 * unit > 100 * 1024) groups++;
-  p.rt = (N + groups - 1) / groups;
-  p.nsb = 32 / (L5 * p.rt);
-  if (p.nsb < 1) p.nsb = 1;
-  // small lattices: fewer sites per block while that leaves schedulers idle (152 SMs x 4)
-  while (p.nsb > 1 && (Vh / p.nsb) * ((p.nsb * L5 * p.rt + 3) / 4) * groups < 608) p.nsb--;
-  return p;
-}
-
 template <int EPI, bool API>
-cudaError_t launch64_one(const FastArgs<double, double>& a, cudaStream_t st) {
-  const Shape64 p = shape64(a.L5, a.N, a.g.Vh);
-  const int units = p.nsb * a.L5 * p.rt;
-  const int warps = (units + 3) / 4;
+cudaError_t launch64_one(const FastArgs<double, double>& a, const Tiling& t, cudaStream_t st) {
+  const int warps = (t.threads + 3) / 4;                   // four units per warp
   // at least three warps: the epilogue's items (24 per unit) fill them where the units don't
   // (4^3 x 8, L5 = 4: 9.1 ms per FP64 solve with one warp per block, 8.7 with three)
   const int threads = 32 * (warps > 8 ? 8 : warps < 3 ? 3 : warps);
-  const size_t smem = (size_t)units * kRow64 * sizeof(double) + sizeof(int) * (p.rt + 1);
+  const size_t smem = (size_t)t.threads * kRow64 * sizeof(double) + sizeof(int) * (t.rt + 1);
   auto* kern = hop64_kernel<EPI, API>;
   if (smem > 48 * 1024) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
   }
-  const dim3 grid((unsigned)((a.g.Vh + p.nsb - 1) / p.nsb), (unsigned)((a.N + p.rt - 1) / p.rt),
-                  API && a.out_par < 0 ? 2u : 1u);
-  kern<<<grid, threads, smem, st>>>(a, p);
+  const dim3 grid((unsigned)t.ntiles, (unsigned)t.ngroups, API && a.out_par < 0 ? 2u : 1u);
+  kern<<<grid, threads, smem, st>>>(a, Shape64{t.nsb, t.rt});
   return cudaGetLastError();
 }
 
@@ -455,28 +437,52 @@ __global__ void __launch_bounds__(kLocal5) k_local5_api(const double* __restrict
 
 }  // namespace
 
-cudaError_t launch_hop64(const FastArgs<double, double>& a, int epi, cudaStream_t st) {
+// Sites and slots per block: about 32 units (one pass of eight warps, a tile of 6.4 KB), whole sites; large sites
+// are split into slot groups so that the tile stays within 100 KB, two blocks per SM.  nsb: that many sites
+// instead, as far as such a tile holds them; 0: the choice made here.
+Tiling hop64_tiling(long Vh, int L5, int N, int nsb) {
+  const size_t unit = kRow64 * sizeof(double), most = 100 * 1024;
+  Tiling t;
+  t.ngroups = 1;
+  while (t.ngroups < N && (size_t)((N + t.ngroups - 1) / t.ngroups) * L5 * unit > most) t.ngroups++;
+  t.rt = (N + t.ngroups - 1) / t.ngroups;
+  t.ngroups = (N + t.rt - 1) / t.rt;
+  t.nsb = nsb > 0 ? (nsb < 64 ? nsb : 64) : 32 / (L5 * t.rt);
+  if (nsb > 0) {
+    while (t.nsb > 1 && (size_t)t.nsb * L5 * t.rt * unit > most) t.nsb--;
+  } else {
+    // small lattices: fewer sites per block while that leaves schedulers idle (152 SMs x 4)
+    while (t.nsb > 1 && (Vh / t.nsb) * ((t.nsb * L5 * t.rt + 3) / 4) * t.ngroups < 608) t.nsb--;
+  }
+  if (t.nsb < 1) t.nsb = 1;
+  t.ntiles = (Vh + t.nsb - 1) / t.nsb;
+  t.threads = t.nsb * L5 * t.rt;                           // units of a block
+  return t;
+}
+
+cudaError_t launch_hop64(const FastArgs<double, double>& a, const Tiling& t, int epi, cudaStream_t st) {
   if (a.N < 1 || a.L5 < 1 || a.g.Vh < 1) return cudaErrorInvalidValue;
   switch (epi) {
-    case E_RAW: return launch64_one<E_RAW, false>(a, st);
-    case E_BAINV: return launch64_one<E_BAINV, false>(a, st);
-    case E_AINVD_BD: return launch64_one<E_AINVD_BD, false>(a, st);
-    case E_A_SAME: return launch64_one<E_A_SAME, false>(a, st);
-    case E_AD_SAME_BD: return launch64_one<E_AD_SAME_BD, false>(a, st);
-    case E_AINV_SAME: return launch64_one<E_AINV_SAME, false>(a, st);
-    case E_SAME_AINV: return launch64_one<E_SAME_AINV, false>(a, st);
-    case E_SAME_BD: return launch64_one<E_SAME_BD, false>(a, st);
-    case E_AINVD_SAME: return launch64_one<E_AINVD_SAME, false>(a, st);
+    case E_RAW: return launch64_one<E_RAW, false>(a, t, st);
+    case E_BAINV: return launch64_one<E_BAINV, false>(a, t, st);
+    case E_AINVD_BD: return launch64_one<E_AINVD_BD, false>(a, t, st);
+    case E_A_SAME: return launch64_one<E_A_SAME, false>(a, t, st);
+    case E_AD_SAME_BD: return launch64_one<E_AD_SAME_BD, false>(a, t, st);
+    case E_AINV_SAME: return launch64_one<E_AINV_SAME, false>(a, t, st);
+    case E_SAME_AINV: return launch64_one<E_SAME_AINV, false>(a, t, st);
+    case E_SAME_BD: return launch64_one<E_SAME_BD, false>(a, t, st);
+    case E_AINVD_SAME: return launch64_one<E_AINVD_SAME, false>(a, t, st);
     default: return cudaErrorInvalidValue;
   }
 }
 
 cudaError_t launch_hop64_api(const FastArgs<double, double>& a, int epi, cudaStream_t st) {
   if (a.N != 1 || a.L5 < 1 || a.g.Vh < 1) return cudaErrorInvalidValue;
+  const Tiling t = hop64_tiling(a.g.Vh, a.L5, 1, 0);
   switch (epi) {
-    case E_RAW: return launch64_one<E_RAW, true>(a, st);
-    case E_A_SAME: return launch64_one<E_A_SAME, true>(a, st);
-    case E_AD_SAME_BD: return launch64_one<E_AD_SAME_BD, true>(a, st);
+    case E_RAW: return launch64_one<E_RAW, true>(a, t, st);
+    case E_A_SAME: return launch64_one<E_A_SAME, true>(a, t, st);
+    case E_AD_SAME_BD: return launch64_one<E_AD_SAME_BD, true>(a, t, st);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -327,7 +327,7 @@ struct FastOp {
 
   cudaError_t dispatch(const FastArgs<S, T>& a, int epi) const {
     if constexpr (std::is_same<S, double>::value) {
-      return launch_hop64(a, epi, st);
+      return launch_hop64(a, tl, epi, st);
     } else {
       if constexpr (std::is_same<S, __half>::value) {
         if (mma) return launch_fast_mma(a, tl, epi, st, stage, mma_pipelined);
@@ -433,7 +433,7 @@ Tiling fast_tiling(const Geom& g, int L5, int N, int nsb_req, bool* staged, bool
   using T = typename StoreTraits<S>::T;
   *staged = false;
   if constexpr (std::is_same<S, double>::value) {
-    return make_tiling(g.Vh, L5, N, 1, 512);   // the FP64 hop has its own shape (hop64.cu)
+    return hop64_tiling(g.Vh, L5, N, nsb_req);
   } else {
   int maxthr = fast_max_threads<S, T>();
   if (maxthr > 1024) maxthr = 1024;
@@ -684,8 +684,10 @@ struct BatchSolver {
     auto it = ctx->tuned.find(key);
     if (it == ctx->tuned.end()) {
       std::vector<std::array<int, 2>> cand;
-      for (int nsbc : {1, 2, 4, 8})
-        if (nsbc * L5 <= 1024) cand.push_back({HOP_DIRECT, nsbc});
+      if (kFP64) cand.push_back({HOP_DIRECT, 0});      // the tiling is a rule's (hop64_tiling)
+      else
+        for (int nsbc : {1, 2, 4, 8})
+          if (nsbc * L5 <= 1024) cand.push_back({HOP_DIRECT, nsbc});
       // fp16 storage: the prefetching form of the paired hop, the same bits
       if (std::is_same<S, __half>::value)
         for (int nsbc : {1, 2, 4})
@@ -706,7 +708,7 @@ struct BatchSolver {
         choose_hop(opS, cfg, cnd[1], cnd[0], &stage);
         if (cnd[0] == HOP_MMA && !opS.mma) continue;
         if (cnd[0] == HOP_STAGED && opS.stage == nullptr) continue;
-        if ((cnd[0] == HOP_DIRECT || cnd[0] == HOP_PAIR_PF) && opS.tl.nsb != cnd[1]) continue;
+        if ((cnd[0] == HOP_DIRECT || cnd[0] == HOP_PAIR_PF) && cnd[1] > 0 && opS.tl.nsb != cnd[1]) continue;
         float ms = 0.f;
         cudaError_t e = cudaSuccess;
         for (int rep = 0; rep < 3 && e == cudaSuccess; rep++) {

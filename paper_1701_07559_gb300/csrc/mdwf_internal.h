@@ -367,8 +367,10 @@ template <typename S, typename T>
 cudaError_t launch_fast(const FastArgs<S, T>& a, const Tiling& t, int epi, cudaStream_t st,
                         const StageInfo* stage = nullptr);
 // FP64 hop (hop64.cu), on parity fields (a.active masks slots) or on the caller's arrays (one slot; out_par -1:
-// both parities; E_RAW, E_A_SAME, E_AD_SAME_BD); u = B x on the caller's layout, V sites.
-cudaError_t launch_hop64(const FastArgs<double, double>& a, int epi, cudaStream_t st);
+// both parities; E_RAW, E_A_SAME, E_AD_SAME_BD); u = B x on the caller's layout, V sites.  Its tiling: nsb sites per
+// block, or as many as the rule there takes (0); every tiling gives the same bits.
+Tiling hop64_tiling(long Vh, int L5, int N, int nsb);
+cudaError_t launch_hop64(const FastArgs<double, double>& a, const Tiling& t, int epi, cudaStream_t st);
 cudaError_t launch_hop64_api(const FastArgs<double, double>& a, int epi, cudaStream_t st);
 cudaError_t bop_api(const double* x, double* u, long V, int L5, double b5, double c5, double m, cudaStream_t st);
 // out_s = sum_s' G[chirality][s][s'] in_s' on the caller's layout (one right-hand side); L5 <= 32.
