@@ -341,7 +341,6 @@ template <int OP>
 __device__ __forceinline__ void cg_step(const Scal& c, const Slot& s, int r, double v, double w, double* out) {
   if (OP == FIN_STORE) out[r] = v;
   if (OP == FIN_ALPHA) {
-    c.qq[r] = v;
     if (s.active) c.alpha[r] = v > 0.0 ? s.gamma / v : 0.0;
     if (s.active) c.taken[r] = c.pos + 1;
     else if (c.pos == 0) c.taken[r] = 0;

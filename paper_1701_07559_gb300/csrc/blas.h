@@ -19,7 +19,7 @@ struct PGroup {
 
 // Per-slot scalars of the batched CG.
 struct Scal {
-  double *gamma, *gamma_prev, *alpha, *beta, *rho2, *rho2_max, *stop2, *qq, *rr, *tmp, *bhat2, *upd2;
+  double *gamma, *gamma_prev, *alpha, *beta, *rho2, *rho2_max, *stop2, *rr, *tmp, *bhat2, *upd2;
   int *active, *flags, *iters;
   int* since;     // CG iterations since the last reliable update of the slot
   int stag_max;   // that many without one: the inner recursion stagnates

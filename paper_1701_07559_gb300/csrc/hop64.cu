@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(256, 3) hop64_kernel(FastArgs<double, double> 
       const bool ef = cm == Lm - 1, eb = cm == 0;
       const long nf = ef ? lex - (long)(Lm - 1) * st : lex + st;
       const long nb = eb ? lex + (long)(Lm - 1) * st : lex - st;
-      const bool hf = mu == 3 && ef && a.halo_fwd != nullptr, hb = mu == 3 && eb && a.halo_fwd != nullptr;
+      const bool halo = API && mu == 3 && a.halo_fwd != nullptr, hf = halo && ef, hb = halo && eb;
       const bool flf = mu == 3 && ef && a.antiperiodic, flb = mu == 3 && eb && a.antiperiodic;
       // projected neighbours
       auto project = [&](long n, double sg, double* v) {

@@ -319,9 +319,6 @@ struct FastOp {
   const StageInfo* stage = nullptr;   // neighbour staging through shared memory, when the tiling allows
   const uint32_t* F16 = nullptr;      // fp16 link fragments for the tensor-core hop
   const float* U12 = nullptr;         // two-row links: the paired hop reconstructs the third row
-  const T* halo_fwd = nullptr;        // time-split domain decomposition: faces of the neighbours
-  const T* halo_bwd = nullptr;
-  T halo_sgn_fwd = T(1), halo_sgn_bwd = T(1);
   bool mma = false;                   // use the tensor-core hop (fp16 storage only)
   bool mma_pipelined = false;         // its bulk-copy pipelined form
 
@@ -343,7 +340,6 @@ struct FastOp {
     a.in = in.v; a.in_nrm = in.n; a.same = same.v; a.same_nrm = same.n; a.add = add.v; a.add_nrm = add.n;
     a.out = out.v; a.out_nrm = out.n; a.U = U; a.F16 = F16; a.U12 = U12; a.f = f; a.g_same = g_same;
     a.kappa = kappa;
-    a.halo_fwd = halo_fwd; a.halo_bwd = halo_bwd; a.halo_sgn_fwd = halo_sgn_fwd; a.halo_sgn_bwd = halo_sgn_bwd;
     a.active = active;
     a.partials = partials;
     if (launches) *launches += 1;
@@ -640,18 +636,17 @@ struct BatchSolver {
     }
     part = (double*)ws_get(c, wsp + "partials", sizeof(double) * g.Vh * N, &e); CK(e);
     part2 = (double*)ws_get(c, wsp + "partials2", sizeof(double) * g.Vh * N, &e); CK(e);
-    double* d = (double*)ws_get(c, wsp + "scal_d", sizeof(double) * (11 + kGroup) * N, &e); CK(e);
+    double* d = (double*)ws_get(c, wsp + "scal_d", sizeof(double) * (10 + kGroup) * N, &e); CK(e);
     int* ip = (int*)ws_get(c, wsp + "scal_i", sizeof(int) * 5 * N, &e); CK(e);
     umask_d = (int*)ws_get(c, wsp + "umask", sizeof(int) * N, &e); CK(e);
-    sc.gamma = d; sc.gamma_prev = d + N; sc.alpha = d + 11 * N; sc.beta = d + 3 * N; sc.rho2 = d + 4 * N;
-    sc.rho2_max = d + 5 * N; sc.stop2 = d + 6 * N; sc.qq = d + 7 * N; sc.rr = d + 8 * N; sc.tmp = d + 9 * N;
-    sc.bhat2 = d + 10 * N;
-    sc.upd2 = d + 2 * N;
+    sc.gamma = d; sc.gamma_prev = d + N; sc.upd2 = d + 2 * N; sc.beta = d + 3 * N; sc.rho2 = d + 4 * N;
+    sc.rho2_max = d + 5 * N; sc.stop2 = d + 6 * N; sc.rr = d + 7 * N; sc.tmp = d + 8 * N; sc.bhat2 = d + 9 * N;
+    sc.alpha = d + 10 * N;
     sc.active = ip; sc.flags = ip + N; sc.iters = ip + 2 * N; sc.since = ip + 3 * N;
     sc.taken = ip + 4 * N;
     sc.pos = 0;
     sc.stag_max = 128;
-    CK(cudaMemsetAsync(d, 0, sizeof(double) * (11 + kGroup) * N, st));
+    CK(cudaMemsetAsync(d, 0, sizeof(double) * (10 + kGroup) * N, st));
     CK(cudaMemsetAsync(ip, 0, sizeof(int) * 5 * N, st));
     const size_t b64 = sizeof(double) * 24 * (size_t)units;
     CK(cudaMemsetAsync(x_acc.v, 0, b64, st));
@@ -1323,8 +1318,8 @@ struct SessionImpl : SessionBase {
     const double zd = 0.0;
     int* ia[] = {sv.sc.active, sv.sc.flags, sv.sc.iters, sv.sc.since};
     for (int* a : ia) CK(cudaMemcpyAsync(a + r, &zi, sizeof(int), cudaMemcpyHostToDevice, st));
-    double* da[] = {sv.sc.gamma, sv.sc.gamma_prev, sv.sc.alpha, sv.sc.beta, sv.sc.rho2, sv.sc.rho2_max, sv.sc.qq,
-                    sv.sc.rr, sv.sc.tmp, sv.sc.bhat2, sv.sc.upd2};
+    double* da[] = {sv.sc.gamma, sv.sc.gamma_prev, sv.sc.alpha, sv.sc.beta, sv.sc.rho2, sv.sc.rho2_max, sv.sc.rr,
+                    sv.sc.tmp, sv.sc.bhat2, sv.sc.upd2};
     for (double* a : da)
       CK(cudaMemcpyAsync(a + r, &zd, sizeof(double), cudaMemcpyHostToDevice, st));
     const int* m = sv.umask_d;
