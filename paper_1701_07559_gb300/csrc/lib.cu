@@ -590,7 +590,7 @@ struct BatchSolver {
     choose_hop(op64, cf, 0, HOP_DIRECT, &stage);
     choose_hop(op32, cf, nsb, (variant == HOP_AUTO || variant == HOP_TUNE_ALL) ? HOP_DIRECT : variant, &stage);
     choose_hop(opS, cf, nsb, (variant == HOP_AUTO || variant == HOP_TUNE_ALL) ? HOP_DIRECT : variant, &stage);
-    tune_request = (variant == HOP_AUTO || variant == HOP_TUNE_ALL) && nsb == 0 ? variant : -1;
+    tune_request = (variant == HOP_AUTO || variant == HOP_TUNE_ALL) && nsb == 0 && !kFP64 ? variant : -1;
     // 12-real links (the third row reconstructed) for the inner hops; the FP32
     // reliable updates keep the full links
     opS.U12 = (!kFP64 && o.link_recon == 12) ? cf->U12 : nullptr;
