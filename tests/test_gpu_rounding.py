@@ -13,6 +13,7 @@ import numpy as np
 import pytest
 
 import synth
+from oracle import flow as F
 from oracle import mdwf_oracle as O
 
 pytestmark = pytest.mark.gpu
@@ -138,3 +139,16 @@ def test_flow_rounds_the_links_once_per_stage():
     assert float(diag.min()) > 0.5
     err = (got[..., i, i].real - diag).astype(np.float64)
     assert np.sqrt(np.mean(err ** 2)) <= np.sqrt(2 * 3 * steps) * 2.0 ** -54 / np.sqrt(3)
+
+
+def test_flow_of_large_steps():
+    """|X| above 1/2: exp(X) - 1 by squarings of a scaled one."""
+    dims, eps = (4, 2, 2, 4), 0.5
+    U = synth.random_gauge(dims, 6, 0.7)
+    assert 3.0 * eps / 4 * np.sqrt(np.sum(np.abs(F.flow_generator(U)) ** 2, axis=(-2, -1))).max() > 1.0
+    ctx = M.mdwf_create(dims, 0)
+    d = torch.from_numpy(U).cuda()
+    M.mdwf_wilson_flow_dev(ctx, d, eps, 1)
+    got = d.cpu().numpy()
+    M.mdwf_destroy(ctx)
+    assert np.abs(got - F.wilson_flow(U, eps, 1)).max() <= 1e-12
