@@ -27,8 +27,8 @@
 //   multiply-adds of exp(X) U left 5.35e-16 and the matrix products before it 4.65e-16; it costs 1 % of a step.
 // Z keeps the nine independent reals of an anti-Hermitian matrix, one plane each.
 // Ten steps at 16^3 x 48: 297 ms with a thread per link and the matrix Taylor series
-// (which spilled), 71 ms so (2.4 ms per stage; its 1800 multiply-adds per link take 2.3 ms
-// at 6.2e11 per second, the FP64 rate of the part).
+// (which spilled), 72 ms so (2.4 ms per stage; its 1800 FP64 instructions per link take 2.25 ms
+// at 6.3e11 per second, two lanes per SM and clock at 2070 MHz).
 //
 // Layout of U: the C ABI's gauge layout U[t][z][y][x][mu][a][b], complex (re, im).
 // Input preparation: the solver reads links only through mdwf_load_gauge.

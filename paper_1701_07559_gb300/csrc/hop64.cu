@@ -3,8 +3,8 @@
 // fields or directly on the caller's arrays (C ABI layout).
 //
 // What bounds it: an FP64 instruction of a warp occupies its scheduler's FP64
-// unit for 64 clocks however many of its lanes are active (1.0 TFLOP/s for the
-// whole chip, measured), 40 times the cost of anything else the kernel does.  So
+// unit for 64 clocks however many of its lanes are active (two lanes per SM and clock: 6.3e11
+// instructions per second on 152 SMs at 2070 MHz), 40 times the cost of anything else the kernel does.  So
 // the kernel is built for full warps and few FP64 instructions, and spends loads,
 // shuffles and integer work freely:
 // * eight lanes per unit (site, s, r): lane (mu, j) does both hops of direction mu
@@ -14,8 +14,8 @@
 //   times wider.
 // * x_b = U^+ h_b and x_f = U h_f, each rounded by itself, then S = x_b + x_f and D = x_b - x_f: the
 //   upper spins sum S over the directions, the lower ones D with the gamma matrices' factors: 105
-//   instructions per lane, 840 per unit, where the accumulation of every product into all four spins took
-//   864.  Chaining U h_f onto x_b and taking D = 2 x_b - S saves 6 of the 105, but rounds at the size of
+//   instructions per lane, 840 per unit (896 by ncu, with the signs of the projections), where the
+//   accumulation of every product into all four spins took 864.  Chaining U h_f onto x_b and taking D = 2 x_b - S saves 6 of the 105, but rounds at the size of
 //   the sum: 1.05 times the error of that accumulation in H (1.57e-16 against 1.49e-16, rms of the result,
 //   extended precision as the reference), this order 0.93 times (1.38e-16).
 // * the sums over the directions are a reduce-scatter by shuffles; factors 1, -1, i, -i
@@ -25,12 +25,13 @@
 // * the epilogues run over (unit, component) or (column, component) items of a
 //   shared-memory tile, with the coefficients folded (3 to 4 instructions per
 //   component).
-// * three blocks of eight warps per SM (80 registers): 24 warps hide the loads and shuffles
-//   better than the 16 of an unbounded kernel (104 registers), 4.68 against 4.50 ms for D below;
-//   32 (64 registers) measured the same as 24.
-// D of one field at 16^3 x 48, L5 = 12: 6.61 -> 4.50 ms (1000 instructions per unit and
-// packing to parity fields before; 870 now, 3.3 ms of FP64); H^+ at 6 x 4 x 2 x 10, L5 = 5:
-// 138 -> 25 us; an FP64 solve at 4^3 x 8, L5 = 4: 28.0 -> 8.7 ms.
+// * three blocks of eight warps per SM (80 registers, with up to 20 bytes of spills per thread, 60 to 68 in three
+//   of the column epilogues): 24 warps hide the loads and shuffles better than the 16 of an unbounded kernel (104
+//   registers; D below, measured with the chained products: 4.50 ms with 24 warps, 4.68 with 16); 32 (64
+//   registers) measured the same as 24.
+// D of one field at 16^3 x 48, L5 = 12: 6.61 ms with a thread per unit and packing to parity fields, 4.73 so,
+// of which 3.9 ms are FP64 (962 instructions per unit here, 72 in B in); H^+ at 6 x 4 x 2 x 10, L5 = 5:
+// 138 -> 26 us; an FP64 solve at 4^3 x 8, L5 = 4: 28.2 -> 8.7 ms.
 // A unit's result depends on nothing but its inputs: every block shape, slot count
 // and mask, the decomposed lattice (halo terms) and both layouts give the same bits.
 #include "mdwf_internal.h"
